@@ -7,6 +7,7 @@
 #include <math.h>
 
 #include "../../include/smerf.h"
+#include "smerf_fixed.cuh"
 
 #ifndef SMERF_PI
 #define SMERF_PI 3.14159265358979323846
@@ -214,15 +215,10 @@ __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, float& n0, fl
     n1 = r * s;
 }
 
+// FP64: 64-bit fixed point on the integer lanes (smerf_fixed.cuh)
 __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, double& n0, double& n1)
 {
-    const double u0 = ((double)a + 0.5) * 0x1p-32;
-    const double u1 = ((double)b + 0.5) * 0x1p-32;
-    const double r = sqrt(-2.0 * log(u0));
-    double s, c;
-    sincospi(2.0 * u1, &s, &c);
-    n0 = r * c;
-    n1 = r * s;
+    fx_box_muller(a, b, kFxLog[fx_log_index(a)], n0, n1);
 }
 
 // ------------------------------------------------------------------ complex helpers
