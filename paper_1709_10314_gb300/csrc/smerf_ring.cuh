@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(RingPass<LG>::NT, MINB) ring_kernel(SamplePara
     static_assert(!PACKED || sizeof(TabT) == 4, "packed tables are FP32");
     static_assert(Nc / 2 == U * NT, "8 units of two slots per thread");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint2 rk[10];  // Philox round keys of the CTA's realisation
+    __shared__ uint4 rk[kKeyWords];  // Philox round keys of the CTA's realisation
 
     const Segment sg = P.segs[blockIdx.y];
     const int r0 = blockIdx.x;
@@ -202,10 +202,7 @@ __global__ void __launch_bounds__(RingPass<LG>::NT, MINB) ring_kernel(SamplePara
 
     float2* X = reinterpret_cast<float2*>(smem_raw);                 // the ring, Nc complex
     float4* park = reinterpret_cast<float4*>(smem_raw + (size_t)Nc * sizeof(float2));  // [PARK][NT]
-    if (tid < 10) {
-        const uint64_t key = P.seed + (uint64_t)r0;
-        rk[tid] = make_uint2((uint32_t)key + (uint32_t)tid * 0x9E3779B9u, (uint32_t)(key >> 32) + (uint32_t)tid * 0xBB67AE85u);
-    }
+    if (tid < kKeyWords) rk[tid] = round_key_word(P.seed + (uint64_t)r0, tid);
     const float* xrg = anc + aoff<1>(P, c, r0, has_right ? sg.right : 0, 0, 0);
 
     float4 xreg[UP > 0 ? UP : 1];

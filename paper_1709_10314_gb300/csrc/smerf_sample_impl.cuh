@@ -714,16 +714,32 @@ __device__ __forceinline__ void step_state(const Real* t, Real (&x)[M], const Re
     for (int q = 0; q < M; ++q) x[q] = xn[q];
 }
 
-// Philox4x32-10 with precomputed round keys rk[i] = (k0 + i W0, k1 + i W1), i < 10
-__device__ __forceinline__ uint4 philox_rk(uint4 c, const uint2* rk)
+// Round keys of a realisation in shared memory: word i holds those of rounds 2i and 2i + 1,
+// (k0 + 2i W0, k1 + 2i W1, k0 + (2i + 1) W0, k1 + (2i + 1) W1), so that two rounds take one
+// 16-byte broadcast load.
+constexpr int kKeyWords = 5;
+__device__ __forceinline__ uint4 round_key_word(uint64_t key, int i)
 {
-    const uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
+    const uint32_t W0 = 0x9E3779B9u, W1 = 0xBB67AE85u;
+    const uint32_t k0 = (uint32_t)key + 2u * i * W0, k1 = (uint32_t)(key >> 32) + 2u * i * W1;
+    return make_uint4(k0, k1, k0 + W0, k1 + W1);
+}
+
+__device__ __forceinline__ uint4 philox_round(uint4 c, uint32_t k0, uint32_t k1)
+{
+    const uint64_t p0 = (uint64_t)0xD2511F53u * c.x;
+    const uint64_t p1 = (uint64_t)0xCD9E8D57u * c.z;
+    return make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k0, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k1, (uint32_t)p0);
+}
+
+// Philox4x32-10 with precomputed round keys
+__device__ __forceinline__ uint4 philox_rk(uint4 c, const uint4* rk)
+{
 #pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint2 k = rk[r];
-        const uint64_t p0 = (uint64_t)M0 * c.x;
-        const uint64_t p1 = (uint64_t)M1 * c.z;
-        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k.x, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k.y, (uint32_t)p0);
+    for (int i = 0; i < kKeyWords; ++i) {
+        const uint4 k = rk[i];
+        c = philox_round(c, k.x, k.y);
+        c = philox_round(c, k.z, k.w);
     }
     return c;
 }
@@ -732,23 +748,19 @@ __device__ __forceinline__ uint4 philox_rk(uint4 c, const uint2* rk)
 // generator chains are independent and run interleaved; the first round's products, which
 // depend on the counter only, are shared.
 template <class Real, int NB, int NC = 1>
-__device__ __forceinline__ void unit_normals_multi(const uint2 (*rk)[10], uint32_t u, uint32_t ring, Real (&n)[NB][4 * NC])
+__device__ __forceinline__ void unit_normals_multi(const uint4 (*rk)[kKeyWords], uint32_t u, uint32_t ring, Real (&n)[NB][4 * NC])
 {
-    const uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
 #pragma unroll
     for (int j = 0; j < NC; ++j) {  // the unit's Philox calls NC u + j
         uint4 c[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) c[b] = make_uint4(u * NC + j, ring, 0u, 0u);
 #pragma unroll
-        for (int r = 0; r < 10; ++r) {
+        for (int i = 0; i < kKeyWords; ++i) {
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
-                const uint2 k = rk[b][r];
-                const uint64_t p0 = (uint64_t)M0 * c[b].x;
-                const uint64_t p1 = (uint64_t)M1 * c[b].z;
-                c[b] = make_uint4((uint32_t)(p1 >> 32) ^ c[b].y ^ k.x, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c[b].w ^ k.y,
-                                  (uint32_t)p0);
+                const uint4 k = rk[b][i];
+                c[b] = philox_round(philox_round(c[b], k.x, k.y), k.z, k.w);
             }
         }
 #pragma unroll
@@ -760,7 +772,7 @@ __device__ __forceinline__ void unit_normals_multi(const uint2 (*rk)[10], uint32
 }
 
 template <class Real, int NC = 1>
-__device__ __forceinline__ void unit_normals_rk(const uint2* rk, uint32_t u, uint32_t ring, Real (&n)[4 * NC])
+__device__ __forceinline__ void unit_normals_rk(const uint4* rk, uint32_t u, uint32_t ring, Real (&n)[4 * NC])
 {
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
@@ -787,7 +799,7 @@ __global__ void __launch_bounds__(1024, 1) segment_kernel(SampleParams P)
     constexpr int UP = UPT - PARK;        // units whose state stays in registers during the FFT
     constexpr int NU = unit_vals(M), NC = unit_calls(M);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint2 rk[10];              // Philox round keys of the CTA's realisation
+    __shared__ uint4 rk[kKeyWords];       // Philox round keys of the CTA's realisation
 
     const Segment sg = P.segs[blockIdx.y];
     const int r0 = blockIdx.x;
@@ -804,10 +816,7 @@ __global__ void __launch_bounds__(1024, 1) segment_kernel(SampleParams P)
     Real* park = reinterpret_cast<Real*>(buf0 + Nc);
     const C* twp = (const C*)P.tw;
     const C* pre = (const C*)P.pre;
-    if (tid < 10) {
-        const uint64_t key = P.seed + (uint64_t)r0;
-        rk[tid] = make_uint2((uint32_t)key + (uint32_t)tid * 0x9E3779B9u, (uint32_t)(key >> 32) + (uint32_t)tid * 0xBB67AE85u);
-    }
+    if (tid < kKeyWords) rk[tid] = round_key_word(P.seed + (uint64_t)r0, tid);
     // right-anchor states are read from the scratch ([slot][2M])
     const Real* xrg = anc + aoff<M>(P, c, r0, has_right ? sg.right : 0, 0, 0);
 
@@ -1312,7 +1321,7 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
     constexpr int RB = RMAX < SMERF_RB ? RMAX : SMERF_RB;  // realisations whose noise is drawn together
     constexpr int NU = unit_vals(M), NC = unit_calls(M);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint2 rk[RMAX][10];
+    __shared__ uint4 rk[RMAX][kKeyWords];
 
     const Segment sg = P.segs[seg_index];
     const int r0 = group * RMAX;
@@ -1332,10 +1341,9 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
     Real* xRs = reinterpret_cast<Real*>(bufs + (size_t)3 * RMAX * Nc);
     const C* twp = (const C*)P.tw;
     const C* pre = (const C*)P.pre;
-    if (tid < RMAX * 10) {
-        const int r = tid / 10, i = tid % 10;
-        const uint64_t key = P.seed + (uint64_t)(r0 + r);
-        rk[r][i] = make_uint2((uint32_t)key + (uint32_t)i * 0x9E3779B9u, (uint32_t)(key >> 32) + (uint32_t)i * 0xBB67AE85u);
+    if (tid < RMAX * kKeyWords) {
+        const int r = tid / kKeyWords, i = tid % kKeyWords;
+        rk[r][i] = round_key_word(P.seed + (uint64_t)(r0 + r), i);
     }
     if (has_right) {
         const int per = 2 * M * Nc;
