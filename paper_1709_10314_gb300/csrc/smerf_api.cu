@@ -42,7 +42,7 @@ void free_plan_memory(smerf_plan* pl)
     cudaFree(pl->segs_dev);
     free(pl->segs_host);
     cudaFree(pl->rings_n_dev);
-    cudaFree(pl->rings_h_dev);
+    cudaFree(pl->rings_ph_dev);
     cudaFree(pl->rings_off_dev);
     free(pl->theta_host);
     cudaFree(pl->theta_dev);
@@ -51,10 +51,10 @@ void free_plan_memory(smerf_plan* pl)
 void free_rings(smerf_plan* pl)
 {
     cudaFree(pl->rings_n_dev);
-    cudaFree(pl->rings_h_dev);
+    cudaFree(pl->rings_ph_dev);
     cudaFree(pl->rings_off_dev);
     pl->rings_n_dev = nullptr;
-    pl->rings_h_dev = nullptr;
+    pl->rings_ph_dev = nullptr;
     pl->rings_off_dev = nullptr;
     pl->rings_total = 0;
 }
@@ -623,8 +623,9 @@ int smerf_sample_launches(const smerf_plan* plan, int n_samples)
 {
     if (!plan || n_samples < 0) return SMERF_EINVAL;
     if (n_samples == 0) return 0;
-    // anchor and segment launches, and ahead of them the short conversion of the coarse and
-    // start tables when the call stages FP64 tables (the anchor launch converts the step tables)
+    // anchor and segment launches, and ahead of them the conversion of the coarse and start tables
+    // (the anchor launch converts the step tables; of all tables where few anchor threads run)
+    // when the call stages FP64 tables
     return use_stage(plan, n_samples) ? 3 : 2;
 }
 
@@ -690,7 +691,7 @@ int smerf_plan_set_rings(smerf_plan* plan, const int* n_phi_ring, const double* 
         return SMERF_OK;
     }
     std::vector<int> n(plan->n_theta);
-    std::vector<double> h(plan->n_theta);
+    std::vector<unsigned long long> ph(plan->n_theta);
     std::vector<long long> off(plan->n_theta);
     long long total = 0;
     for (int k = 0; k < plan->n_theta; ++k) {
@@ -698,7 +699,11 @@ int smerf_plan_set_rings(smerf_plan* plan, const int* n_phi_ring, const double* 
         const double p0 = phi0_ring ? phi0_ring[k] : 0.0;
         if ((nk & 1) || nk < 4 || nk > plan->n_phi || !isfinite(p0)) return SMERF_EINVAL;
         n[k] = nk;
-        h[k] = fmod(p0 / SMERF_PI, 2.0);
+        // the offset as a signed 64-bit fraction of a turn (2^-65 turns off at most)
+        double turns = 0.5 * fmod(p0 / SMERF_PI, 2.0);
+        turns -= rint(turns);
+        if (turns >= 0.5) turns -= 1.0;
+        ph[k] = (unsigned long long)llrint(ldexp(turns, 64));
         off[k] = total;
         total += nk;
     }
@@ -710,12 +715,12 @@ int smerf_plan_set_rings(smerf_plan* plan, const int* n_phi_ring, const double* 
     free_rings(plan);
     int rc = SMERF_OK;
     if (smerf::dev_malloc((void**)&plan->rings_n_dev, sizeof(int) * n.size()) != cudaSuccess ||
-        smerf::dev_malloc((void**)&plan->rings_h_dev, sizeof(double) * h.size()) != cudaSuccess ||
+        smerf::dev_malloc((void**)&plan->rings_ph_dev, sizeof(unsigned long long) * ph.size()) != cudaSuccess ||
         smerf::dev_malloc((void**)&plan->rings_off_dev, sizeof(long long) * off.size()) != cudaSuccess)
         rc = SMERF_ENOMEM;
     if (rc == SMERF_OK &&
         (cudaMemcpy(plan->rings_n_dev, n.data(), sizeof(int) * n.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-         cudaMemcpy(plan->rings_h_dev, h.data(), sizeof(double) * h.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+         cudaMemcpy(plan->rings_ph_dev, ph.data(), sizeof(unsigned long long) * ph.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
          cudaMemcpy(plan->rings_off_dev, off.data(), sizeof(long long) * off.size(), cudaMemcpyHostToDevice) != cudaSuccess))
         rc = SMERF_ECUDA;
     if (rc != SMERF_OK) {
@@ -923,7 +928,7 @@ int smerf_plan_autotune_anchor(smerf_plan* plan, int n_samples, const int* candi
         // tables go with `best`
         std::swap(*plan, *best);
         std::swap(plan->rings_n_dev, best->rings_n_dev);
-        std::swap(plan->rings_h_dev, best->rings_h_dev);
+        std::swap(plan->rings_ph_dev, best->rings_ph_dev);
         std::swap(plan->rings_off_dev, best->rings_off_dev);
         std::swap(plan->rings_total, best->rings_total);
         if (chosen) *chosen = plan->H;

@@ -1,0 +1,362 @@
+// smerf_band.cuh -- the segment kernel for requests that leave most of the GPU idle (few
+// segments, few realisations) and for plans with ring-dependent longitudes.  Included by
+// smerf_sample_impl.cuh.
+//
+// The warp-specialised kernel walks a segment ring by ring, so a request of a few segments takes
+// the latency of a whole ring (noise, step, FFT: 2 us and more) for each ring of a segment while
+// most SMs idle.  Here a CTA takes one realisation's segment in chunks of rings and does each
+// part of the work for the whole chunk at once, with every thread:
+//   1. the noise of every (ring, unit) of the chunk, which depends on no state;
+//   2. the recursion, one thread per unit, nothing but its table rows and a few multiply-adds per
+//      ring (Eq. (state_space), with step_state's operations in step_state's order, so that the
+//      field is the warp-specialised kernel's bit for bit);
+//   3. the C2R FFTs of the chunk's rings side by side, written straight to the output.
+// A segment can be split further over `splits` CTAs: each repeats parts 1 and 2 from the
+// segment's start (they are cheap) and synthesises only its own share of the rings.
+//
+// Rings with their own point count n: Y_q = sum over m = q (mod n) of c_m e^{i m phi0} is formed
+// and packed for an n/2-point complex FFT, which runs in Stockham passes over the factors of n/2
+// (4, 2, then the odd primes), one output point per thread from r terms with the roots of unity
+// from a table of the ring's own, a group of threads per ring.  HEALPix's polar rings (4i points)
+// took O(n^2) terms in the FFT warps of one CTA per segment before: Nside 128, 16 realisations,
+// 4266 -> 137 us a call.  One FP64 realisation of 64 x 128 in Alg. 2's order: 166 -> 33 us; one of
+// 181 x 512, p = 2: 31.1 -> 23.6 us (the anchor tiles among them).
+#pragma once
+
+namespace smerf {
+
+constexpr int kBandThreads = 256;
+
+// e^{2 pi i p}, p = ph 2^-64 turns
+template <class Real> __device__ __forceinline__ cplx<Real> cis_turns(uint64_t ph)
+{
+    Real sn, cs;
+    if constexpr (sizeof(Real) == 4) sincospif((float)(int32_t)(ph >> 32) * 0x1p-31f, &sn, &cs);
+    else fx_cis(ph, cs, sn);
+    return cmk<cplx<Real>>(cs, sn);
+}
+
+// threads that share a ring of its own point count, and such groups per CTA: a warp for rings up
+// to 512 points, the whole CTA from 4096 on
+__host__ __device__ inline int band_group(int Nc) { return Nc <= 256 ? 32 : Nc >= 2048 ? 256 : Nc / 8; }
+
+__device__ __forceinline__ void band_group_sync(int gs, int g)
+{
+    if (gs == 32) __syncwarp();
+    else bar_sync(6 + g, gs);
+}
+
+// Y_q of the ring's coefficients X (slot 0 = (g_0, Re g_M), slot m = g_m, M = Nc): the real field
+// T(phi) = sum_{|m| <= M} c_m e^{i m phi}, c_0 = g_0, c_{+-m} = g_m, conj g_m, c_{+-M} = Re g_M / 2, has
+// Y_q = sum over m = q (mod n) of c_m e^{i m phi0} (modes above the ring's own Nyquist alias onto it)
+template <class Real>
+__device__ __forceinline__ cplx<Real> band_fold(const cplx<Real>* X, int Nc, int n, uint64_t ph, int q)
+{
+    using C = cplx<Real>;
+    C acc = cmk<C>(0, 0);
+    auto term = [&](int m) {
+        const C g = m == 0 ? cmk<C>(X[0].x, 0) : (m == Nc ? cmk<C>((Real)0.5 * X[0].y, 0) : X[m]);
+        return ph == 0 ? g : cmul(g, cis_turns<Real>((uint64_t)m * ph));
+    };
+    for (int m = q; m <= Nc; m += n) acc = cadd(acc, term(m));
+    for (int m = q == 0 ? n : n - q; m <= Nc; m += n) acc = cadd(acc, cconj(term(m)));  // -m < 0
+    return acc;
+}
+
+// One ring of n = 2 N points from its coefficients in X (destroyed) with W as second buffer and
+// RT for the N roots e^{2 pi i t / n}, by the gs threads of a group (lane l of group g)
+template <class Real>
+__device__ __noinline__ void band_ragged_ring(cplx<Real>* X, cplx<Real>* W, cplx<Real>* RT, int Nc, int n, uint64_t ph,
+                                              cplx<Real>* gout, int l, int gs, int g)
+{
+    using C = cplx<Real>;
+    const int N = n / 2;
+    {
+        // t / n as a 64-bit fraction: t (2^64 / n) with the division's remainder r < n <= 2^13 (t r < 2^26)
+        const uint64_t q = ~0ull / (unsigned)n;
+        const unsigned r = (unsigned)(~0ull - q * (unsigned)n) + 1u;
+        for (int t = l; t < N; t += gs) RT[t] = cis_turns<Real>((uint64_t)t * q + ((unsigned)t * r) / (unsigned)n);
+    }
+    band_group_sync(gs, g);
+    // fold and C2R packing (c2r_pack's Z), the pair q, N - q together
+    for (int q = l; 2 * q <= N; q += gs) {
+        const C a = band_fold<Real>(X, Nc, n, ph, q), b = cconj(band_fold<Real>(X, Nc, n, ph, N - q));
+        if (q == 0) {
+            W[0] = cmk<C>(a.x + b.x, a.x - b.x);
+        } else {
+            const C e = cadd(a, b), o = cmuli(cmul(RT[q], csub(a, b)));
+            W[q] = cadd(e, o);
+            if (2 * q < N) W[N - q] = cconj(csub(e, o));
+        }
+    }
+    band_group_sync(gs, g);
+    C* src = W;
+    C* dst = X;
+    int Ns = 1, rem = N, p = 3;
+    while (rem > 1) {
+        int r;
+        if ((rem & 3) == 0) r = 4;
+        else if ((rem & 1) == 0) r = 2;
+        else {
+            while (p * p <= rem && rem % p) p += 2;
+            r = rem % p ? rem : p;
+        }
+        rem /= r;
+        const int Wn = Ns * r, m = N / r, unit = N / Wn;
+        for (int e = l; e < N; e += gs) {
+            const int blk = e / Wn, w = e - blk * Wn, st = w * unit;  // w = kk + a Ns
+            const C* in = src + blk * Ns + w % Ns;
+            C acc = in[0];
+            int t = st;
+            for (int i = 1; i < r; ++i) {
+                const int u = 2 * t;  // root of order N: e^{2 pi i t / N} = e^{2 pi i u / n}, half a turn from t = N / 2 on
+                const C x = in[i * m], y = u < N ? RT[u] : RT[u - N];
+                const C z = cmul(x, y);
+                acc = u < N ? cadd(acc, z) : csub(acc, z);
+                t += st;
+                if (t >= N) t -= N;
+            }
+            if (rem == 1) __stcs(gout + e, acc);
+            else dst[e] = acc;
+        }
+        Ns = Wn;
+        band_group_sync(gs, g);
+        C* s = src;
+        src = dst;
+        dst = s;
+    }
+    if (N == 1 && l == 0) __stcs(gout, W[0]);
+}
+
+// Table rows of unit u at one position, G rows of step_row(M) values, converted to Real; ny: the
+// Nyquist chain's row (unit 0 only)
+template <class Real, class TabT, int M>
+__device__ __forceinline__ void band_rows(const TabT* tb, int u, Real (&t)[kG<M>][step_row(M)])
+{
+    constexpr int G = kG<M>, ROW = step_row(M);
+#pragma unroll
+    for (int g = 0; g < G; ++g) load_row<Real, TabT, ROW>(tb + (size_t)(G * u + g) * ROW, t[g]);
+}
+
+// One ring's step of a unit (table rows t, the Nyquist chain's row ny, normals nr, the right
+// anchor's states xr), as in ws_body
+template <class Real, int M>
+__device__ __forceinline__ void band_step(const Real (&t)[kG<M>][step_row(M)], const Real* ny, bool first_unit,
+                                          bool has_right, const Real* nr, const Real* xr, Real (&x)[unit_vals(M)])
+{
+    constexpr int G = kG<M>, ROW = step_row(M);
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+            Real(&xs)[M] = *reinterpret_cast<Real(*)[M]>(&x[g * 2 * M + part * M]);
+            const Real* xi = nr + g * 2 * M + part * M;
+            const Real* xq = xr + g * 2 * M + part * M;
+            if (g == 0 && part == 1 && first_unit) {
+                Real tn[ROW];  // slot 0, second part: the Nyquist chain
+                VecN<Real, ROW>::ld(ny, tn);
+                if (has_right) step_state<Real, M, true>(tn, xs, xi, xq);
+                else step_state<Real, M, false>(tn, xs, xi, nullptr);
+            } else if (has_right) {
+                step_state<Real, M, true>(t[g], xs, xi, xq);
+            } else {
+                step_state<Real, M, false>(t[g], xs, xi, nullptr);
+            }
+        }
+}
+
+// What a (ring, unit) of a chunk keeps in shared memory between parts 1 and 2: its normals and,
+// staged, its table rows; an odd number of 16-byte words, so that neighbouring units' vector
+// accesses fall on different banks
+template <class Real, int M, bool STAGE>
+__host__ __device__ constexpr int band_unit_reals()
+{
+    const int v = unit_vals(M) + (STAGE ? unit_slots(M) * step_row(M) : 0), w = 16 / (int)sizeof(Real);
+    return STAGE && (v / w) % 2 == 0 ? v + w : v;
+}
+
+// Shared memory (cplx = 2 Real): X [chunk][Nc] cplx; the units' words [chunk][units][UV] Real, the
+// same memory then the FFTs' second buffer [chunk][Nc] cplx; the states [units][NU] Real; the
+// Nyquist chain's rows [chunk][ROW] Real; the root tables [groups][Nc] cplx (ring-dependent
+// longitudes only)
+template <class Real, int M, bool STAGE>
+__host__ __device__ inline size_t band_smem(int Nc, int chunk, bool rings)
+{
+    const int units = Nc / unit_slots(M);
+    const size_t x = (size_t)Nc * 2 * sizeof(Real), uv = (size_t)units * band_unit_reals<Real, M, STAGE>() * sizeof(Real);
+    return chunk * (x + uv + step_row(M) * sizeof(Real)) + (size_t)units * unit_vals(M) * sizeof(Real) +
+           (rings ? (kBandThreads / band_group(Nc)) * x : 0);
+}
+
+// grid (splits, realisations, segments)
+// STAGE: the chunk's table rows go through shared memory, loaded in part 1 beside the noise by
+// every thread, so that the recursion waits for no global load
+template <class Real, class TabT, int M, bool STAGE>
+__global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SampleParams P, int chunk)
+{
+    using C = cplx<Real>;
+    constexpr int G = kG<M>, ROW = step_row(M), NU = unit_vals(M), NC = unit_calls(M);
+    constexpr int UV = band_unit_reals<Real, M, STAGE>();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint4 rk[kKeyWords];
+
+    const Segment sg = P.segs[blockIdx.z];
+    const int r = blockIdx.y, c = sg.chain;
+    const int tid = threadIdx.x, nt = kBandThreads;
+    const int Nc = P.Nc, n_units = P.n_units;
+    const size_t mp = P.n_modes_pad;
+    const bool has_right = sg.right >= 0;
+    // this CTA's share of the segment's rings (the start ring is written by the northern chain)
+    const int first = (c == 1 && sg.p0 == 0) ? 1 : sg.p0, len = sg.p1 - first;
+    const int own0 = first + (int)((long long)len * blockIdx.x / gridDim.x);
+    const int own1 = first + (int)((long long)len * (blockIdx.x + 1) / gridDim.x);
+    if (own0 >= own1) return;
+
+    C* X = reinterpret_cast<C*>(smem_raw);
+    Real* NZ = reinterpret_cast<Real*>(X + (size_t)chunk * Nc);
+    C* W = reinterpret_cast<C*>(NZ);
+    Real* S = NZ + (size_t)chunk * n_units * UV;
+    Real* NY = S + (size_t)n_units * NU;
+    C* RT = reinterpret_cast<C*>(NY + (size_t)chunk * ROW);
+    const Real* anc = (const Real*)P.anc;
+    const Real* xrg = anc + aoff<M>(P, c, r, has_right ? sg.right : 0, 0, 0);
+    const Real* xlg = anc + aoff<M>(P, c, r, sg.left, 0, 0);
+    const TabT* steps = (const TabT*)(c == 0 ? P.steps[0] : P.steps[1]);
+    if (tid < kKeyWords) rk[tid] = round_key_word(P.seed + (uint64_t)r, tid);
+    for (int u = tid; u < n_units; u += nt) {
+        Real v[NU];
+        VecN<Real, NU>::ldg(xlg + (size_t)NU * u, v);
+        VecN<Real, NU>::st(S + (size_t)NU * u, v);
+    }
+    __syncthreads();
+
+    for (int c0 = sg.p0; c0 < own1; c0 += chunk) {
+        const int nk = min(chunk, own1 - c0);
+        const int ring0 = c == 0 ? P.k0 - c0 : P.k0 + c0, dir = c == 0 ? -1 : 1;  // ring of pos c0 + k: ring0 + dir k
+        for (int idx = tid; idx < nk * n_units; idx += nt) {
+            const int k = idx / n_units, u = idx - k * n_units;
+            if (c0 + k == sg.p0) continue;  // the segment's left end: its state is the anchor's
+            Real* w = NZ + (size_t)idx * UV;
+            const TabT* tb = steps + (size_t)(c0 + k) * mp * ROW;
+            if constexpr (STAGE) {
+                Real t[G][ROW];
+                band_rows<Real, TabT, M>(tb, u, t);
+#pragma unroll
+                for (int g = 0; g < G; ++g) VecN<Real, ROW>::st(w + NU + g * ROW, t[g]);
+            }
+            if (u == 0) {
+                Real tn[ROW];
+                load_row<Real, TabT, ROW>(tb + (size_t)Nc * ROW, tn);
+                VecN<Real, ROW>::st(NY + (size_t)k * ROW, tn);
+            }
+            Real nr[NU];
+            unit_normals_rk<Real, NC>(rk, (uint32_t)u, (uint32_t)(ring0 + dir * k), nr);
+            VecN<Real, NU>::st(w, nr);
+        }
+        __syncthreads();
+        if constexpr (STAGE) {
+            // one thread per real chain f (slot f / 2, Re or Im): a small grid has few units, and in
+            // FP64 a warp's multiply-add holds the SM's two lanes for 16 cycles
+            for (int f = tid; f < 2 * Nc; f += nt) {
+                const int u = f / (2 * G), in_unit = f - u * 2 * G;
+                Real x[M], xr[M];
+#pragma unroll
+                for (int q = 0; q < M; ++q) {
+                    x[q] = S[(size_t)f * M + q];
+                    xr[q] = has_right ? __ldg(xrg + (size_t)f * M + q) : (Real)0;
+                }
+#pragma unroll 2
+                for (int k = 0; k < nk; ++k) {
+                    const int pos = c0 + k;
+                    if (pos > sg.p0) {
+                        const Real* w = NZ + ((size_t)k * n_units + u) * UV;
+                        // chain 1 is the Nyquist mode's (its own table row)
+                        const Real* row = f == 1 ? NY + (size_t)k * ROW : w + NU + (in_unit >> 1) * ROW;
+                        Real t[ROW], xi[M];
+                        VecN<Real, ROW>::ld(row, t);
+#pragma unroll
+                        for (int q = 0; q < M; ++q) xi[q] = w[in_unit * M + q];
+                        if (has_right) step_state<Real, M, true>(t, x, xi, xr);
+                        else step_state<Real, M, false>(t, x, xi, nullptr);
+                    }
+                    if (pos >= own0) reinterpret_cast<Real*>(X)[(size_t)k * 2 * Nc + f] = x[0];
+                }
+#pragma unroll
+                for (int q = 0; q < M; ++q) S[(size_t)f * M + q] = x[q];
+            }
+        } else {
+            for (int u = tid; u < n_units; u += nt) {
+                Real x[NU], xr[NU];
+                VecN<Real, NU>::ld(S + (size_t)NU * u, x);
+                if (has_right) VecN<Real, NU>::ldg(xrg + (size_t)NU * u, xr);
+#pragma unroll 2
+                for (int k = 0; k < nk; ++k) {
+                    const int pos = c0 + k;
+                    if (pos > sg.p0) {
+                        Real nr[NU], t[G][ROW];
+                        VecN<Real, NU>::ld(NZ + ((size_t)k * n_units + u) * UV, nr);
+                        band_rows<Real, TabT, M>(steps + (size_t)pos * mp * ROW, u, t);
+                        band_step<Real, M>(t, NY + (size_t)k * ROW, u == 0, has_right, nr, xr, x);
+                    }
+                    if (pos >= own0) put_unit<C, Real, M>(X + (size_t)k * Nc, u, x);
+                }
+                VecN<Real, NU>::st(S + (size_t)NU * u, x);
+            }
+        }
+        __syncthreads();
+        const int k0 = max(0, own0 - c0);
+        if (k0 >= nk) continue;  // nothing of this chunk is this CTA's (NZ is rewritten: no reader is left)
+        if (P.ring_n) {
+            // whole rings with an offset become whole rings without one; rings of their own
+            // point count are synthesised by the thread groups
+            const int gs = band_group(Nc), g = tid / gs, groups = nt / gs;
+            for (int k = k0; k < nk; ++k) {
+                const int ring = ring0 + dir * k;
+                const uint64_t ph = P.ring_ph[ring];
+                if (P.ring_n[ring] != P.n_phi || ph == 0) continue;
+                C* x = X + (size_t)k * Nc;
+                for (int s = tid; s < Nc; s += nt) {
+                    if (s == 0) x[0].y *= cis_turns<Real>((uint64_t)Nc * ph).x;
+                    else x[s] = cmul(x[s], cis_turns<Real>((uint64_t)s * ph));
+                }
+            }
+            int turn = 0;
+            for (int k = k0; k < nk; ++k) {
+                const int ring = ring0 + dir * k, n = P.ring_n[ring];
+                if (n == P.n_phi) continue;
+                if (turn++ % groups != g) continue;
+                band_ragged_ring<Real>(X + (size_t)k * Nc, W + (size_t)k * Nc, RT + (size_t)g * Nc, Nc, n, P.ring_ph[ring],
+                                       (C*)((Real*)P.out + (size_t)r * P.ring_total + P.ring_off[ring]), tid - g * gs, gs, g);
+            }
+            __syncthreads();
+        }
+        for (int k = k0; k < nk;) {
+            // a run of whole rings: their FFTs together
+            int e = nk;
+            const int ring = ring0 + dir * k;
+            C* base = (C*)((Real*)P.out + ((size_t)r * P.n_theta + ring) * (size_t)P.n_phi);
+            if (P.ring_n) {
+                if (P.ring_n[ring] != P.n_phi) {
+                    ++k;
+                    continue;
+                }
+                for (e = k + 1; e < nk && P.ring_n[ring0 + dir * e] == P.n_phi;) ++e;
+                base = (C*)((Real*)P.out + (size_t)r * P.ring_total + P.ring_off[ring]);
+            }
+            const RingOut<C> gout{base, (size_t)((long long)dir * Nc), (reinterpret_cast<uintptr_t>(base) & 15) == 0};
+            C* x = X + (size_t)k * Nc;
+            C* w = W + (size_t)k * Nc;
+            const C* pre = (const C*)P.pre;
+            if constexpr (sizeof(Real) == 4) {
+                if (!P.fft_r4) hr_c2r<C, 2, 12, true>(P.lgNc, x, w, e - k, (const C*)P.tw, (const C*)P.tw2, pre, gout, tid, nt);
+                else grp_c2r_rt<C>(x, w, e - k, P.lgNc, (const C*)P.tw, pre, gout, tid, nt);
+            } else {
+                grp_c2r_rt<C>(x, w, e - k, P.lgNc, (const C*)P.tw, pre, gout, tid, nt);
+            }
+            k = e;
+        }
+        __syncthreads();  // X and W (the noise) are rewritten by the next chunk
+    }
+}
+
+}  // namespace smerf

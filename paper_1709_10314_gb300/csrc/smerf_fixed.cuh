@@ -163,10 +163,9 @@ SMERF_HD void fx_sqrt2(uint64_t m, int x, uint64_t& r, int& xr)
     if (!(r >> 63)) r = s1 > (3ull << 61) ? ~0ull : 1ull << 63;  // within rounding of 1 or of 1/2
 }
 
-// Box-Muller: n0 + i n1 = sqrt(-2 ln u0) e^{2 pi i u1}, u = (word + 1/2) 2^-32
+// (r 2^(xr - 64)) (t 2^(xt - 64)) rounded to a double
 SMERF_HD double fx_normal(uint64_t r, int xr, uint64_t t, int xt, bool neg)
 {
-    // (r 2^(xr - 64)) (t 2^(xt - 64)), rounded to 53 bits
     const uint64_t p = fx_mulhi(r, t);
     const int n = fx_clz(p);
     const uint64_t m = ((p << n) >> 11) + (((p << n) >> 10) & 1);  // 2^52 .. 2^53
@@ -174,19 +173,12 @@ SMERF_HD double fx_normal(uint64_t r, int xr, uint64_t t, int xt, bool neg)
     const uint64_t bits = ((uint64_t)(uint32_t)(1022 + xr + xt - n - 1) << 52) + m;
     return fx_double(bits | (neg ? 0x8000000000000000ull : 0ull));
 }
-SMERF_HD void fx_box_muller(uint32_t a, uint32_t b, FxLog lt, double& n0, double& n1)
+// t = T 2^-64 in [0, 1): S with sin(pi/4 t) = t S 2^-64, and cos(pi/4 t) as a 64-bit fraction
+SMERF_HD void fx_octant(uint64_t T, uint64_t& sn, uint64_t& cs)
 {
-    uint64_t m, r;
-    int x, xr;
-    fx_neg_log(a, lt, m, x);
-    fx_sqrt2(m, x, r, xr);
-    // octant and the angle pi/4 T 2^-64 within it, reflected in the odd ones
-    const int o = (int)(b >> 29);
-    uint32_t w = 2 * (b & 0x1fffffffu) + 1;  // of 2^30
-    if (o & 1) w = (1u << 30) - w;
-    const uint64_t T = (uint64_t)w << 34, T2 = fx_mulhi(T, T);
+    const uint64_t T2 = fx_mulhi(T, T);
     const uint32_t th = (uint32_t)(T2 >> 32);
-    // sin(pi/4 t) = t S(t^2), cos(pi/4 t) = 1 - D(t^2): Taylor series
+    // sin(pi/4 t) = t S(t^2), cos(pi/4 t) = 1 - t^2 D(t^2): Taylor series
     uint32_t q = 0x0000b7d7u - fx_mulhi(th, 0x0000006bu);
     q = 0x00f47a1au - fx_mulhi(th, q);
     q = 0xf183a7efu - fx_mulhi(th, q);
@@ -203,9 +195,36 @@ SMERF_HD void fx_box_muller(uint32_t a, uint32_t b, FxLog lt, double& n0, double
     D = 0x00155d3c7e3cbffaull - fx_mulhi(T2, D);
     D = 0x040f07c206d6b0edull - fx_mulhi(T2, D);
     D = 0x4ef4f326f9177969ull - fx_mulhi(T2, D);
-    const uint64_t cs = 0ull - (fx_mulhi(T2, D) | 1);       // in [0.707, 1)
+    sn = S;
+    cs = 0ull - (fx_mulhi(T2, D) | 1);  // in [0.707, 1)
+}
+// e^{2 pi i p}, p = ph 2^-64 turns, to 2^-63 (four FP64 instructions)
+SMERF_HD void fx_cis(uint64_t ph, double& c, double& s)
+{
+    const int o = (int)(ph >> 61);
+    uint64_t T = ph << 3, S, cs;
+    if (o & 1) T = ~T;
+    fx_octant(T, S, cs);
+    const double a = (double)(int64_t)(fx_mulhi(T, S) >> 1) * 0x1p-63, b = (double)(int64_t)(cs >> 1) * 0x1p-63;
+    const bool swap = (o + 1) & 2;
+    c = ((o + 2) & 4) ? -(swap ? a : b) : (swap ? a : b);
+    s = (o & 4) ? -(swap ? b : a) : (swap ? b : a);
+}
+// Box-Muller: n0 + i n1 = sqrt(-2 ln u0) e^{2 pi i u1}, u = (word + 1/2) 2^-32
+SMERF_HD void fx_box_muller(uint32_t a, uint32_t b, FxLog lt, double& n0, double& n1)
+{
+    uint64_t m, r, S, cs;
+    int x, xr;
+    fx_neg_log(a, lt, m, x);
+    fx_sqrt2(m, x, r, xr);
+    // octant and the angle pi/4 T 2^-64 within it, reflected in the odd ones
+    const int o = (int)(b >> 29);
+    uint32_t w = 2 * (b & 0x1fffffffu) + 1;  // of 2^30
+    if (o & 1) w = (1u << 30) - w;
+    const uint64_t T = (uint64_t)w << 34;
+    fx_octant(T, S, cs);
     const int lw = fx_clz(T);
-    const uint64_t sn = fx_mulhi(T << lw, S);                // sin 2^(64 + lw)
+    const uint64_t sn = fx_mulhi(T << lw, S);  // sin 2^(64 + lw)
     const bool swap = (o + 1) & 2;
     n0 = fx_normal(r, xr, swap ? sn : cs, swap ? -lw : 0, (o + 2) & 4);
     n1 = fx_normal(r, xr, swap ? cs : sn, swap ? 0 : -lw, o & 4);

@@ -73,7 +73,7 @@ struct smerf_plan {
     int dev;
     // ring-dependent longitudes (smerf_plan_set_rings; rings_total = 0: none)
     int* rings_n_dev;
-    double* rings_h_dev;
+    unsigned long long* rings_ph_dev;  // offsets as 64-bit fractions of a turn
     long long* rings_off_dev;
     long long rings_total;
     // launch parameters chosen by smerf_plan_autotune (valid = 0: built-in heuristic)
@@ -113,10 +113,10 @@ struct SampleParams {
     int lgNc;
     int fft_r4;       // warp-specialised kernel, FP32: 1 = radix-4 FFT passes, 0 = the high-radix plan
     // iso-latitude grid with ring-dependent longitudes (null: the full n_theta x n_phi grid):
-    // ring k holds ring_n[k] points from phi0 = ring_h[k] pi, at ring_off[k] within a
+    // ring k holds ring_n[k] points from phi0 = 2 pi ring_ph[k] 2^-64, at ring_off[k] within a
     // realisation of ring_total points
     const int* ring_n;
-    const double* ring_h;
+    const unsigned long long* ring_ph;
     const long long* ring_off;
     long long ring_total;
 };

@@ -428,6 +428,106 @@ __global__ void __launch_bounds__(128, anchor_minb(4, M)) anchor_stage_kernel(Sa
     h.rest(stepped);
 }
 
+// The same anchors by CTAs of 32 units: kTileProducers warps draw the normals of the next
+// kTileAnchors anchors into shared memory while 2 G warps, one thread per real chain (slot, Re or
+// Im), walk the anchors before them, their table values fetched tile_ahead(M) anchors ahead.  A
+// thread of anchor_kernel draws and steps in turn, so an anchor costs the noise's latency (0.9 us
+// and up, 8 to 13 warps per SM); here the walk waits for two multiply-adds per anchor.  The
+// operations of a chain are anchor_body's in its order (the same states bit for bit).
+constexpr int kTileProducers = 8;
+__host__ __device__ constexpr int tile_anchors(int M) { return M == 3 ? 4 : 8; }
+__host__ __device__ constexpr int tile_ahead(int M) { return M == 3 ? 4 : 8; }
+__host__ __device__ constexpr int tile_threads(int M) { return 32 * (kTileProducers + 2 * unit_slots(M)); }
+template <class Real, class TabT, int M>
+__global__ void __launch_bounds__(tile_threads(M)) anchor_tile_kernel(SampleParams P)
+{
+    constexpr int G = kG<M>, Ec = coarse_elems(M), NU = unit_vals(M), NC = unit_calls(M);
+    constexpr int CH = tile_anchors(M), AD = tile_ahead(M);
+    __shared__ Real nz[2][CH][NU][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int u = blockIdx.x * 32 + lane, r = blockIdx.y, c = blockIdx.z;
+    const uint64_t key = P.seed + (uint64_t)r;
+    const int na = c == 0 ? P.n_anchors[0] : P.n_anchors[1];
+    const int chunks = (na + CH) / CH;  // anchors 0 (the start ring) .. na
+    const int g = (warp - kTileProducers) >> 1, part = warp & 1, s = G * u + g;
+    const bool walker = warp >= kTileProducers, live = walker && u < P.n_units;
+    const size_t mp = P.n_modes_pad;
+    const TabT* tb = (const TabT*)(c == 0 ? P.coarse[0] : P.coarse[1]) + ((part == 1 && s == 0) ? P.Nc : s);
+    Real* anc = (Real*)P.anc;
+    Real x[M], tq[AD][Ec];
+    if (live) {
+#pragma unroll
+        for (int d = 0; d < AD; ++d)
+            if (1 + d <= na) {
+#pragma unroll
+                for (int e = 0; e < Ec; ++e) tq[d][e] = tabcvt<Real, TabT>(__ldg(tb + ((size_t)(1 + d) * Ec + e) * mp));
+            }
+    }
+    for (int i = 0; i <= chunks; ++i) {
+        if (!walker) {
+            for (int it = warp; it < CH * NC && i < chunks; it += kTileProducers) {
+                const int a = it / NC, k = it - a * NC, j = i * CH + a;
+                if (j > na) break;
+                Real n[4];
+                const uint32_t ring = (uint32_t)(c == 0 ? P.k0 - j * P.H : P.k0 + j * P.H);
+                const uint4 w = philox4x32_10(make_uint4((uint32_t)(u * NC + k), ring, 0u, 0u),
+                                              PhiloxKey{(uint32_t)key, (uint32_t)(key >> 32)});
+                box_muller(w.x, w.y, n[0], n[1]);
+                box_muller(w.z, w.w, n[2], n[3]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) nz[i & 1][a][4 * k + q][lane] = n[q];
+            }
+        } else if (i > 0 && live) {
+            const int f = g * 2 * M + part * M;  // the chain's first normal and state value
+#pragma unroll
+            for (int a = 0; a < CH; ++a) {
+                const int j = (i - 1) * CH + a;
+                if (j > na) break;
+                Real nr[M];
+#pragma unroll
+                for (int q = 0; q < M; ++q) nr[q] = nz[(i - 1) & 1][a][f + q][lane];
+                if (j == 0) {
+                    // start ring: x = B_eq xi; the southern chain keeps S x
+                    const TabT* bq = (const TabT*)P.beq + ((part == 1 && s == 0) ? P.Nc : s);
+                    int e = 0;
+#pragma unroll
+                    for (int p = 0; p < M; ++p) {
+                        Real acc = 0;
+#pragma unroll
+                        for (int q = 0; q <= p; ++q, ++e) acc += tabld<Real, TabT>(bq + (size_t)e * mp) * nr[q];
+                        x[p] = (c == 1 && (p & 1)) ? -acc : acc;
+                    }
+                } else {
+                    // anchor j's values sit in ring slot (j - 1) mod AD = (a - 1) mod AD (CH a multiple of AD)
+                    static_assert(CH % AD == 0, "ring slots by the anchor's place in its chunk");
+                    Real(&t)[Ec] = tq[(a + AD - 1) % AD];
+                    Real xn[M];
+#pragma unroll
+                    for (int p = 0; p < M; ++p) {
+                        Real acc = 0;
+#pragma unroll
+                        for (int q = 0; q < M; ++q) acc += t[p * M + q] * x[q];
+                        int e = M * M + p * (p + 1) / 2;
+#pragma unroll
+                        for (int q = 0; q <= p; ++q, ++e) acc += t[e] * nr[q];
+                        xn[p] = acc;
+                    }
+#pragma unroll
+                    for (int q = 0; q < M; ++q) x[q] = xn[q];
+                    if (j + AD <= na) {
+#pragma unroll
+                        for (int e = 0; e < Ec; ++e) t[e] = tabcvt<Real, TabT>(__ldg(tb + ((size_t)(j + AD) * Ec + e) * mp));
+                    }
+                }
+                Real* dst = anc + aoff<M>(P, c, r, j, part * M, s);
+#pragma unroll
+                for (int q = 0; q < M; ++q) dst[q] = x[q];
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // batched: item = (request, block of 128 units, realisation, chain)
 template <class Real, class TabT, int M>
 __global__ void __launch_bounds__(128, anchor_minb(sizeof(Real), M)) anchor_batched_kernel(const SampleParams* __restrict__ descs,
@@ -441,10 +541,12 @@ __global__ void __launch_bounds__(128, anchor_minb(sizeof(Real), M)) anchor_batc
 
 // ------------------------------------------------------------------ FFT
 // Output rows of ring `ring` for the realisations of a CTA: gout[r] = base + r * stride
-// (complex elements; stride = one realisation, n_theta x n_phi / 2).
+// (complex elements; stride = one realisation, n_theta x n_phi / 2).  wide: every row starts on a
+// 16-byte boundary (rings of their own point counts may start on 8 bytes).
 template <class C> struct RingOut {
     C* base;
     size_t stride;
+    bool wide = true;
     __device__ __forceinline__ C* operator[](int r) const { return base + (size_t)r * stride; }
 };
 
@@ -1045,8 +1147,14 @@ __device__ __forceinline__ void hr_pass(const C* __restrict__ src, C* __restrict
             if constexpr (LAST) {
                 C* D = gout[r] + idx;
 #pragma unroll
-                for (int a = 0; a < RP; ++a)
-                    __stcs(reinterpret_cast<float4*>(D + a * Ns), make_float4(v0[a].x, v0[a].y, v1[a].x, v1[a].y));
+                for (int a = 0; a < RP; ++a) {
+                    if (gout.wide) {
+                        __stcs(reinterpret_cast<float4*>(D + a * Ns), make_float4(v0[a].x, v0[a].y, v1[a].x, v1[a].y));
+                    } else {
+                        __stcs(D + a * Ns, v0[a]);
+                        __stcs(D + a * Ns + 1, v1[a]);
+                    }
+                }
             } else {
                 // hr_swz(idx + a Ns + 1) = hr_swz(idx + a Ns) ^ 1 (idx + a Ns even)
                 float4* D = reinterpret_cast<float4*>(dst + (r << LGNC));
@@ -1140,167 +1248,6 @@ __host__ __device__ constexpr int ws_lg_hi(int UPT, int M)
                : 12;
 }
 
-// ---- iso-latitude grids with ring-dependent longitudes (the paper's Sec. 1 remark)
-// e^{i pi x} for a real x given in half-turns, reduced to [-1, 1) in FP64 first so that the
-// phase of a large multiple of a small offset keeps full accuracy
-template <class Real> __device__ __forceinline__ cplx<Real> cis_halfturns(double x)
-{
-    x -= 2.0 * floor(0.5 * x + 0.5);
-    Real sn, cs;
-    if constexpr (sizeof(Real) == 4) sincospif((float)x, &sn, &cs);
-    else sincospi(x, &sn, &cs);
-    return cmk<cplx<Real>>(cs, sn);
-}
-
-// e^{2 pi i a / n} for integers 0 <= a < n: the fraction 2a / n in the recursion precision (exact
-// for a power-of-two n, within half an ulp otherwise), then sincospi
-template <class Real> __device__ __forceinline__ cplx<Real> ring_phase(int a, int n)
-{
-    Real sn, cs;
-    if constexpr (sizeof(Real) == 4) sincospif(2.0f * (float)a / (float)n, &sn, &cs);
-    else sincospi(2.0 * (double)a / (double)n, &sn, &cs);
-    return cmk<cplx<Real>>(cs, sn);
-}
-
-// Ring `ring` of n = 2 Ncp points from phi0 = h pi: the C2R input X' (slot 0 = (Y_0, Y_Ncp),
-// slot q = Y_q) of the real field T(phi) = sum_{|m| <= M} c_m e^{i m phi} at its points, where
-// c_0 = g_0, c_{+-m} = g_m, conj g_m (0 < m < M) and c_{+-M} = Re g_M / 2 (the Nyquist mode's real
-// part); Y_q = sum over m = q (mod n) of c_m e^{i m phi0} (modes above the ring's own Nyquist
-// alias onto it).  B: the ring's coefficients (slot 0 = (g_0, Re g_M), slot m = g_m) at stride
-// Nc per realisation; W: the folded rings at stride Ncp.
-template <class Real>
-__device__ __forceinline__ void ring_fold(const cplx<Real>* B, cplx<Real>* W, int R, int Nc, int n, double h, int ftid,
-                                          int nf)
-{
-    using C = cplx<Real>;
-    const int Ncp = n / 2, M = Nc;
-    // e^{i m phi0} along m = m0 + k n: exact (FP64-reduced) every 16 terms, products by
-    // e^{i n phi0} between, so that rounding grows over at most 16 products
-    const C step = cis_halfturns<Real>(h * n);
-    for (int idx = ftid; idx < R * (Ncp + 1); idx += nf) {
-        const int r = idx / (Ncp + 1), q = idx - r * (Ncp + 1);
-        const C* X = B + (size_t)r * Nc;
-        C acc = cmk<C>(0, 0);
-        C e = cmk<C>(1, 0);
-        int k = 0;
-        for (int m = q; m <= M; m += n, ++k) {  // m >= 0
-            e = (k & 15) == 0 ? cis_halfturns<Real>(h * m) : cmul(e, step);
-            const C g = m == 0 ? cmk<C>(X[0].x, 0) : (m == M ? cmk<C>((Real)0.5 * X[0].y, 0) : X[m]);
-            acc = cadd(acc, m == 0 ? g : cmul(g, e));
-        }
-        k = 0;
-        for (int m = q == 0 ? n : n - q; m <= M; m += n, ++k) {  // the conjugate terms, -m < 0
-            e = (k & 15) == 0 ? cis_halfturns<Real>(h * m) : cmul(e, step);
-            const C g = m == M ? cmk<C>((Real)0.5 * X[0].y, 0) : X[m];
-            acc = cadd(acc, cconj(cmul(g, e)));
-        }
-        C* Y = W + (size_t)r * Ncp;
-        if (q == 0) Y[0].x = acc.x;
-        else if (q == Ncp) Y[0].y = acc.x;
-        else Y[q] = acc;
-    }
-}
-
-// C2R of R rings of n = 2 Ncp points (Ncp = 2^lg >= 2) from their folded input in src (stride
-// Ncp), ping-ponging with dst, last pass to gout: radix-4 Stockham passes (radix 2 last when lg
-// is odd) with the twiddles computed, the packing factors e^{2 pi i s / n} = pre[s pstride] from
-// the plan's table of its full ring.
-template <class C>
-__device__ __forceinline__ void ragged_c2r(C* src, C* dst, int R, int lg, const C* __restrict__ pre, int pstride,
-                                           RingOut<C> gout, int ftid, int nf)
-{
-    using Real = decltype(C::x);
-    const int Nc = 1 << lg;
-    int Ns = 1;
-    bool first = true;
-    while (Ns < Nc) {
-        const int RP = Nc / Ns >= 4 ? 4 : 2, LR = RP == 4 ? 2 : 1;
-        const bool last = Ns * RP == Nc;
-        const int lgnb = lg - LR, nb = 1 << lgnb, total = R << lgnb;
-        for (int b = ftid; b < total; b += nf) {
-            const int r = b >> lgnb, j = b & (nb - 1);
-            const C* S = src + ((size_t)r << lg);
-            C v[4];
-            int kk = 0;
-            if (first) {
-                for (int i = 0; i < RP; ++i) {
-                    const int sidx = j + i * nb;
-                    if (sidx == 0) {
-                        v[i] = cmk<C>(S[0].x + S[0].y, S[0].x - S[0].y);
-                    } else {
-                        const C a = S[sidx], bb = cconj(S[Nc - sidx]);
-                        v[i] = cadd(cadd(a, bb), cmuli(cmul(__ldg(pre + (size_t)sidx * pstride), csub(a, bb))));
-                    }
-                }
-            } else {
-                kk = j & (Ns - 1);
-                for (int i = 0; i < RP; ++i) v[i] = S[j + i * nb];
-                for (int i = 1; i < RP; ++i) v[i] = cmul(v[i], ring_phase<Real>(i * kk, Ns * RP));
-            }
-            if (RP == 4) dft4(v);
-            else dft2(v[0], v[1]);
-            const int idx = ((j - kk) << LR) + kk;
-            if (last) {
-                C* D = gout[r] + idx;
-                for (int a = 0; a < RP; ++a) __stcs(D + a * Ns, v[a]);
-            } else {
-                C* D = dst + ((size_t)r << lg) + idx;
-                for (int a = 0; a < RP; ++a) D[a * Ns] = v[a];
-            }
-        }
-        Ns *= RP;
-        first = false;
-        if (!last) bar_sync(kBarFft, nf);
-        C* t = src;
-        src = dst;
-        dst = t;
-    }
-}
-
-// Rings of an even point count n that is not a power of two (HEALPix polar caps): the real
-// synthesis T_j = Y_0 + (-1)^j Y_{n/2} + 2 sum_{0<q<n/2} Re(Y_q e^{2 pi i q j / n}) of the folded
-// input directly, O(n^2) per ring; the phases e^{2 pi i q j / n} exact (integer reduction of
-// q j mod n) every 16 terms and products by e^{2 pi i j / n} between.
-template <class Real>
-__device__ __forceinline__ void ring_direct(const cplx<Real>* W, int R, int n, cplx<Real>* gbase, size_t gstride,
-                                            int ftid, int nf)
-{
-    using C = cplx<Real>;
-    const int Ncp = n / 2;
-    for (int idx = ftid; idx < R * n; idx += nf) {
-        const int r = idx / n, j = idx - r * n;
-        const C* Y = W + (size_t)r * Ncp;
-        Real t = Y[0].x + ((j & 1) ? -Y[0].y : Y[0].y);
-        const C w = ring_phase<Real>(j, n);
-        C e = w;
-        for (int q = 1; q < Ncp; ++q) {
-            if ((q & 15) == 0) e = ring_phase<Real>((int)(((long long)q * j) % n), n);
-            t += (Real)2 * (Y[q].x * e.x - Y[q].y * e.y);
-            e = cmul(e, w);
-        }
-        reinterpret_cast<Real*>(gbase + (size_t)r * gstride)[j] = t;
-    }
-}
-
-// A ring whose point count or offset differs from the plan's full ring: fold, then the
-// runtime-size C2R (n a power of two) or the direct synthesis (other even n).  Not inlined, so
-// that the warp-specialised bodies keep their register allocation for the full-ring path.
-template <class Real>
-__device__ __noinline__ void ragged_ring(cplx<Real>* B, cplx<Real>* W, int R, int Nc, int n, double h,
-                                         const cplx<Real>* pre, int n_phi, cplx<Real>* gbase, size_t gstride,
-                                         int ftid, int nf)
-{
-    ring_fold<Real>(B, W, R, Nc, n, h, ftid, nf);
-    bar_sync(kBarFft, nf);
-    if (n & (n - 1)) {
-        ring_direct<Real>(W, R, n, gbase, gstride, ftid, nf);
-        return;
-    }
-    int lg = 0;
-    while ((2 << lg) < n) ++lg;
-    ragged_c2r<cplx<Real>>(W, B, R, lg, pre, n_phi / n, RingOut<cplx<Real>>{gbase, gstride}, ftid, nf);
-}
-
 // Warp-specialised segment kernel.  Threads [0, NP) are the producer group: the recursion of
 // ring k (state in registers, units tid, tid + NP, ...) into coefficient buffer B[k & 1].
 // Threads [NP, NP + NF) are the FFT group: the C2R FFT of ring k from B[k & 1] (with W as
@@ -1309,10 +1256,9 @@ __device__ __noinline__ void ragged_ring(cplx<Real>* B, cplx<Real>* W, int R, in
 //             syncs the two outstanding EMPTY barriers
 //   FFT:      sync FULL[k&1]; FFT; arrive EMPTY[k&1]
 // Every FULL/EMPTY barrier counts NP + NF threads; the FFT passes use a group barrier.
-// RINGS: the request may have ring-dependent longitudes (single-request launches; batches never do).
 // CG: the anchor states were written by the same launch (read through L2, not the read-only path).
 // PAIR: see hr_pass (false in the persistent batch kernels).
-template <class Real, class TabT, int M, int UPT, int RMAX, bool RINGS = true, bool CG = false, bool PAIR = true>
+template <class Real, class TabT, int M, int UPT, int RMAX, bool CG = false, bool PAIR = true>
 __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, int group)
 {
     using C = cplx<Real>;
@@ -1480,17 +1426,7 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
             if (!(c == 1 && pos == 0)) {  // the start ring is written by the northern chain
                 RingOut<C> gout{(C*)((Real*)P.out + ((size_t)r0 * P.n_theta + ring) * (size_t)P.n_phi),
                                 (size_t)P.n_theta * (size_t)(P.n_phi / 2)};
-                int n_ring = P.n_phi;
-                double h_ring = 0.0;
-                if (RINGS && P.ring_n) {  // ring-dependent longitudes: the rings lie back to back
-                    n_ring = P.ring_n[ring];
-                    h_ring = P.ring_h[ring];
-                    gout = RingOut<C>{(C*)((Real*)P.out + (size_t)r0 * P.ring_total + P.ring_off[ring]),
-                                      (size_t)(P.ring_total / 2)};
-                }
-                if (RINGS && (n_ring != P.n_phi || h_ring != 0.0)) {
-                    ragged_ring<Real>(B, W, R, Nc, n_ring, h_ring, pre, P.n_phi, gout.base, gout.stride, ftid, NF);
-                } else if (sizeof(Real) == 4 && !P.fft_r4) {
+                if (sizeof(Real) == 4 && !P.fft_r4) {
                     if constexpr (sizeof(Real) == 4)
                         hr_c2r<C, ws_lg_lo(UPT, M), ws_lg_hi(UPT, M), PAIR>(P.lgNc, B, W, R, twp, (const C*)P.tw2, pre, gout,
                                                                        ftid, NF);
@@ -1517,7 +1453,7 @@ __global__ void __launch_bounds__(ws_max_threads(MINB, M), MINB) segment_ws_batc
 {
     const int4 it = items[blockIdx.x];
     const SampleParams P = descs[it.x];
-    ws_body<Real, TabT, M, UPT, RMAX, false>(P, it.y, it.z);
+    ws_body<Real, TabT, M, UPT, RMAX>(P, it.y, it.z);
 }
 
 // ---- uneven batches: one persistent launch, or an anchor launch and a persistent launch
@@ -1593,7 +1529,7 @@ template <class Real, class TabT, int SH>
 __device__ __forceinline__ void queue_segment(const SampleParams& P, int seg, int grp)
 {
     constexpr int M = SH / kQueueBuilds + 1, B = SH % kQueueBuilds;
-    ws_body<Real, TabT, M, queue_upt(B), queue_rmax(B), false, true, false>(P, seg, grp);
+    ws_body<Real, TabT, M, queue_upt(B), queue_rmax(B), true, false>(P, seg, grp);
 }
 
 template <class Real, class TabT>
@@ -1661,7 +1597,7 @@ template <class Real, class TabT, int SH>
 __device__ __forceinline__ void queue_segment_after(const SampleParams& P, int seg, int grp)
 {
     constexpr int M = SH / kQueueBuilds + 1, B = SH % kQueueBuilds;
-    ws_body<Real, TabT, M, queue_upt(B), queue_rmax(B), false, false, false>(P, seg, grp);
+    ws_body<Real, TabT, M, queue_upt(B), queue_rmax(B), false, false>(P, seg, grp);
 }
 
 template <class Real, class TabT>
@@ -1694,6 +1630,7 @@ __global__ void __launch_bounds__(kQueueThreads, kQueueMinBlocks) segment_queue_
 
 }  // namespace smerf
 
+#include "smerf_band.cuh"
 #include "smerf_ring.cuh"
 
 namespace smerf {
@@ -1762,7 +1699,14 @@ int launch_inplace(const SampleParams& P, int n_segments, int nt, size_t smem, c
 // upt (<= 512), FFT threads np/2, rmax realisations per CTA (as many as registers and shared
 // memory allow).  Otherwise the in-place kernel (one FFT buffer, anchors read from the
 // scratch, one realisation per CTA, up to 1024 threads).
-struct SegConfig { int ws, upt, nt, np, rmax, park, minb; size_t smem; int ring; int radix; };
+struct SegConfig {
+    int ws, upt, nt, np, rmax, park, minb;
+    size_t smem;
+    int ring, radix;
+    int band_splits, band_chunk;  // > 0: the band kernel, so many CTAs per segment, rings per chunk
+    bool band_stage;
+    size_t band_smem;
+};
 
 // Long rings with p = 1 in FP32 (Nc = 8192 or 16384): the ring kernel (smerf_ring.cuh), NT =
 // Nc / 16 threads, 8 units per thread of which 6 are parked in shared memory; at Nc = 8192 two
@@ -1921,9 +1865,61 @@ inline SegConfig seg_config(const smerf_plan* pl)
     return cfg;
 }
 
+// Whether a request runs on the band kernel (smerf_band.cuh) in place of the warp-specialised one,
+// and with how many CTAs per segment and rings per chunk: always with ring-dependent longitudes;
+// else where the CTAs (segments x realisations) are few for the ring length.  Both kernels were
+// timed over n_phi 128 to 8192, p = 1 .. 3, FP32 and FP64, 1 to 256 realisations, Alg. 2's and the
+// anchored order.  In FP32 the band kernel wins while its CTAs fit the GPU two per SM (1.1 to 2.5
+// times; up to 3.7 in Alg. 2's order), longer for rings so short that its CTAs are brief (64
+// points up to 1280 CTAs); from 2048 complex points on it loses at every count.  In FP64 a split
+// segment repeats its recursion on the narrow FP64 pipe, so the line lies lower, and for p = 3
+// (24-value table rows) it stops at 128 points.
+template <class Real>
+inline void band_config(const smerf_plan* pl, int n, SegConfig& cfg)
+{
+    const int Nc = pl->n_phi / 2, M = pl->p;
+    const bool rings = pl->rings_total != 0;
+    const long long ctas = (long long)pl->n_segments * n;
+    long long most;
+    if (sizeof(Real) == 8 && Nc <= (M == 3 ? 32 : 64)) most = 1ll << 40;
+    else if (M == 3) most = Nc <= 128 ? 20480 / Nc : 0;
+    else if (sizeof(Real) == 8) most = Nc <= 512 ? 38912 / Nc : 0;
+    else most = Nc <= 128 ? 73728 / Nc : Nc <= 512 ? 304 : Nc <= 1024 && ctas >= 100 ? 304 : 0;
+    if (!rings && ctas > most) return;
+    const int seg_len = pl->H > 0 ? pl->H : (pl->chain[0].len > pl->chain[1].len ? pl->chain[0].len : pl->chain[1].len) + 1;
+    long long splits = ctas > 0 && ctas < 152 ? 152 / ctas : 1;  // one CTA per SM
+    if (splits > seg_len) splits = seg_len;
+    auto smem = [&](int chunk, bool stage) {
+        return M == 1 ? (stage ? band_smem<Real, 1, true>(Nc, chunk, rings) : band_smem<Real, 1, false>(Nc, chunk, rings))
+             : M == 2 ? (stage ? band_smem<Real, 2, true>(Nc, chunk, rings) : band_smem<Real, 2, false>(Nc, chunk, rings))
+                      : (stage ? band_smem<Real, 3, true>(Nc, chunk, rings) : band_smem<Real, 3, false>(Nc, chunk, rings));
+    };
+    size_t budget = ctas * splits <= 152 ? kMaxSmem : kMaxSmem / 2;
+    bool stage = Nc / unit_slots(M) <= 128 && smem(4, true) <= budget;
+    if (smem(1, stage) > budget) budget = kMaxSmem;
+    if (smem(1, stage) > budget) return;
+    int chunk = 1;
+    while (chunk < 16 && chunk < seg_len && smem(chunk + 1, stage) <= budget) ++chunk;
+    cfg.band_splits = (int)splits;
+    cfg.band_chunk = chunk;
+    cfg.band_stage = stage;
+    cfg.band_smem = smem(chunk, stage);
+}
+
+template <class Real, class TabT, int M>
+int launch_band(const SampleParams& P, int n_segments, const SegConfig& cfg, cudaStream_t st)
+{
+    auto kern = cfg.band_stage ? segment_band_kernel<Real, TabT, M, true> : segment_band_kernel<Real, TabT, M, false>;
+    if (set_smem_attr(kern, cfg.band_smem) != cudaSuccess) return SMERF_ECUDA;
+    dim3 grid(cfg.band_splits, P.n_samples, n_segments);
+    kern<<<grid, kBandThreads, cfg.band_smem, st>>>(P, cfg.band_chunk);
+    return cudaGetLastError() == cudaSuccess ? SMERF_OK : SMERF_ECUDA;
+}
+
 template <class Real, class TabT, int M>
 int dispatch_segments(const SampleParams& P, int n_segments, const SegConfig& cfg, cudaStream_t st)
 {
+    if (cfg.band_splits > 0) return launch_band<Real, TabT, M>(P, n_segments, cfg, st);
     if (cfg.ws) {
         if constexpr (sizeof(Real) == 8 || M == 3) {
             if (cfg.rmax != 1 || cfg.minb != 1) return SMERF_EUNSUPPORTED;
@@ -1985,7 +1981,8 @@ int dispatch_segments(const SampleParams& P, int n_segments, const SegConfig& cf
 
 // The request's kernel parameters and launch configuration.
 template <class Real, class TabT>
-int fill_params(const smerf_plan* pl, uint64_t seed, int n, void* out, void* scratch, SampleParams& P, SegConfig& cfg)
+int fill_params(const smerf_plan* pl, uint64_t seed, int n, void* out, void* scratch, SampleParams& P, SegConfig& cfg,
+                bool batch = false)
 {
     P.segs = pl->segs_dev;
     P.steps[0] = pl->steps[0];
@@ -2022,14 +2019,37 @@ int fill_params(const smerf_plan* pl, uint64_t seed, int n, void* out, void* scr
     while ((1 << lg) < P.Nc) ++lg;
     P.lgNc = lg;
     P.ring_n = pl->rings_total ? pl->rings_n_dev : nullptr;
-    P.ring_h = pl->rings_total ? pl->rings_h_dev : nullptr;
+    P.ring_ph = pl->rings_total ? pl->rings_ph_dev : nullptr;
     P.ring_off = pl->rings_total ? pl->rings_off_dev : nullptr;
     P.ring_total = pl->rings_total;
-    // ring-dependent longitudes are synthesised by the warp-specialised kernels' FFT group only,
-    // and p = 3 is built for those kernels only (rings up to 4096 complex points in FP32, 2048
-    // in FP64)
+    // ring-dependent longitudes (the band kernel) and p = 3 are built for the rings that the
+    // warp-specialised kernels hold (up to 4096 complex points in FP32, 2048 in FP64)
     if ((pl->rings_total || pl->p == 3) && !cfg.ws) return SMERF_EUNSUPPORTED;
+    if (cfg.ws && n > 0 && !batch) band_config<Real>(pl, n, cfg);
+    if (pl->rings_total && n > 0 && !batch && cfg.band_splits == 0) return SMERF_EUNSUPPORTED;
     return SMERF_OK;
+}
+
+// Whether a request's anchors run on anchor_tile_kernel: chains of a few anchors at least, and no
+// more CTAs than stay resident together (beyond them anchor_kernel's threads hide their own
+// latencies and the tiles' idle walkers cost).  Both ways over p = 1 .. 3, FP32 and FP64, n_phi 512
+// to 8192 and 1 to 256 realisations: up to 512 tiles 3 to 20 % faster per call or equal within 2 %,
+// from 1024 on as often slower as faster (by up to 6 %).
+inline bool use_tile(const SampleParams& P)
+{
+    return P.na_max >= 4 && 2ll * ((P.n_units + 31) / 32) * P.n_samples <= 512;
+}
+
+// The anchor launch of one request
+template <class Real, class TabT, int M>
+int launch_anchors(const SampleParams& P, cudaStream_t st)
+{
+    if (use_tile(P)) {
+        anchor_tile_kernel<Real, TabT, M><<<dim3((P.n_units + 31) / 32, P.n_samples, 2), tile_threads(M), 0, st>>>(P);
+    } else {
+        anchor_kernel<Real, TabT, M><<<dim3((P.n_units + 127) / 128, P.n_samples, 2), 128, 0, st>>>(P);
+    }
+    return cudaGetLastError() == cudaSuccess ? SMERF_OK : SMERF_ECUDA;
 }
 
 // Anchor and segment launches of one request (state size M = p).
@@ -2041,15 +2061,37 @@ int launch_sample_m(const smerf_plan* pl, uint64_t seed, int n, void* out, void*
     SegConfig cfg;
     int rc = fill_params<Real, TabT>(pl, seed, n, out, scratch, P, cfg);
     if (rc != SMERF_OK) return rc;
-    {
-        dim3 ga((P.n_units + 127) / 128, n, 2);
-        anchor_kernel<Real, TabT, M><<<ga, 128, 0, st>>>(P);
-        if (cudaGetLastError() != cudaSuccess) return SMERF_ECUDA;
-    }
+    rc = launch_anchors<Real, TabT, M>(P, st);
+    if (rc != SMERF_OK) return rc;
     if (ev0 && cudaEventRecord(ev0, st) != cudaSuccess) return SMERF_ECUDA;
     rc = dispatch_segments<Real, TabT, M>(P, pl->n_segments, cfg, st);
     if (rc == SMERF_OK && ev1 && cudaEventRecord(ev1, st) != cudaSuccess) return SMERF_ECUDA;
     return rc;
+}
+
+// All of a plan's FP64 tables -> FP32 in one launch (tabcvt), two elements per thread and step of
+// the grid: 16-byte loads and 8-byte stores, 12 bytes per element through HBM (156 MB in 23 us).
+// Element counts are multiples of 32 modes.
+constexpr int kStageThreads = 256;
+struct StageAll {
+    const double* src[5];
+    float* dst[5];
+    unsigned long long n[5];
+};
+static __global__ void __launch_bounds__(kStageThreads) stage_all_kernel(StageAll J)
+{
+    const size_t step = (size_t)gridDim.x * kStageThreads;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        const double2* src = reinterpret_cast<const double2*>(J.src[q]);
+        float2* dst = reinterpret_cast<float2*>(J.dst[q]);
+        const size_t n = J.n[q] / 2;
+#pragma unroll 4
+        for (size_t i = (size_t)blockIdx.x * kStageThreads + threadIdx.x; i < n; i += step) {
+            const double2 v = __ldcs(src + i);
+            dst[i] = make_float2(tabcvt<float, double>(v.x), tabcvt<float, double>(v.y));
+        }
+    }
 }
 
 // FP64 coarse and start tables -> FP32 (a few rows per mode; one element per thread)
@@ -2076,6 +2118,26 @@ int launch_sample_staged_m(const smerf_plan* sh, const StageSmall& S, StageJob J
     SegConfig cfg;
     int rc = fill_params<float, float>(sh, seed, n, out, scratch, P, cfg);
     if (rc != SMERF_OK) return rc;
+    if (use_tile(P)) {
+        // few anchor threads: they cannot carry the conversion, which takes the whole GPU instead
+        StageAll A;
+        unsigned long long most = 0;
+        for (int q = 0; q < 5; ++q) {
+            A.src[q] = q < kStageParts ? J.src[q] : S.src[q - kStageParts];
+            A.dst[q] = q < kStageParts ? J.dst[q] : S.dst[q - kStageParts];
+            A.n[q] = q < kStageParts ? J.n[q] : S.end[q - kStageParts] - (q > kStageParts ? S.end[q - kStageParts - 1] : 0u);
+            most = A.n[q] > most ? A.n[q] : most;
+        }
+        const unsigned long long blocks = (most / 2 + 4 * kStageThreads - 1) / (4 * kStageThreads);
+        stage_all_kernel<<<(unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), kStageThreads, 0, st>>>(A);
+        if (cudaGetLastError() != cudaSuccess) return SMERF_ECUDA;
+        rc = launch_anchors<float, float, M>(P, st);
+        if (rc != SMERF_OK) return rc;
+        if (ev0 && cudaEventRecord(ev0, st) != cudaSuccess) return SMERF_ECUDA;
+        rc = dispatch_segments<float, float, M>(P, sh->n_segments, cfg, st);
+        if (rc == SMERF_OK && ev1 && cudaEventRecord(ev1, st) != cudaSuccess) return SMERF_ECUDA;
+        return rc;
+    }
     if (S.end[2] > 0) {
         const unsigned blocks = (S.end[2] + 255) / 256;
         stage_small_kernel<<<blocks < 152 * 8 ? blocks : 152 * 8, 256, 0, st>>>(S);
@@ -2202,7 +2264,7 @@ int fill_params_c(const smerf_plan* pl, uint64_t seed, int n, void* out, void* s
                   int* batchable, int* rmax)
 {
     SegConfig cfg;
-    const int rc = fill_params<Real, TabT>(pl, seed, n, out, scratch, *P, cfg);
+    const int rc = fill_params<Real, TabT>(pl, seed, n, out, scratch, *P, cfg, true);
     *batchable = rc == SMERF_OK && cfg.ws;
     *rmax = cfg.rmax;
     return rc;
