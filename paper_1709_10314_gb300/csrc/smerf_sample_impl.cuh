@@ -1802,8 +1802,61 @@ inline int tune_candidates(const smerf_plan* pl, int* cand, int max_n)
     return n < max_n ? n : max_n;
 }
 
+// CTAs of a launch over the slots of `per_sm` CTAs on each of the 152 SMs, in whole waves
+inline long long waves(long long ctas, int per_sm) { return (ctas + 152ll * per_sm - 1) / (152ll * per_sm); }
+
+// The built-in choice where it differs from the general rule of seg_config below: (units per
+// producer thread, realisations per CTA, FFT threads as a fraction of the producers, CTAs per SM).
+// The general rule gives each producer as few units as fit, hence one large CTA per SM; a CTA of
+// fewer, busier producers lets two or three run on an SM and fill each other's barriers.  Timed
+// against every candidate over n_phi 256 to 8192, p = 1 .. 3 and 8 to 512 realisations; e.g. 1024 x
+// 2048, 64 realisations: p = 1 430 -> 387 us, p = 2 756 -> 621 us, p = 3 1714 -> 1401 us; 512 x 1024,
+// 512 realisations, p = 3 4048 -> 2601 us.  n = 0: many realisations (batches).
 template <class Real>
-inline SegConfig seg_config(const smerf_plan* pl)
+inline bool seg_choice(const smerf_plan* pl, int n, int& upt, int& rmax, int& nf, int& minb)
+{
+    const int M = pl->p, units = pl->n_slots / unit_slots(M);
+    const long long many = 1 << 20;
+    const long long ctas = n > 0 ? (long long)pl->n_segments * n : many;
+    rmax = 1;
+    minb = 1;
+    if (sizeof(Real) == 8) {
+        // the FP64 pipe is the limit: half the producers leave it to more FFT threads
+        if (M == 1 && units >= 128 && units <= 512) { upt = 2; nf = units / 2 < 128 ? units / 2 : 128; return true; }
+        if (M == 2 && units >= 256 && units <= 512) { upt = 2; nf = units / 4; return true; }
+        if (M == 2 && units == 1024) { upt = 4; nf = 128; return true; }
+        if (M == 3 && units == 256) { upt = 2; nf = 64; return true; }
+        return false;
+    }
+    if (M == 3) {
+        if (units == 128 && ctas >= 608) { upt = 2; nf = 32; return true; }
+        if (units == 256) { upt = 2; nf = 32; return true; }
+        // 160-thread CTAs three per SM against 384-thread CTAs one per SM, twice the time per wave
+        if (units == 512 && 2 * waves(ctas, 3) < waves(ctas, 1)) { upt = 4; nf = 32; return true; }
+        return false;
+    }
+    if (M == 2 && units == 128) { upt = 1; rmax = 4; nf = 32; return true; }
+    if (units == 256) { upt = 2; rmax = 2; nf = M == 1 ? 64 : 32; return true; }
+    if (units == 512) { upt = 4; nf = M == 1 ? 64 : 32; minb = M; return true; }
+    if (units == 1024 && M == 1) { upt = 4; nf = 128; return true; }
+    if (units == 1024) {
+        // 320-thread CTAs three per SM against 640-thread CTAs of two realisations one per SM
+        // (four fifths of the time per wave)
+        const long long pairs = n > 0 ? (long long)pl->n_segments * ((n + 1) / 2) : many / 2;
+        upt = 5 * waves(ctas, 3) <= 4 * waves(pairs, 1) ? 4 : 2;
+        rmax = upt == 4 ? 1 : 2;
+        nf = upt == 4 ? 64 : 128;
+        minb = upt == 4 ? 2 : 1;
+        return true;
+    }
+    if (units == 2048 && M == 2) { upt = 4; rmax = n == 1 ? 1 : 2; nf = 128; return true; }
+    if (units == 4096 && M == 2) { upt = 8; nf = 128; return true; }
+    return false;
+}
+
+// n: the realisations of the call (0: a batch's descriptors, whose launch must not depend on it)
+template <class Real>
+inline SegConfig seg_config(const smerf_plan* pl, int n)
 {
     SegConfig cfg{};
     const int M = pl->p;
@@ -1822,6 +1875,20 @@ inline SegConfig seg_config(const smerf_plan* pl)
         cfg.smem = ws_smem<Real>(pl, cfg.rmax);
         cfg.radix = pl->tune.radix;
         return cfg;
+    }
+    {
+        int upt, rmax, nf, minb;
+        if (seg_choice<Real>(pl, n, upt, rmax, nf, minb) && ws_smem<Real>(pl, rmax) <= kMaxSmem) {
+            cfg.ws = 1;
+            cfg.upt = upt;
+            cfg.rmax = rmax;
+            cfg.minb = minb;
+            cfg.np = (n_units + upt - 1) / upt;
+            cfg.nt = cfg.np + nf;
+            cfg.smem = ws_smem<Real>(pl, rmax);
+            cfg.radix = sizeof(Real) == 4 ? 16 : 4;
+            return cfg;
+        }
     }
     auto np_of = [&](int u) { return (((n_units + u - 1) / u + 31) / 32) * 32; };
     auto nf_of = [](int np) { return np / 2 > 32 ? ((np / 2 + 31) / 32) * 32 : 32; };
@@ -2008,7 +2075,7 @@ int fill_params(const smerf_plan* pl, uint64_t seed, int n, void* out, void* scr
     P.n_anchors[0] = pl->chain[0].n_anchors;
     P.n_anchors[1] = pl->chain[1].n_anchors;
     P.na_max = P.n_anchors[0] > P.n_anchors[1] ? P.n_anchors[0] : P.n_anchors[1];
-    cfg = seg_config<Real>(pl);
+    cfg = seg_config<Real>(pl, batch ? 0 : n);
     if (cfg.smem > kMaxSmem) return SMERF_EUNSUPPORTED;  // one ring per realisation must fit on chip
     if (!cfg.ws && (pl->n_slots / unit_slots(pl->p) + cfg.upt - 1) / cfg.upt > kMaxThreads) return SMERF_EUNSUPPORTED;
     if (pl->n_segments > 65535) return SMERF_EUNSUPPORTED;
@@ -2275,7 +2342,7 @@ template <class Real, class TabT, int M>
 int launch_group_m(const smerf_plan* rep, const SampleParams* d, const int4* anc_items, int n_anc,
                    const int4* seg_items, int n_seg, cudaStream_t st)
 {
-    const SegConfig cfg = seg_config<Real>(rep);
+    const SegConfig cfg = seg_config<Real>(rep, 0);
     if (!cfg.ws) return SMERF_EUNSUPPORTED;
     if (n_anc > 0) {
         anchor_batched_kernel<Real, TabT, M><<<n_anc, 128, 0, st>>>(d, anc_items);
