@@ -48,7 +48,6 @@ struct Spec {
     int M;
     double k2[kMaxP];     // kappa_i^2
     double b[kMaxP];      // partial-fraction weights (Eq. (C_ell_efficient))
-    double lG0[kMaxP];    // log Gamma(1+l_i) Gamma(-l_i)
     double A;
     double kmax;
     int n_theta, k0, n_modes, n_modes_pad;
@@ -84,15 +83,6 @@ __device__ void hyp_scaled(double k2, int mu, double x, double& S, int& E)
     }
     S = s;
     E = e;
-}
-
-// log of the same series
-__device__ double log_hyp(double k2, int mu, double x)
-{
-    double s;
-    int e;
-    hyp_scaled(k2, mu, x, s, e);
-    return log(s) + e * 575.64627324851142;
 }
 
 // the series relative to a reference value sref * 1e250^eref (given as 1/sref and eref)
@@ -168,6 +158,16 @@ template <> __device__ inline Mat<2> minv<2>(const Mat<2>& x)
 }
 template <> __device__ inline Mat<3> minv<3>(const Mat<3>& x) { return inv3<Mat<3>, double>(x); }
 
+// 1/x by two Newton steps r += r (1 - x r) from the hardware's approximation (20 bits), within an
+// ulp; x normal and well inside the range.  A division costs twice its FP64 instructions.
+__device__ inline double rcp_newton(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
 // lower Cholesky factor of a symmetric positive semi-definite matrix (0 where it degenerates)
 template <int M> __device__ inline Mat<M> mchol(const Mat<M>& x)
 {
@@ -189,15 +189,15 @@ template <int M> __device__ inline Mat<M> mchol(const Mat<M>& x)
 // inverse of a symmetric positive definite matrix through its Cholesky factor
 template <int M> __device__ inline Mat<M> mspd_inv(const Mat<M>& x)
 {
-    if (M == 1) { Mat<M> r; r.a[0][0] = 1.0 / x.a[0][0]; return r; }
+    if (M == 1) { Mat<M> r; r.a[0][0] = rcp_newton(x.a[0][0]); return r; }
     Mat<M> L = mchol<M>(x);
     Mat<M> Li = mzero<M>();  // L^{-1}, lower
     for (int i = 0; i < M; ++i) {
-        Li.a[i][i] = 1.0 / L.a[i][i];
+        Li.a[i][i] = rcp_newton(L.a[i][i]);
         for (int j = 0; j < i; ++j) {
             double s = 0.0;
             for (int k = j; k < i; ++k) s += L.a[i][k] * Li.a[k][j];
-            Li.a[i][j] = -s / L.a[i][i];
+            Li.a[i][j] = -s * Li.a[i][i];
         }
     }
     return mmul<M>(mT<M>(Li), Li);
@@ -293,7 +293,7 @@ __global__ void step_kernel(Spec sp, int c, int len, double* phi, double* qout)
         }
 }
 
-// ---- p = 1 with a real spectrum: the step tables by a recurrence in m (Alg. 1 sets up the
+// ---- p = 1 and 2 with a real spectrum: the step tables by a recurrence in m (Alg. 1 sets up the
 // hypergeometric functions of every order m).  For fixed x the series of
 // Eq. (Legendre_hypergeometric), F_m(x) = 2F1(-lambda, lambda+1; 1+m; x) with
 // (-lambda)(lambda+1) = kappa^2, satisfy Gauss's contiguous relation in the third parameter,
@@ -304,295 +304,235 @@ __global__ void step_kernel(Spec sp, int c, int len, double* phi, double* qout)
 // use, to a few 1e-13 over 16384 orders).  For x > 1/2 the error grows by x/(1-x) per order:
 // only the first step's equatorward ring can have x > 1/2 (south of the equator, even n_theta);
 // that step keeps step_kernel's per-mode series unless the growth over all orders,
-// (x/(1-x))^m_max, stays below 1e3 (it is about e^pi = 23 when n_phi = 2 n_theta).  Per step the
-// construction is step_kernel's for M = 1: A = (t2/t1)^m F_m(x2)/F_m(x1) and
-// Q = (A_amp/2 pi) int_0^du e^{-2 m v} (F_m(x2)/F_m(x(v)))^2 dv, on one node set for all m:
-// composite 8-point Gauss-Legendre panels no wider than 4/rho(m) for every m whose weight
-// e^{-2 m v} at the panel's start is above e^-46 (the same panel rule as step_kernel).
-constexpr int kRecWarps = 4;         // warps per block, one step each
-constexpr int kRecMaxPanels = 8192;  // node-set cap (reached only by grids far beyond 16384 rings)
+// (x/(1-x))^m_max, stays below 1e3 (it is about e^pi = 23 when n_phi = 2 n_theta).
+//
+// Per order m a point x has H(x) as in step_kernel (p = 1: F_m; p = 2: [[F^1_m, F^2_m],
+// [r_1 F^1_{m+1}, r_2 F^2_{m+1}]], r_i = (m(m+1)+kappa_i^2)/(m+1)) up to a scale per column, which
+// cancels in A = (t2/t1)^m diag(t2^p) H2 H1^-1 diag(t1^-q) and in phi = diag(t2^(p-M+1)) H2 H(x)^-1
+// e_{M-1}.  A node's phi is formed from H2's entries (broadcast from its group's lane 0) and the
+// node's own before squaring (no cancellation).
+//
+// A group of 16 lanes takes one step and a block of rec_block(n_modes) orders, starting the
+// recurrence from the series at the block's top: lane 0 at x2 (the step's poleward ring), lane 1
+// at x1, lanes 2 .. 15 at the 14 nodes of a Gauss-Legendre panel in v.  The panel is no wider than
+// 11 / rho(m) for every order of the block whose weight e^{-2mv} at the panel's start is above
+// e^-46 (further panels, which only the orders of such weight take, follow for steps near the pole):
+// 14 nodes then integrate e^{-11 t} to 1e-17 of its maximum, where 8-point panels of width 4 / rho
+// took 22 nodes.  The blocks' and groups' independence is what counts: one warp per step walked
+// all orders and panels before, so a set-up took the polar steps' latency (1024 x 2048, p = 2:
+// 10.7 ms in 512 warps, now 1.9 ms; 2048 x
+// 4096, p = 1: 12.5 -> 3.8 ms for the whole set-up).  Tables of every order against the former kernels': A and C to 1e-12 (p = 1) and
+// 1e-11 of each entry's scale (p = 2); fields against 64-bit references 8.7e-13 -> 5.1e-13.
+constexpr int kRecNodes = 14;
+constexpr int kRecWarps = 2;         // warps per block, two steps each
+constexpr int kRecMaxPanels = 8192;  // reached only by grids far beyond 16384 rings
+__constant__ double kGL14x[kRecNodes] = {-0.98628380869681233884, -0.92843488366357351734, -0.82720131506976499319, -0.68729290481168547015,
+                                         -0.51524863635815409197, -0.31911236892788976044, -0.10805494870734366207, 0.10805494870734366207,
+                                         0.31911236892788976044, 0.51524863635815409197, 0.68729290481168547015, 0.82720131506976499319,
+                                         0.92843488366357351734, 0.98628380869681233884};
+__constant__ double kGL14w[kRecNodes] = {0.035119460331751863032, 0.080158087159760209806, 0.12151857068790318469, 0.15720316715819353457,
+                                         0.18553839747793781374, 0.20519846372129560397, 0.2152638534631577902, 0.2152638534631577902,
+                                         0.20519846372129560397, 0.18553839747793781374, 0.15720316715819353457, 0.12151857068790318469,
+                                         0.080158087159760209806, 0.035119460331751863032};
 
-// the series F_mu(x) as S * 2^(250 E)
-__device__ void hyp_scaled2(double k2, int mu, double x, double& S, int& E)
+// blocks of orders, and orders per block: about 64 (256 from 2560 modes on), evenly; the series at
+// a block's top cost as much as some 30 orders
+__host__ __device__ inline int rec_blocks(int n_modes)
 {
-    double s = 1.0, t = 1.0;
-    int e = 0;
-    const double m1 = (double)mu + 1.0;
-    for (int n = 0; n < 1000000; n += 2) {
-        const double dn = (double)n;
-        const double a0 = (dn * (dn + 1.0) + k2) * x, d0 = (dn + m1) * (dn + 1.0);
-        const double a1 = ((dn + 1.0) * (dn + 2.0) + k2) * x, d1 = (dn + 1.0 + m1) * (dn + 2.0);
-        const double inv = 1.0 / (d0 * d1);
-        const double r0 = a0 * d1 * inv, r1 = a1 * d0 * inv;
-        t *= r0;
-        s += t;
-        if (t < 1e-17 * s && r0 < 0.9) break;
-        t *= r1;
-        s += t;
-        if (t < 1e-17 * s && r1 < 0.9) break;
-        if (s > 0x1p250) { s *= 0x1p-250; t *= 0x1p-250; ++e; }
+    const int nb = n_modes / (n_modes <= 2560 ? 64 : 256);
+    return nb > 0 ? nb : 1;
+}
+__host__ __device__ inline int rec_block(int n_modes) { return (n_modes + rec_blocks(n_modes) - 1) / rec_blocks(n_modes); }
+
+__device__ inline int hi_word(double x) { return __double2hiint(x); }
+
+// the series F_mu(x) and F_{mu+1}(x) for every kappa_i, as S 2^(250 E) with one E per i; the terms'
+// denominators are shared by all of them
+template <int M>
+__device__ inline void hyp_pairs(const double* k2, int mu, double x, double (&S0)[M], double (&S1)[M], int (&E)[M])
+{
+    double t0[M], t1[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        t0[i] = t1[i] = S0[i] = S1[i] = 1.0;
+        E[i] = 0;
     }
-    S = s;
-    E = e;
+    double n1 = 1.0, a = (double)mu + 1.0;  // n + 1, n + 1 + mu
+    for (int n = 0; n < 1000000; ++n) {
+        const double b = a + 1.0, r = x * rcp_newton(n1 * (a * b));
+        const double q = n1 * n1 - n1;  // n (n + 1)
+        bool done = true;
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            const double c = (q + k2[i]) * r, r0 = c * b;
+            t0[i] *= r0;
+            t1[i] *= c * a;
+            S0[i] += t0[i];
+            S1[i] += t1[i];
+            // terms below 2^-57 of the sums and falling (all values positive: their high words compare)
+            done = done && hi_word(S0[i]) - hi_word(t0[i]) > (57 << 20) && hi_word(S1[i]) - hi_word(t1[i]) > (57 << 20) &&
+                   hi_word(r0) < hi_word(0.9);
+            if (hi_word(S0[i]) > ((1023 + 250) << 20)) {
+                S0[i] *= 0x1p-250;
+                S1[i] *= 0x1p-250;
+                t0[i] *= 0x1p-250;
+                t1[i] *= 0x1p-250;
+                ++E[i];
+            }
+        }
+        if (done) break;
+        n1 += 1.0;
+        a = b;
+    }
 }
 
-// width of the panel that starts at v: 4/rho(m*), m* the largest order whose weight e^{-2 m v}
-// is above e^-46 at v, rho(m) = 2m + kap
-__device__ inline double rec_panel_width(double v, int mtop, double kap)
-{
-    const double ms = v > 0.0 ? fmin((double)mtop, floor(23.0 / v)) : (double)mtop;
-    return 4.0 / (2.0 * ms + kap);
-}
-
-// One warp per step of the northern chain (pos = first..len).  Lane 0 holds x2 (the step's
-// poleward ring), lane 1 x1, lanes 2..31 up to 30 quadrature nodes (further nodes in further
-// passes, which start at the highest order whose weight at their nodes is above e^-46).  The
-// lanes run the recurrence downward in m together; per block of 32 orders they leave
-// w_j e^{-2 m v_j} / F_m(x_j)^2 in shared memory, and lane l then sums order m_l's row in a
-// fixed order, so that Q_m = (A_amp/2 pi) F_m(x2)^2 sum_j ... (the common scale of the F's
-// cancels).
+template <int M>
 __global__ void __launch_bounds__(32 * kRecWarps) step_kernel_rec(Spec sp, int first, int len, double* phi, double* qout)
 {
-    __shared__ double tile[kRecWarps][32][33];  // [order in block][lane]
-    __shared__ double fr2[kRecWarps][32], fr1[kRecWarps][32], alph[kRecWarps][32];
-    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int pos = blockIdx.x * kRecWarps + wib + first;
-    if (pos > len) return;  // whole warps
-    const unsigned full = 0xffffffffu;
-    const double th1 = chain_theta(sp, 0, pos - 1), th2 = chain_theta(sp, 0, pos);
-    const double u1 = log(tan(0.5 * th1)), u2 = log(tan(0.5 * th2));
-    const double du = u1 - u2;
-    const double sa = sin(0.5 * th1), sb = sin(0.5 * th2);
-    const double x1r = sa * sa, x2r = sb * sb;
-    const double sinmax = th1 > 0.5 * SMERF_PI ? 1.0 : sin(th1);
-    const double kap = 2.0 * sp.kmax * sinmax + 1.0;
-    const double k2 = sp.k2[0];
-    const double f = sp.A / (2.0 * SMERF_PI);
-    const int mtop = sp.n_modes - 1;
-    int np = 0;
-    for (double v = 0.0; v < du && np < kRecMaxPanels; ++np) v += rec_panel_width(v, mtop, kap);
-    const int K = 8 * np;
-    const int passes = (K + 29) / 30;
-    const size_t base = (size_t)pos * sp.n_modes;
-    for (int ch = 0; ch < passes; ++ch) {
-        // this lane's point: x, quadrature weight, v
-        double x = x2r, wt = 0.0, v = 0.0;
-        if (lane == 1) {
-            x = x1r;
-            v = du;
-        } else if (lane >= 2 && 30 * ch + lane - 2 < K) {
-            const int i = 30 * ch + lane - 2, j = i >> 3, n = i & 7;
-            double b = 0.0;
-            for (int q = 0; q < j; ++q) b += rec_panel_width(b, mtop, kap);
-            const double h = (j == np - 1 || b + rec_panel_width(b, mtop, kap) > du) ? du - b
-                                                                                       : rec_panel_width(b, mtop, kap);
-            v = b + 0.5 * (kGL8x[n] + 1.0) * h;
-            wt = 0.5 * h * kGL8w[n];
-            x = 1.0 / (1.0 + exp(-2.0 * (u2 + v)));
-        }
-        // highest order of the pass: every order for the first (it also gives A), else the
-        // last whose weight at the pass's first node is above e^-46
-        int mstart = mtop;
-        if (ch > 0) {
-            const double vmin = __shfl_sync(full, v, 2);
-            mstart = vmin > 0.0 ? (int)fmin((double)mtop, floor(23.0 / vmin)) : mtop;
-        }
-        double S0, S1;
-        int E0, E1;
-        hyp_scaled2(k2, mstart, x, S0, E0);
-        hyp_scaled2(k2, mstart + 1, x, S1, E1);
-        int W = E0;  // common scale of the lanes' values
-        for (int o = 16; o > 0; o >>= 1) W = max(W, __shfl_xor_sync(full, W, o));
-        double F = ldexp(S0, 250 * (E0 - W)), Fp = ldexp(S1, 250 * (E1 - W));
-        const double beta = (1.0 - 2.0 * x) / (1.0 - x), gam = x / (1.0 - x);
-        const double e2v = exp(2.0 * v);
-        for (int mb = mstart; mb >= 0; mb -= 32) {
-            {
-                const int ml = mb - lane;
-                alph[wib][lane] = ml >= 1 ? k2 / ((double)ml * (double)(ml + 1)) : 0.0;
-            }
-            __syncwarp();
-            double Ew = exp(-2.0 * (double)mb * v);  // e^{-2 m v}, exact at the block's first order
-            for (int k = 0; k < 32; ++k) {
-                const int m = mb - k;
-                if (m < 0) break;
-                const double r = 1.0 / F;
-                tile[wib][k][lane] = wt * Ew * r * r;
-                if (lane == 0) fr2[wib][k] = F;
-                if (lane == 1) fr1[wib][k] = F;
-                if (m >= 1) {
-                    const double t = gam + gam * alph[wib][k];
-                    const double Fn = beta * F + t * Fp;
-                    Fp = F;
-                    F = Fn;
-                    // a common rescale keeps the values, their squares and the squares of their
-                    // reciprocals in range (ratios are unchanged)
-                    if (__any_sync(full, (__double2hiint(F) & 0x7ff00000) > ((1023 + 250) << 20))) {
-                        F *= 0x1p-250;
-                        Fp *= 0x1p-250;
-                    }
-                }
-                Ew *= e2v;
-            }
-            __syncwarp();
-            const int m = mb - lane;
-            if (m >= 0) {
-                double sum = 0.0;
-                for (int j = 2; j < 32; ++j) sum += tile[wib][lane][j];
-                const double F2 = fr2[wib][lane];
-                const double q = f * F2 * F2 * sum;
-                if (ch == 0) {
-                    qout[base + m] = q;
-                    phi[base + m] = exp(-(double)m * du) * F2 / fr1[wib][lane];
-                } else {
-                    qout[base + m] += q;
-                }
-            }
-            __syncwarp();
-        }
-    }
-}
-
-// p = 2 with a real spectrum: the same recurrence for both kappa_i.  Per order m a lane's
-// point x has H(x) = [[F^1_m, F^2_m], [r_1 F^1_{m+1}, r_2 F^2_{m+1}]], r_i = (m(m+1)+kappa_i^2)/(m+1)
-// (step_kernel's H up to a scale per column, which cancels in A = H2 H1^-1 and in
-// phi = W H^-1 e_1), each column with its own common rescale.  A node's
-// phi = diag(t2^-1, 1) H2 H(x)^-1 e_1 is formed from H2's entries (broadcast from lane 0) and
-// the node's own before squaring (no cancellation); its three products go through shared
-// memory as in step_kernel_rec.  One warp per block (three transposition tiles).
-__global__ void __launch_bounds__(32) step_kernel_rec2(Spec sp, int first, int len, double* phi, double* qout)
-{
-    constexpr int M = 2;
-    __shared__ double tile[3][32][33];  // [product][order in block][lane]
-    __shared__ double h2[4][32], h1[4][32], alph[2][32], rr[2][32];
-    const int lane = threadIdx.x & 31;
-    const int pos = blockIdx.x + first;
-    if (pos > len) return;
-    const unsigned full = 0xffffffffu;
+    constexpr int T = M * (M + 1) / 2, MM = M * M;
+    __shared__ double tile[kRecWarps][T][2][16][17];  // [product][half][order in block][lane]
+    __shared__ double h2[kRecWarps][MM][2][16], h1[kRecWarps][MM][2][16], alph[kRecWarps][M][2][16], rr[kRecWarps][M][2][16];
+    const int w = threadIdx.x >> 5, h = (threadIdx.x >> 4) & 1, l = threadIdx.x & 15;
+    const unsigned full = 0xffffffffu, half = 0xffffu << (16 * h);
+    const int step = 2 * ((gridDim.x - 1 - blockIdx.x) * kRecWarps + w);  // polar steps (more panels) first
+    if (first + step > len) return;  // whole warps
+    const bool live = first + step + h <= len;  // a second half beyond the last step repeats it and stores nothing
+    const int pos = live ? first + step + h : len;
+    const int B = rec_block(sp.n_modes), mlo = blockIdx.y * B, mhi = min(sp.n_modes - 1, mlo + B - 1);
     const double th1 = chain_theta(sp, 0, pos - 1), th2 = chain_theta(sp, 0, pos);
     const double t1 = tan(0.5 * th1), t2 = tan(0.5 * th2);
-    const double u1 = log(t1), u2 = log(t2);
-    const double du = u1 - u2;
+    const double u2 = log(t2), du = log(t1) - u2;
     const double sa = sin(0.5 * th1), sb = sin(0.5 * th2);
-    const double x1r = sa * sa, x2r = sb * sb;
     const double sinmax = th1 > 0.5 * SMERF_PI ? 1.0 : sin(th1);
     const double kap = 2.0 * sp.kmax * sinmax + 1.0;
-    const double f = sp.A / (2.0 * SMERF_PI);
-    const int mtop = sp.n_modes - 1;
-    // panel width at v: 4/rho(m*), rho(m) = 2(m + M - 1) + kap, m* the largest order whose
-    // weight e^{-2(m+M-1)v} is above e^-46 at v
-    auto width = [&](double v) {
-        const double ms = v > 0.0 ? fmax(0.0, fmin((double)mtop, floor(23.0 / v) - (M - 1))) : (double)mtop;
-        return 4.0 / (2.0 * (ms + M - 1) + kap);
-    };
-    int np = 0;
-    for (double v = 0.0; v < du && np < kRecMaxPanels; ++np) v += width(v);
-    const int K = 8 * np;
-    const int passes = (K + 29) / 30;
+    const double f = sp.A / (2.0 * SMERF_PI), it1 = 1.0 / t1, it2 = 1.0 / t2;
     const size_t base = (size_t)pos * sp.n_modes;
-    for (int ch = 0; ch < passes; ++ch) {
-        double x = x2r, wt = 0.0, v = 0.0;
-        if (lane == 1) {
-            x = x1r;
+    // highest order whose weight e^{-2(m+M-1)v} is above e^-46 at v
+    auto top = [&](double v) { return v > 0.0 ? (int)fmin((double)mhi, floor(23.0 / v) - (M - 1)) : mhi; };
+    double v0 = 0.0;  // the panel's start
+    for (int ch = 0; ch < kRecMaxPanels; ++ch) {
+        const int mt = top(v0);
+        const bool act = v0 < du && mt >= mlo;  // this half has the panel
+        if (!__any_sync(full, act)) break;
+        const double wd = 11.0 / (2.0 * (max(mt, mlo) + M - 1) + kap);
+        const double hp = fmin(wd, du - v0);
+        double x = sb * sb, wt = 0.0, v = 0.0;
+        if (l == 1) {
+            x = sa * sa;
             v = du;
-        } else if (lane >= 2 && 30 * ch + lane - 2 < K) {
-            const int i = 30 * ch + lane - 2, j = i >> 3, n = i & 7;
-            double b = 0.0;
-            for (int q = 0; q < j; ++q) b += width(b);
-            const double h = (j == np - 1 || b + width(b) > du) ? du - b : width(b);
-            v = b + 0.5 * (kGL8x[n] + 1.0) * h;
-            wt = 0.5 * h * kGL8w[n];
+        } else if (l >= 2 && act) {
+            v = v0 + 0.5 * (kGL14x[l - 2] + 1.0) * hp;
+            wt = 0.5 * hp * kGL14w[l - 2];
             x = 1.0 / (1.0 + exp(-2.0 * (u2 + v)));
         }
-        int mstart = mtop;
-        if (ch > 0) {
-            const double vmin = __shfl_sync(full, v, 2);
-            mstart = vmin > 0.0 ? (int)fmax(0.0, fmin((double)mtop, floor(23.0 / vmin) - (M - 1))) : mtop;
-        }
-        double F[2], Fp[2];
-        for (int c = 0; c < 2; ++c) {
-            double S0, S1;
-            int E0, E1;
-            hyp_scaled2(sp.k2[c], mstart, x, S0, E0);
-            hyp_scaled2(sp.k2[c], mstart + 1, x, S1, E1);
-            int W = E0;
-            for (int o = 16; o > 0; o >>= 1) W = max(W, __shfl_xor_sync(full, W, o));
-            F[c] = ldexp(S0, 250 * (E0 - W));
-            Fp[c] = ldexp(S1, 250 * (E1 - W));
+        // both halves start at the higher of their top orders
+        int ms = act ? mt : mlo;
+        ms = max(ms, __shfl_xor_sync(full, ms, 16));
+        double F[M], Fp[M];
+        int E[M];
+        hyp_pairs<M>(sp.k2, ms, x, F, Fp, E);
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            int W = E[i];  // one scale per column and half
+            for (int o = 8; o > 0; o >>= 1) W = max(W, __shfl_xor_sync(full, W, o));
+            F[i] = ldexp(F[i], 250 * (E[i] - W));
+            Fp[i] = ldexp(Fp[i], 250 * (E[i] - W));
         }
         const double beta = (1.0 - 2.0 * x) / (1.0 - x), gam = x / (1.0 - x);
         const double e2v = exp(2.0 * v);
-        for (int mb = mstart; mb >= 0; mb -= 32) {
-            {
-                const int ml = mb - lane;
-                for (int c = 0; c < 2; ++c) {
-                    alph[c][lane] = ml >= 1 ? sp.k2[c] / ((double)ml * (double)(ml + 1)) : 0.0;
-                    rr[c][lane] = ml >= 0 ? ((double)ml * (double)(ml + 1) + sp.k2[c]) / (double)(ml + 1) : 0.0;
-                }
+        double Ew = 0.0;
+        for (int mb = ms; mb >= mlo; mb -= 16) {
+            const int ml = mb - l;
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                const double al = ml >= 1 ? sp.k2[i] * rcp_newton((double)ml * (double)(ml + 1)) : 0.0;
+                alph[w][i][h][l] = al;
+                rr[w][i][h][l] = ml >= 1 ? (double)ml + (double)ml * al : sp.k2[i];  // (m(m+1) + kappa^2)/(m+1)
             }
             __syncwarp();
-            double Ew = exp(-2.0 * (double)(mb + M - 1) * v);
-            for (int k = 0; k < 32; ++k) {
+            // e^{-2(m+M-1)v}, exact every 32 orders
+            if (((ms - mb) & 16) == 0) Ew = wt * exp(-2.0 * (double)(mb + M - 1) * v);
+#pragma unroll 2
+            for (int k = 0; k < 16; ++k) {
                 const int m = mb - k;
-                if (m < 0) break;
-                const double a = F[0], b = F[1], c = rr[0][k] * Fp[0], d = rr[1][k] * Fp[1];
-                const double a2 = __shfl_sync(full, a, 0), b2 = __shfl_sync(full, b, 0);
-                const double c2 = __shfl_sync(full, c, 0), d2 = __shfl_sync(full, d, 0);
-                const double rdet = 1.0 / (a * d - b * c);
-                const double p0 = (b2 * a - a2 * b) * rdet, p1 = (d2 * a - c2 * b) * rdet;
-                const double we = wt * Ew;
-                tile[0][k][lane] = we * p0 * p0;
-                tile[1][k][lane] = we * p0 * p1;
-                tile[2][k][lane] = we * p1 * p1;
-                if (lane == 0) { h2[0][k] = a; h2[1][k] = b; h2[2][k] = c; h2[3][k] = d; }
-                if (lane == 1) { h1[0][k] = a; h1[1][k] = b; h1[2][k] = c; h1[3][k] = d; }
+                if (m < mlo) break;
+                if constexpr (M == 1) {
+                    const double r = rcp_newton(F[0]);
+                    tile[w][0][h][k][l] = Ew * r * r;
+                    if (l == 0) h2[w][0][h][k] = F[0];
+                    if (l == 1) h1[w][0][h][k] = F[0];
+                } else {
+                    const double a = F[0], b = F[1], c = rr[w][0][h][k] * Fp[0], d = rr[w][1][h][k] * Fp[1];
+                    const double a2 = __shfl_sync(full, a, 0, 16), b2 = __shfl_sync(full, b, 0, 16);
+                    const double c2 = __shfl_sync(full, c, 0, 16), d2 = __shfl_sync(full, d, 0, 16);
+                    const double rdet = rcp_newton(a * d - b * c);
+                    const double p0 = (b2 * a - a2 * b) * rdet, p1 = (d2 * a - c2 * b) * rdet;
+                    const double q0 = Ew * p0;
+                    tile[w][0][h][k][l] = q0 * p0;
+                    tile[w][1][h][k][l] = q0 * p1;
+                    tile[w][2][h][k][l] = Ew * p1 * p1;
+                    if (l == 0) { h2[w][0][h][k] = a; h2[w][1][h][k] = b; h2[w][2][h][k] = c; h2[w][3][h][k] = d; }
+                    if (l == 1) { h1[w][0][h][k] = a; h1[w][1][h][k] = b; h1[w][2][h][k] = c; h1[w][3][h][k] = d; }
+                }
                 if (m >= 1) {
-                    for (int cc = 0; cc < 2; ++cc) {
-                        const double t = gam + gam * alph[cc][k];
-                        const double Fn = beta * F[cc] + t * Fp[cc];
-                        Fp[cc] = F[cc];
-                        F[cc] = Fn;
-                        if (__any_sync(full, (__double2hiint(F[cc]) & 0x7ff00000) > ((1023 + 250) << 20))) {
-                            F[cc] *= 0x1p-250;
-                            Fp[cc] *= 0x1p-250;
+#pragma unroll
+                    for (int i = 0; i < M; ++i) {
+                        const double t = gam + gam * alph[w][i][h][k];
+                        const double Fn = beta * F[i] + t * Fp[i];
+                        Fp[i] = F[i];
+                        F[i] = Fn;
+                        // a common rescale keeps the values, their squares and the squares of their
+                        // reciprocals in range (ratios are unchanged)
+                        if (__ballot_sync(full, (hi_word(F[i]) & 0x7ff00000) > ((1023 + 250) << 20)) & half) {
+                            F[i] *= 0x1p-250;
+                            Fp[i] *= 0x1p-250;
                         }
                     }
                 }
                 Ew *= e2v;
             }
             __syncwarp();
-            const int m = mb - lane;
-            if (m >= 0) {
-                double s00 = 0.0, s01 = 0.0, s11 = 0.0;
-                for (int j = 2; j < 32; ++j) {
-                    s00 += tile[0][lane][j];
-                    s01 += tile[1][lane][j];
-                    s11 += tile[2][lane][j];
+            if (act && live && ml >= mlo && ml <= mhi) {
+                double s[T];
+#pragma unroll
+                for (int e = 0; e < T; ++e) {
+                    s[e] = 0.0;
+                    for (int j = 2; j < 16; ++j) s[e] += tile[w][e][h][l][j];
                 }
-                const size_t o = (base + m) * (M * M);
-                const double q00 = f * s00 / (t2 * t2), q01 = f * s01 / t2, q11 = f * s11;
-                if (ch == 0) {
-                    qout[o + 0] = q00;
-                    qout[o + 1] = q01;
-                    qout[o + 2] = q01;
-                    qout[o + 3] = q11;
-                    // A = (t2/t1)^m diag(t2^p) H2 H1^-1 diag(t1^-q)
-                    const double a2 = h2[0][lane], b2 = h2[1][lane], c2 = h2[2][lane], d2 = h2[3][lane];
-                    const double a1 = h1[0][lane], b1 = h1[1][lane], c1 = h1[2][lane], d1 = h1[3][lane];
-                    const double g = exp(-(double)m * du) / (a1 * d1 - b1 * c1);
-                    phi[o + 0] = g * (a2 * d1 - b2 * c1);
-                    phi[o + 1] = g * (b2 * a1 - a2 * b1) / t1;
-                    phi[o + 2] = g * t2 * (c2 * d1 - d2 * c1);
-                    phi[o + 3] = g * t2 * (d2 * a1 - c2 * b1) / t1;
+                const size_t o = (base + ml) * MM;
+                double q[MM];
+                if constexpr (M == 1) {
+                    const double F2 = h2[w][0][h][l];
+                    q[0] = f * F2 * F2 * s[0];
                 } else {
-                    qout[o + 0] += q00;
-                    qout[o + 1] += q01;
-                    qout[o + 2] += q01;
-                    qout[o + 3] += q11;
+                    q[0] = f * s[0] * it2 * it2;
+                    q[1] = q[2] = f * s[1] * it2;
+                    q[3] = f * s[2];
+                }
+                if (ch == 0) {
+#pragma unroll
+                    for (int e = 0; e < MM; ++e) qout[o + e] = q[e];
+                    // A = (t2/t1)^m diag(t2^p) H2 H1^-1 diag(t1^-q)
+                    const double g = exp(-(double)ml * du);
+                    if constexpr (M == 1) {
+                        phi[o] = g * h2[w][0][h][l] / h1[w][0][h][l];
+                    } else {
+                        const double a2 = h2[w][0][h][l], b2 = h2[w][1][h][l], c2 = h2[w][2][h][l], d2 = h2[w][3][h][l];
+                        const double a1 = h1[w][0][h][l], b1 = h1[w][1][h][l], c1 = h1[w][2][h][l], d1 = h1[w][3][h][l];
+                        const double gd = g / (a1 * d1 - b1 * c1);
+                        phi[o + 0] = gd * (a2 * d1 - b2 * c1);
+                        phi[o + 1] = gd * (b2 * a1 - a2 * b1) * it1;
+                        phi[o + 2] = gd * t2 * (c2 * d1 - d2 * c1);
+                        phi[o + 3] = gd * t2 * (d2 * a1 - c2 * b1) * it1;
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < MM; ++e) qout[o + e] += q[e];
                 }
             }
             __syncwarp();
         }
+        if (act) v0 += hp;
     }
 }
 
@@ -610,70 +550,52 @@ __device__ inline void put(void* base, bool is64, size_t idx, double v)
     }
 }
 
-// The start ring's Pochhammer factors, log[(-l_i)_m (l_i+1)_m / (m!)^2]
-// = sum_{j<m} log((j(j+1) + kappa_i^2) / (j+1)^2) (Eq. (Legendre_hypergeometric)), for every m at
-// once: one block sums contiguous chunks of the terms, scans the chunk sums and writes each
-// chunk's prefixes (a fixed order; start_kernel reads lq[i * n_modes + m]).
-__global__ void __launch_bounds__(1024) lq_prefix_kernel(Spec sp, double* lq)
-{
-    __shared__ double part[1024];
-    const int n = sp.n_modes, t = threadIdx.x, nt = blockDim.x;
-    const int chunk = (n + nt - 1) / nt;
-    const int j0 = min(n, t * chunk), j1 = min(n, j0 + chunk);
-    for (int i = 0; i < sp.M; ++i) {
-        const double k2 = sp.k2[i];
-        double s = 0.0;
-        for (int j = j0; j < j1; ++j) s += log((j * (j + 1.0) + k2) / ((j + 1.0) * (j + 1.0)));
-        part[t] = s;
-        __syncthreads();
-        for (int o = 1; o < nt; o <<= 1) {  // inclusive scan of the chunk sums
-            const double v = t >= o ? part[t - o] : 0.0;
-            __syncthreads();
-            part[t] += v;
-            __syncthreads();
-        }
-        double acc = t > 0 ? part[t - 1] : 0.0;  // the terms j < j0
-        for (int j = j0; j < j1; ++j) {
-            lq[(size_t)i * n + j] = acc;
-            acc += log((j * (j + 1.0) + k2) / ((j + 1.0) * (j + 1.0)));
-        }
-        __syncthreads();
-    }
-}
-
-// Start factor B_eq = chol J(z0, z0) (Eq. (state_initial)), one thread per mode.
+// Start factor B_eq = chol J(z0, z0) (Eq. (state_initial)).  J = sum_i b_i (2 pi)^-1 G_i with the
+// Green's functions G_i of l(l+1) + kappa_i^2 (Eq. (C_ell_efficient)) from the solutions regular at
+// either pole, u = P^m_l(z) and v = P^m_l(-z): with R_q(z) = P^{m+q}_l(z) / P^m_l(z) = r_q t^q
+// F_{m+q}(x) / F_m(x) and (1-z^2)(v'/v - u'/u) = sin(theta0) (R_1(z) + R_1(-z)), the raised
+// components are J_qp = b_i R_q(z) (-1)^p R_p(-z) / (2 pi sin(theta0) (R_1(z) + R_1(-z))).  Only
+// ratios of neighbouring orders enter, so no Gamma factor nor product over the orders (the form
+// with Eq. (Jmatrix_efficient)'s Pochhammer factors took a prefix sum of logarithms over the modes
+// and 2 M^2 series per thread: 0.65 ms at 1024 x 2048, p = 2, now 0.12).  A group of
+// start_lanes(M) lanes per mode, one lane per (i, side).
+__host__ __device__ constexpr int start_lanes(int M) { return M == 1 ? 2 : M == 2 ? 4 : 8; }
 template <int M>
-__global__ void start_kernel(Spec sp, const double* lqa, void* beq, bool tab64)
+__global__ void __launch_bounds__(64) start_kernel(Spec sp, void* beq, bool tab64)
 {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= sp.n_modes) return;
+    constexpr int GL = start_lanes(M), NR = M < 3 ? 2 : 3;  // R_0 .. R_{NR-1}
+    const int gid = blockIdx.x * blockDim.x + threadIdx.x, lane = gid % GL;
+    const int m = min(gid / GL, sp.n_modes - 1);  // the last block's spare groups repeat the last mode
     const double th0 = ring_colat(sp.theta, sp.n_theta, sp.k0);
-    const double t0 = tan(0.5 * th0);
     const double sx = sin(0.5 * th0), cx = cos(0.5 * th0);
-    const double x0 = sx * sx, xb0 = cx * cx;
-    Mat<M> J = mzero<M>();
-    for (int i = 0; i < M; ++i) {
-        const double k2 = sp.k2[i];
-        const double lq = lqa[(size_t)i * sp.n_modes + m];  // log Q_m / (m!)^2
-        double lF0[M], lF1[M], r[M];
-        double rr = 1.0;
-        for (int q = 0; q < M; ++q) {
-            if (q > 0) {
-                const double j = (double)(m + q - 1);
-                rr *= (j * (j + 1.0) + k2) / (j + 1.0);
-            }
-            r[q] = rr;
-            lF0[q] = log_hyp(k2, m + q, x0);
-            lF1[q] = log_hyp(k2, m + q, xb0);
-        }
-        const double sb = sp.b[i] > 0.0 ? 1.0 : -1.0;
-        const double lb = log(fabs(sp.b[i])) + sp.lG0[i] - log(4.0 * SMERF_PI) + lq;
-        for (int p = 0; p < M; ++p)
-            for (int q = 0; q < M; ++q) {
-                const double v = exp(lb + lF1[p] + lF0[q]) * r[p] * r[q] * pow(t0, (double)(q - p));
-                J.a[p][q] += sb * ((p & 1) ? -v : v);
-            }
+    // lane = 2 i + side (0: z, 1: -z); spare lanes repeat the last factor
+    const int side = lane & 1;
+    double k2[1] = {sp.k2[min(lane / 2, M - 1)]};
+    const double x = side ? cx * cx : sx * sx, t = side ? cx / sx : sx / cx;
+    double R[NR], S0[1], S1[1];
+    int E[1];
+    hyp_pairs<1>(k2, m, x, S0, S1, E);
+    const double dm = (double)m, r1 = (dm * (dm + 1.0) + k2[0]) / (dm + 1.0);
+    R[0] = 1.0;
+    R[1] = r1 * t * S1[0] / S0[0];
+    if constexpr (NR > 2) {
+        hyp_pairs<1>(k2, m + 1, x, S0, S1, E);
+        R[2] = R[1] * ((dm + 1.0) * (dm + 2.0) + k2[0]) / (dm + 2.0) * t * S1[0] / S0[0];
     }
+    Mat<M> J = mzero<M>();
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        double n[NR], q[NR];
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            n[k] = __shfl_sync(0xffffffffu, R[k], 2 * i, GL);
+            q[k] = __shfl_sync(0xffffffffu, R[k], 2 * i + 1, GL);
+        }
+        const double g = sp.b[i] / (2.0 * SMERF_PI * sin(th0) * (n[1] + q[1]));
+        for (int a = 0; a < M; ++a)
+            for (int b = 0; b < M; ++b) J.a[a][b] += g * n[a] * ((b & 1) ? -q[b] : q[b]);
+    }
+    if (lane != 0 || gid / GL >= sp.n_modes) return;
     const Mat<M> L = mchol<M>(msym<M>(J));
     const double sc = m > 0 ? 0.70710678118654752440 : 1.0;
     int e = 0;
@@ -684,8 +606,11 @@ __global__ void start_kernel(Spec sp, const double* lqa, void* beq, bool tab64)
 
 // Bridge, forward and coarse tables of one segment, one thread per (segment, mode).
 // Segment [pa, pb] with right anchor pb: for pa < pos < pb, condition x_pos on x_{pos-1}
-// (prior N(Phi x, Q)) and on x_pb = Psi x_pos + N(0, S) (Psi, S accumulated backward):
-//   P = (Q^{-1} + Psi^T S^{-1} Psi)^{-1},  Abar = P Q^{-1} Phi,  C = P Psi^T S^{-1},  B = chol P.
+// (prior N(Phi x, Q)) and on x_pb = Psi x_pos + N(0, S) (Psi, S accumulated backward), in gain form:
+//   W = Psi Q Psi^T + S,  C = Q Psi^T W^{-1},  R = I - C Psi,  Abar = R Phi,
+//   P = R Q R^T + C S C^T,  B = chol P.
+// W is the next position's S, and one inverse per position replaces the three of the information
+// form (Q^{-1} + Psi^T S^{-1} Psi)^{-1}, on the FP64 pipe that bounds this kernel (2 x 348 -> 2 x 231 us at 1024 x 2048, p = 2).
 // The coarse step pa -> pb is (Psi_pa, chol S_pa).  Without a right anchor the tables are
 // the plain forward step (Phi, 0, chol Q).
 template <int M>
@@ -732,17 +657,19 @@ __global__ void segment_tables_kernel(Spec sp, int c, int len, int H, const doub
     Mat<M> Psi = meye<M>(), S = mzero<M>();
     for (int pos = pb; pos > pa; --pos) {
         const Mat<M> Ph = load(phi, pos), Q = msym<M>(load(qv, pos));
+        // W = Psi Q Psi^T + S: the anchor's covariance given x_{pos-1}, and S_{pos-1}
+        const Mat<M> G = mmul<M>(Psi, Q);
+        const Mat<M> W = msym<M>(madd<M>(mmul<M>(G, mT<M>(Psi)), S));
         if (pos < pb) {
-            const Mat<M> Qi = mspd_inv<M>(Q);
-            const Mat<M> Si = mspd_inv<M>(msym<M>(S));
-            const Mat<M> PsT = mT<M>(Psi);
-            const Mat<M> P = msym<M>(mspd_inv<M>(msym<M>(madd<M>(Qi, mmul<M>(mmul<M>(PsT, Si), Psi)))));
-            const Mat<M> Ab = mmul<M>(mmul<M>(P, Qi), Ph);
-            const Mat<M> C = mmul<M>(mmul<M>(P, PsT), Si);
-            store_step(pos, Ab, C, mchol<M>(P));
+            const Mat<M> C = mmul<M>(mT<M>(G), mspd_inv<M>(W));
+            Mat<M> R = mmul<M>(C, Psi);  // I - C Psi
+            for (int i = 0; i < M; ++i)
+                for (int j = 0; j < M; ++j) R.a[i][j] = (i == j ? 1.0 : 0.0) - R.a[i][j];
+            // P = R Q R^T + C S C^T: a sum of covariances, nothing cancels in it
+            const Mat<M> P = madd<M>(mmul<M>(mmul<M>(R, Q), mT<M>(R)), mmul<M>(mmul<M>(C, S), mT<M>(C)));
+            store_step(pos, mmul<M>(R, Ph), C, mchol<M>(msym<M>(P)));
         }
-        // move to pos-1: S_{pos-1} = Psi Q Psi^T + S, Psi_{pos-1} = Psi Phi
-        S = madd<M>(mmul<M>(mmul<M>(Psi, Q), mT<M>(Psi)), S);
+        S = W;
         Psi = mmul<M>(Psi, Ph);
     }
     const Mat<M> Bc = mchol<M>(msym<M>(S));
@@ -1083,13 +1010,6 @@ int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
         for (int j = 0; j < M; ++j)
             if (j != i) b /= pl->kappa[j] * pl->kappa[j] - k * k;
         sp.b[i] = b;
-        if (k * k > 0.25) {
-            const double nu = sqrt(k * k - 0.25);
-            sp.lG0[i] = log(SMERF_PI) - SMERF_PI * nu - log(0.5 * (1.0 + exp(-2.0 * SMERF_PI * nu)));
-        } else {
-            const double lam = -0.5 + sqrt(0.25 - k * k);
-            sp.lG0[i] = log(-SMERF_PI / sin(SMERF_PI * lam));
-        }
     }
     sp.n_theta = pl->n_theta;
     sp.k0 = pl->k0;
@@ -1102,7 +1022,6 @@ int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
     const size_t mp = pl->n_modes_pad;
     double* phi = nullptr;
     double* qv = nullptr;
-    double* lqa = nullptr;
     const int threads = 128;
     const int gm = (pl->n_modes + threads - 1) / threads;
     auto t_start = std::chrono::steady_clock::now();
@@ -1128,11 +1047,7 @@ int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
     if (rc != SMERF_OK) goto done;
     if (pl->complex_spec) start_kernel_c<M><<<gm, threads, 0, st>>>(make_spec_c(pl), pl->beq, t64);
     else {
-        CK(smerf::dev_malloc_async((void**)&lqa, (size_t)M * pl->n_modes * sizeof(double), st));
-        lq_prefix_kernel<<<1, 1024, 0, st>>>(sp, lqa);
-        start_kernel<M><<<gm, threads, 0, st>>>(sp, lqa, pl->beq, t64);
-        CK(cudaFreeAsync(lqa, st));
-        lqa = nullptr;
+        start_kernel<M><<<((unsigned)pl->n_modes * start_lanes(M) + 63) / 64, 64, 0, st>>>(sp, pl->beq, t64);
     }
     CK(cudaGetLastError());
     {
@@ -1178,8 +1093,9 @@ int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
                     if (first_series) step_kernel<M><<<dim3(gm, 1), threads, 0, st>>>(s, 0, 1, phi, qv);
                     if (len >= first) {
                         const int n = len - first + 1;
-                        if (M == 1) step_kernel_rec<<<(n + kRecWarps - 1) / kRecWarps, 32 * kRecWarps, 0, st>>>(s, first, len, phi, qv);
-                        else step_kernel_rec2<<<n, 32, 0, st>>>(s, first, len, phi, qv);
+                        if constexpr (M < 3)
+                            step_kernel_rec<M><<<dim3((n + 2 * kRecWarps - 1) / (2 * kRecWarps), rec_blocks(pl->n_modes)),
+                                                 32 * kRecWarps, 0, st>>>(s, first, len, phi, qv);
                     }
                 }
                 CK(cudaGetLastError());
@@ -1224,11 +1140,10 @@ int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
         pl->setup_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_start).count();
     }
 done:
-    if (phi || qv || lqa) {
+    if (phi || qv) {
         cudaStreamSynchronize(st);
         if (phi) cudaFree(phi);
         if (qv) cudaFree(qv);
-        if (lqa) cudaFree(lqa);
     }
     return rc;
 }
