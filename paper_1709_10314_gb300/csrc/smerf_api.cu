@@ -30,15 +30,8 @@ namespace {
 void free_plan_memory(smerf_plan* pl)
 {
     if (!pl) return;
-    cudaFree(pl->beq);
-    for (int c = 0; c < 2; ++c) {
-        cudaFree(pl->steps[c]);
-        cudaFree(pl->coarse[c]);
-    }
-    cudaFree(pl->tw);
-    cudaFree(pl->pre);
-    cudaFree(pl->tw2);
-    cudaFree(pl->tw3);
+    cudaFree(pl->shared);
+    for (int c = 0; c < 2; ++c) cudaFree(pl->steps[c]);
     cudaFree(pl->segs_dev);
     free(pl->segs_host);
     cudaFree(pl->rings_n_dev);
@@ -252,14 +245,15 @@ cudaMemPool_t scratch_pool(int dev, bool create)
 
 // stream-ordered scratch from the device's pool; under stream capture (a graph records the
 // allocation as its own node) and if the pool cannot be made, the stream's default pool
-cudaError_t scratch_alloc(void** p, size_t bytes, int dev, cudaStream_t st)
+}  // namespace
+
+cudaError_t smerf_scratch_alloc(void** p, size_t bytes, int dev, cudaStream_t st)
 {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return cudaGetLastError();
     cudaMemPool_t pool = cs == cudaStreamCaptureStatusNone ? scratch_pool(dev, true) : nullptr;
     return pool ? smerf::dev_malloc_pool(p, bytes, pool, st) : smerf::dev_malloc_async(p, bytes, st);
 }
-}  // namespace
 
 // allocation-failure injection (smerf_debug_fail_alloc): -1 = off, k >= 0 = the allocation
 // after k more succeeds fails
@@ -592,7 +586,7 @@ int smerf_sample_timed(const smerf_plan* plan, uint64_t seed, int n_samples, voi
     void* scratch = nullptr;
     const size_t sb = (smerf_scratch_bytes(plan, n_samples) + 255) / 256 * 256;
     const size_t tb = smerf_stage_bytes(plan, n_samples);
-    cudaError_t e = scratch_alloc(&scratch, sb + tb, dev, st);
+    cudaError_t e = smerf_scratch_alloc(&scratch, sb + tb, dev, st);
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? SMERF_ENOMEM : SMERF_ECUDA;
     const int rc = smerf_launch_sample_staged(plan, seed, n_samples, out, scratch,
                                               tb ? (void*)((unsigned char*)scratch + sb) : nullptr, st,
@@ -646,7 +640,7 @@ int smerf_sample_host(const smerf_plan* plan, uint64_t seed, int n_samples, void
     cudaGetLastError();  // an unregistered pointer is not an error here
     const size_t bytes = (size_t)n_samples * plan_points(plan) * (plan->recur64 ? 8 : 4);
     void* dout = nullptr;
-    cudaError_t e = scratch_alloc(&dout, bytes, plan->dev, st);
+    cudaError_t e = smerf_scratch_alloc(&dout, bytes, plan->dev, st);
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? SMERF_ENOMEM : SMERF_ECUDA;
     int rc = smerf_sample(plan, seed, n_samples, dout, stream);
     if (rc == SMERF_OK && cudaMemcpyAsync(host_out, dout, bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess)

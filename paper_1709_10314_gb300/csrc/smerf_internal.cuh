@@ -57,7 +57,8 @@ struct smerf_plan {
     int n_segments;
     smerf::Segment* segs_host;
     smerf::Segment* segs_dev;
-    // tables (TabT = double if tab64 else float)
+    // tables (TabT = double if tab64 else float); beq, coarse and the FFT tables lie in `shared`
+    void* shared;
     void* beq;             // [tri][n_modes_pad]
     void* steps[2];        // [len+1][n_modes_pad][step_row]
     void* coarse[2];       // [n_anchors+1][Ec][n_modes_pad] (row 0 unused)
@@ -342,6 +343,9 @@ struct StageSmall {
 SMERF_DECLARE_STAGED(1)
 SMERF_DECLARE_STAGED(2)
 SMERF_DECLARE_STAGED(3)
+
+// stream-ordered memory from the library's scratch pool (smerf_api.cu)
+cudaError_t smerf_scratch_alloc(void** p, size_t bytes, int dev, cudaStream_t st);
 
 // dynamic shared-memory attribute bookkeeping (smerf_api.cu)
 int smerf_smem_attr_done(const void* kern, int dev, size_t smem, bool record);

@@ -682,57 +682,43 @@ __global__ void segment_tables_kernel(Spec sp, int c, int len, int H, const doub
         for (int q = 0; q <= p; ++q, ++e) put<double>(coarse, tab64, base + (size_t)e * mp, Bc.a[p][q] * sc * colsign(q));
 }
 
-// FFT tables, in FP64 on the host then rounded to the recursion precision:
+// FFT tables in the recursion precision (formed in FP64):
 //   pre[s] = e^{2 pi i s / n_phi}, s < Nc (C2R packing), and for every radix-RP pass with
 //   Ns > 1 (pass plan: radix 4 while Nc/Ns >= 4, then 2) the block
-//   tw[off + (i-1) Ns + kk] = e^{2 pi i i kk / (Ns RP)}, i = 1..RP-1, kk < Ns.
-template <class R>
-static int upload_fft_tables(int n_phi, void** tw, void** pre, void** tw2, void** tw3)
+//   tw[off + (i-1) Ns + kk] = e^{2 pi i i kk / (Ns RP)}, i = 1..RP-1, kk < Ns;
+//   tw2, tw3: the same for the high-radix plans (passes of at most 16 and at most 8 points).
+__host__ __device__ inline int r4_table(int lgNc)  // entries of tw
 {
-    const int Nc = n_phi / 2;
-    std::vector<R> p(2 * (size_t)Nc), t;
-    for (int s = 0; s < Nc; ++s) {
-        p[2 * s] = (R)cos(2.0 * SMERF_PI * s / n_phi);
-        p[2 * s + 1] = (R)sin(2.0 * SMERF_PI * s / n_phi);
+    int n = 0;
+    for (int l = 2; l < lgNc; l += 2) n += (lgNc - l >= 2 ? 3 : 1) << l;
+    return n;
+}
+template <class R>
+__global__ void __launch_bounds__(256) fft_tables_kernel(int lgNc, cplx<R>* pre, cplx<R>* tw, cplx<R>* tw2, cplx<R>* tw3)
+{
+    const int Nc = 1 << lgNc, t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    auto root = [](int k, int n) {  // e^{2 pi i k / n}, n a power of two
+        double c, s;
+        sincospi(2.0 * (double)k / (double)n, &s, &c);
+        return cmk<cplx<R>>((R)c, (R)s);
+    };
+    for (int s = t0; s < Nc; s += nt) pre[s] = root(s, 2 * Nc);
+    // entry i of a pass of radix 2^b and stride Ns = 2^l: i = (a - 1) Ns + kk
+    auto entry = [&](int i, int l, int b) { return root(((i >> l) + 1) * (i & ((1 << l) - 1)), 1 << (l + b)); };
+    int off = 0;
+    for (int l = 2; l < lgNc; l += 2) {
+        const int b = lgNc - l >= 2 ? 2 : 1, n = ((1 << b) - 1) << l;
+        for (int i = t0; i < n; i += nt) tw[off + i] = entry(i, l, b);
+        off += n;
     }
-    int Ns = 1;
-    while (Ns < Nc) {
-        const int RP = (Nc / Ns >= 4) ? 4 : 2;
-        if (Ns > 1)
-            for (int i = 1; i < RP; ++i)
-                for (int kk = 0; kk < Ns; ++kk) {
-                    const double a = 2.0 * SMERF_PI * (double)i * kk / ((double)Ns * RP);
-                    t.push_back((R)cos(a));
-                    t.push_back((R)sin(a));
-                }
-        Ns *= RP;
-    }
-    if (t.empty()) t.assign(2, (R)0);
-    // high-radix plans (passes of at most 16 and at most 8 points)
-    int L = 0;
-    while ((1 << L) < Nc) ++L;
-    for (int t = 0; t < 2; ++t) {
-        const int MB = t == 0 ? 4 : SMERF_INPLACE_MB;
-        std::vector<R> t2;
-        for (int ps = 1; ps < smerf::hr_passes(L, MB); ++ps) {
-            const int RP = 1 << smerf::hr_bits(L, ps, MB), Ns2 = 1 << smerf::hr_lgns(L, ps, MB);
-            for (int i = 1; i < RP; ++i)
-                for (int kk = 0; kk < Ns2; ++kk) {
-                    const double a = 2.0 * SMERF_PI * (double)i * kk / ((double)Ns2 * RP);
-                    t2.push_back((R)cos(a));
-                    t2.push_back((R)sin(a));
-                }
+    for (int q = 0; q < 2; ++q) {
+        const int MB = q == 0 ? 4 : SMERF_INPLACE_MB;
+        cplx<R>* t = q == 0 ? tw2 : tw3;
+        for (int ps = 1; ps < smerf::hr_passes(lgNc, MB); ++ps) {
+            const int b = smerf::hr_bits(lgNc, ps, MB), l = smerf::hr_lgns(lgNc, ps, MB), n = ((1 << b) - 1) << l;
+            for (int i = t0; i < n; i += nt) t[smerf::hr_off(lgNc, ps, MB) + i] = entry(i, l, b);
         }
-        if (t2.empty()) t2.assign(2, (R)0);
-        void** dst = t == 0 ? tw2 : tw3;
-        if (smerf::dev_malloc(dst, t2.size() * sizeof(R)) != cudaSuccess) return SMERF_ENOMEM;
-        if (cudaMemcpy(*dst, t2.data(), t2.size() * sizeof(R), cudaMemcpyHostToDevice) != cudaSuccess) return SMERF_ECUDA;
     }
-    if (smerf::dev_malloc(tw, t.size() * sizeof(R)) != cudaSuccess) return SMERF_ENOMEM;
-    if (smerf::dev_malloc(pre, p.size() * sizeof(R)) != cudaSuccess) return SMERF_ENOMEM;
-    if (cudaMemcpy(*tw, t.data(), t.size() * sizeof(R), cudaMemcpyHostToDevice) != cudaSuccess) return SMERF_ECUDA;
-    if (cudaMemcpy(*pre, p.data(), p.size() * sizeof(R), cudaMemcpyHostToDevice) != cudaSuccess) return SMERF_ECUDA;
-    return SMERF_OK;
 }
 
 // ---------------------------------------------------------------- complex kappa-hat
@@ -993,6 +979,14 @@ __global__ void repack_rows_kernel(const float* __restrict__ rows, float* __rest
     packed[(pos * 3 + 2) * mp + m] = r.z;
 }
 
+// A set-up's temporaries: from the library's scratch pool (which keeps its memory between calls, so
+// that a program that makes plan after plan maps none), or, when large, from the default pool,
+// which returns them at the set-up's end
+cudaError_t setup_alloc(void** p, size_t bytes, int dev, cudaStream_t st)
+{
+    return bytes <= ((size_t)128 << 20) ? smerf_scratch_alloc(p, bytes, dev, st) : smerf::dev_malloc_async(p, bytes, st);
+}
+
 template <int M>
 int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
 {
@@ -1028,23 +1022,44 @@ int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
 
     pl->table_bytes = 0;
     pl->step_table_bytes = 0;
-    CK(smerf::dev_malloc((void**)&pl->beq, (size_t)tri(M) * mp * es));
-    CK(cudaMemsetAsync(pl->beq, 0, (size_t)tri(M) * mp * es, st));
-    pl->table_bytes += (size_t)tri(M) * mp * es;
+    {
+        // the start factor, the coarse tables and the FFT tables share one allocation (an allocation
+        // and its release cost 40 us each, as much as many a set-up's kernels)
+        int lg = 0;
+        while ((2 << lg) < pl->n_phi) ++lg;
+        const size_t cs = 2 * (pl->recur64 ? 8 : 4);
+        size_t end = 0;
+        auto part = [&end](size_t bytes) { const size_t o = end; end += (bytes + 255) / 256 * 256 + 256; return o; };
+        const size_t beq_b = (size_t)tri(M) * mp * es;
+        size_t coarse_b[2];
+        for (int c = 0; c < 2; ++c) coarse_b[c] = (size_t)(pl->chain[c].n_anchors + 1) * coarse_elems(M) * mp * es;
+        const size_t o_beq = part(beq_b), o_c0 = part(coarse_b[0]), o_c1 = part(coarse_b[1]), tables_end = end;
+        const size_t o_pre = part(cs << lg), o_tw = part(cs * r4_table(lg)),
+                     o_tw2 = part(cs * smerf::hr_off(lg, smerf::hr_passes(lg, 4), 4)),
+                     o_tw3 = part(cs * smerf::hr_off(lg, smerf::hr_passes(lg, SMERF_INPLACE_MB), SMERF_INPLACE_MB));
+        CK(smerf::dev_malloc((void**)&pl->shared, end));
+        CK(cudaMemsetAsync(pl->shared, 0, tables_end, st));
+        unsigned char* at = (unsigned char*)pl->shared;
+        pl->beq = at + o_beq;
+        pl->coarse[0] = at + o_c0;
+        pl->coarse[1] = at + o_c1;
+        pl->pre = at + o_pre;
+        pl->tw = at + o_tw;
+        pl->tw2 = at + o_tw2;
+        pl->tw3 = at + o_tw3;
+        pl->table_bytes += beq_b + coarse_b[0] + coarse_b[1];
+        const int blocks = ((4 << lg) + 255) / 256 < 152 ? ((4 << lg) + 255) / 256 : 152;
+        if (pl->recur64) fft_tables_kernel<double><<<blocks, 256, 0, st>>>(lg, (double2*)pl->pre, (double2*)pl->tw, (double2*)pl->tw2, (double2*)pl->tw3);
+        else fft_tables_kernel<float><<<blocks, 256, 0, st>>>(lg, (float2*)pl->pre, (float2*)pl->tw, (float2*)pl->tw2, (float2*)pl->tw3);
+        CK(cudaGetLastError());
+    }
     for (int c = 0; c < 2; ++c) {
-        const int len = pl->chain[c].len;
-        const size_t sb = (size_t)(len + 1) * step_row(M) * mp * es;
-        const size_t cb = (size_t)(pl->chain[c].n_anchors + 1) * coarse_elems(M) * mp * es;
-        CK(smerf::dev_malloc((void**)&pl->steps[c], sb > 0 ? sb : 16));
-        CK(cudaMemsetAsync(pl->steps[c], 0, sb > 0 ? sb : 16, st));
-        CK(smerf::dev_malloc((void**)&pl->coarse[c], cb > 0 ? cb : 16));
-        CK(cudaMemsetAsync(pl->coarse[c], 0, cb > 0 ? cb : 16, st));
-        pl->table_bytes += sb + cb;
+        const size_t sb = (size_t)(pl->chain[c].len + 1) * step_row(M) * mp * es;
+        CK(smerf::dev_malloc((void**)&pl->steps[c], sb));
+        CK(cudaMemsetAsync(pl->steps[c], 0, sb, st));
+        pl->table_bytes += sb;
         pl->step_table_bytes += sb;
     }
-    rc = pl->recur64 ? upload_fft_tables<double>(pl->n_phi, &pl->tw, &pl->pre, &pl->tw2, &pl->tw3)
-                     : upload_fft_tables<float>(pl->n_phi, &pl->tw, &pl->pre, &pl->tw2, &pl->tw3);
-    if (rc != SMERF_OK) goto done;
     if (pl->complex_spec) start_kernel_c<M><<<gm, threads, 0, st>>>(make_spec_c(pl), pl->beq, t64);
     else {
         start_kernel<M><<<((unsigned)pl->n_modes * start_lanes(M) + 63) / 64, 64, 0, st>>>(sp, pl->beq, t64);
@@ -1076,8 +1091,8 @@ int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
             }
             if (len > 0) {
                 const size_t nb = (size_t)(len + 1) * pl->n_modes * M * M * sizeof(double);
-                CK(smerf::dev_malloc_async((void**)&phi, nb, st));
-                CK(smerf::dev_malloc_async((void**)&qv, nb, st));
+                CK(setup_alloc((void**)&phi, nb, pl->dev, st));
+                CK(setup_alloc((void**)&qv, nb, pl->dev, st));
                 if (len > 65535) { rc = SMERF_EUNSUPPORTED; goto done; }
                 dim3 grid(gm, len);
                 if (pl->complex_spec) step_kernel_c<M><<<grid, threads, 0, st>>>(sc, len, phi, qv);
