@@ -199,6 +199,8 @@ __global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SamplePar
     constexpr int UV = band_unit_reals<Real, M, STAGE>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint4 rk[kKeyWords];
+    __shared__ int fxred[sizeof(Real) == 8 ? 2 * kFxRings : 1];
+    (void)fxred;
 
     const Segment sg = P.segs[blockIdx.z];
     const int r = blockIdx.y, c = sg.chain;
@@ -351,7 +353,8 @@ __global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SamplePar
                 if (!P.fft_r4) hr_c2r<C, 2, 12, true>(P.lgNc, x, w, e - k, (const C*)P.tw, (const C*)P.tw2, pre, gout, tid, nt);
                 else grp_c2r_rt<C>(x, w, e - k, P.lgNc, (const C*)P.tw, pre, gout, tid, nt);
             } else {
-                grp_c2r_rt<C>(x, w, e - k, P.lgNc, (const C*)P.tw, pre, gout, tid, nt);
+                grp_fx_c2r(x, w, e - k, P.lgNc, (const int4*)P.twx, (const int4*)P.prex, gout, fxred, tid, nt, kBarFft);
+                __syncthreads();  // fxred serves the next run
             }
             k = e;
         }

@@ -36,6 +36,14 @@ SMERF_HD uint64_t fx_mulhi(uint64_t a, uint64_t b)
     return (uint64_t)(((unsigned __int128)a * b) >> 64);
 #endif
 }
+// the same without the low words' product: 0 to 2 below the exact high word, with three of the four
+// widening multiplies (32 per SM and clock) and half of the carries.  For everything whose last
+// bits do not count
+SMERF_HD uint64_t fx_mulh(uint64_t a, uint64_t b)
+{
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+    return (uint64_t)ah * bh + (uint32_t)(((uint64_t)ah * bl) >> 32) + (uint32_t)(((uint64_t)al * bh) >> 32);
+}
 SMERF_HD uint32_t fx_mulhi(uint32_t a, uint32_t b)
 {
 #ifdef __CUDA_ARCH__
@@ -108,10 +116,10 @@ SMERF_HD void fx_neg_log(uint32_t a, FxLog lt, uint64_t& m, int& x)
     t = 0x00020000u + fx_mulhi(zt, t);
     t = 0x00924925u + fx_mulhi(zt, t);
     t = 0x2aaaaaabu + fx_mulhi(zt, t);
-    uint64_t h = 0x00000ccccccccccdull + fx_mulhi(zs, (uint64_t)t << 8);
-    h = 0x0004000000000000ull + fx_mulhi(zs, h);
-    h = 0x0155555555555555ull + fx_mulhi(zs, h);
-    h = 0x8000000000000000ull + fx_mulhi(zs, h);
+    uint64_t h = 0x00000ccccccccccdull + fx_mulh(zs, (uint64_t)t << 8);
+    h = 0x0004000000000000ull + fx_mulh(zs, h);
+    h = 0x0155555555555555ull + fx_mulh(zs, h);
+    h = 0x8000000000000000ull + fx_mulh(zs, h);
     const uint64_t zh = fx_mulhi(z, h);
     // f near 1 (c = 1) and no power of two: y = z (1 + zH) alone, from z's own leading bit on;
     // otherwise ln c + the series + k ln 2, to 2^-59 of values above 2^-7
@@ -126,7 +134,7 @@ SMERF_HD void fx_neg_log(uint32_t a, FxLog lt, uint64_t& m, int& x)
         e = -59;
     }
     if (one) {
-        y = zn + fx_mulhi(zn, zh);
+        y = zn + fx_mulh(zn, zh);
         e = -64 - s;
     }
     const int n = fx_clz(y);
@@ -150,8 +158,8 @@ SMERF_HD void fx_sqrt2(uint64_t m, int x, uint64_t& r, int& xr)
     const float qf = 1.0f / sqrtf(vf);
 #endif
     const uint64_t q = (uint64_t)(uint32_t)(qf * 0x1p30f) << 32;  // q 2^-62, in (1, 2]
-    const uint64_t s0 = fx_mulhi(V, q) << 1;                       // s 2^-63
-    const int64_t d0 = (int64_t)((V >> 2) - fx_mulhi(s0, s0));     // v - s0^2, 2^-62, |d0| < 2^42
+    const uint64_t s0 = fx_mulh(V, q) << 1;                       // s 2^-63
+    const int64_t d0 = (int64_t)((V >> 2) - fx_mulh(s0, s0));     // v - s0^2, 2^-62, |d0| < 2^42
     const int64_t c0 = ((d0 >> 8) * (int64_t)(q >> 34)) >> 20;      // q d0 / 2: 2^-54 2^-28 2^-1 2^20 = 2^-63
     const uint64_t s1 = s0 + (uint64_t)c0;
     // v - s1^2 to 2^-94: the exact 128-bit product's bits below 2^-62
@@ -166,37 +174,79 @@ SMERF_HD void fx_sqrt2(uint64_t m, int x, uint64_t& r, int& xr)
 // (r 2^(xr - 64)) (t 2^(xt - 64)) rounded to a double
 SMERF_HD double fx_normal(uint64_t r, int xr, uint64_t t, int xt, bool neg)
 {
-    const uint64_t p = fx_mulhi(r, t);
+    const uint64_t p = fx_mulh(r, t);
     const int n = fx_clz(p);
     const uint64_t m = ((p << n) >> 11) + (((p << n) >> 10) & 1);  // 2^52 .. 2^53
     // value = m 2^(xr + xt - n - 53); a carry to 2^53 moves the exponent by itself
     const uint64_t bits = ((uint64_t)(uint32_t)(1022 + xr + xt - n - 1) << 52) + m;
     return fx_double(bits | (neg ? 0x8000000000000000ull : 0ull));
 }
-// t = T 2^-64 in [0, 1): S with sin(pi/4 t) = t S 2^-64, and cos(pi/4 t) as a 64-bit fraction
+// t = T 2^-64 in [0, 1): S with sin(pi/4 t) = t S 2^-64, and cos(pi/4 t) as a 64-bit fraction, to
+// 2^-60
 SMERF_HD void fx_octant(uint64_t T, uint64_t& sn, uint64_t& cs)
 {
-    const uint64_t T2 = fx_mulhi(T, T);
+    const uint64_t T2 = fx_mulh(T, T);
     const uint32_t th = (uint32_t)(T2 >> 32);
     // sin(pi/4 t) = t S(t^2), cos(pi/4 t) = 1 - t^2 D(t^2): Taylor series
     uint32_t q = 0x0000b7d7u - fx_mulhi(th, 0x0000006bu);
     q = 0x00f47a1au - fx_mulhi(th, q);
     q = 0xf183a7efu - fx_mulhi(th, q);
-    uint64_t S = 0x00000541e0d21fbaull - fx_mulhi(T2, (uint64_t)q << 3);
-    S = 0x000265a599cc57b1ull - fx_mulhi(T2, S);
-    S = 0x00a335e33bad570full - fx_mulhi(T2, S);
-    S = 0x14abbce625be52bfull - fx_mulhi(T2, S);
-    S = 0xc90fdaa22168c235ull - fx_mulhi(T2, S);
+    uint64_t S = 0x00000541e0d21fbaull - fx_mulh(T2, (uint64_t)q << 3);
+    S = 0x000265a599cc57b1ull - fx_mulh(T2, S);
+    S = 0x00a335e33bad570full - fx_mulh(T2, S);
+    S = 0x14abbce625be52bfull - fx_mulh(T2, S);
+    S = 0xc90fdaa22168c235ull - fx_mulh(T2, S);
     q = 0x00009063u - fx_mulhi(th, 0x0000004bu);
     q = 0x00db7128u - fx_mulhi(th, q);
     q = 0xfce9c51cu - fx_mulhi(th, q);
-    uint64_t D = 0x00000069b47ca881ull - fx_mulhi(T2, (uint64_t)(q >> 1));
-    D = 0x00003c3ea0d12375ull - fx_mulhi(T2, D);
-    D = 0x00155d3c7e3cbffaull - fx_mulhi(T2, D);
-    D = 0x040f07c206d6b0edull - fx_mulhi(T2, D);
-    D = 0x4ef4f326f9177969ull - fx_mulhi(T2, D);
+    uint64_t D = 0x00000069b47ca881ull - fx_mulh(T2, (uint64_t)(q >> 1));
+    D = 0x00003c3ea0d12375ull - fx_mulh(T2, D);
+    D = 0x00155d3c7e3cbffaull - fx_mulh(T2, D);
+    D = 0x040f07c206d6b0edull - fx_mulh(T2, D);
+    D = 0x4ef4f326f9177969ull - fx_mulh(T2, D);
     sn = S;
-    cs = 0ull - (fx_mulhi(T2, D) | 1);  // in [0.707, 1)
+    cs = 0ull - (fx_mulh(T2, D) | 1);  // in [0.707, 1)
+}
+// The same to about a unit, for tables of factors: each coefficient normalised (c 2^(64 + shift)), so
+// that a term's rounding counts by its own size, and every product rounded
+SMERF_HD uint64_t fx_mulr(uint64_t a, uint64_t b) { return fx_mulhi(a, b) + ((a * b) >> 63); }
+SMERF_HD uint64_t fx_horner(uint64_t T2, const uint64_t* c, const int* shift, int n)
+{
+    uint64_t v = c[n - 1];
+    for (int k = n - 2; k >= 0; --k) {
+        const int d = shift[k + 1] - shift[k];
+        const uint64_t p = fx_mulr(T2, v);
+        v = c[k] - (d > 0 ? (p >> d) + ((p >> (d - 1)) & 1) : p);
+    }
+    return v;
+}
+SMERF_HD void fx_octant_exact(uint64_t T, uint64_t& sn, uint64_t& cs)
+{
+    const uint64_t c[10] = {0xc90fdaa22168c235ull, 0xa55de7312df295f5ull, 0xa335e33bad570e92ull, 0x9969667315ec2df3ull,
+                            0xa83c1a43f73c0dc8ull, 0xf183a7ef4438fb12ull, 0xf47a1a680c6b1994ull, 0xb7d6dcf8aaba1c8bull,
+                            0xd5761957c99ac950ull, 0xc5202108fcaa382eull};
+    const int cx[10] = {0, 3, 8, 14, 21, 29, 37, 45, 54, 63};
+    const uint64_t d[10] = {0x9de9e64df22ef2d2ull, 0x81e0f840dad61d9bull, 0xaae9e3f1e5ffcfe3ull, 0xf0fa83448dd5d7a3ull,
+                            0xd368f95102545d4dull, 0xfce9c51bb1e6146full, 0xdb7127a25894796eull, 0x9063161796bfa54cull,
+                            0x95062c8d7c18a243ull, 0xf7b71846b68e1c74ull};
+    const int dx[10] = {1, 5, 11, 18, 25, 33, 41, 49, 58, 68};
+    const uint64_t T2 = fx_mulr(T, T);
+    sn = fx_horner(T2, c, cx, 10);
+    const uint64_t p = fx_mulr(T2, fx_horner(T2, d, dx, 10));  // 2 (1 - cos)
+    cs = 0ull - (((p >> 1) + (p & 1)) | (p == 0));
+}
+// e^{2 pi i p}, p = ph 2^-64 turns, in units of 2^-62 (to one unit)
+SMERF_HD void fx_cis62(uint64_t ph, int64_t& c, int64_t& s)
+{
+    const int o = (int)(ph >> 61);
+    uint64_t T = ph << 3, S, cs;
+    if (o & 1) T = ~T;
+    fx_octant_exact(T, S, cs);
+    const uint64_t sn = fx_mulr(T, S);
+    const int64_t a = (int64_t)((sn >> 2) + ((sn >> 1) & 1)), b = (int64_t)((cs >> 2) + ((cs >> 1) & 1));
+    const bool swap = (o + 1) & 2;
+    c = ((o + 2) & 4) ? -(swap ? a : b) : (swap ? a : b);
+    s = (o & 4) ? -(swap ? b : a) : (swap ? b : a);
 }
 // e^{2 pi i p}, p = ph 2^-64 turns, to 2^-63 (four FP64 instructions)
 SMERF_HD void fx_cis(uint64_t ph, double& c, double& s)
@@ -224,10 +274,46 @@ SMERF_HD void fx_box_muller(uint32_t a, uint32_t b, FxLog lt, double& n0, double
     const uint64_t T = (uint64_t)w << 34;
     fx_octant(T, S, cs);
     const int lw = fx_clz(T);
-    const uint64_t sn = fx_mulhi(T << lw, S);  // sin 2^(64 + lw)
+    const uint64_t sn = fx_mulh(T << lw, S);  // sin 2^(64 + lw)
     const bool swap = (o + 1) & 2;
     n0 = fx_normal(r, xr, swap ? sn : cs, swap ? -lw : 0, (o + 2) & 4);
     n1 = fx_normal(r, xr, swap ? cs : sn, swap ? 0 : -lw, o & 4);
+}
+
+// ---- 64-bit fixed-point values of a ring's FFT
+// v in units of 2^-S, |v| 2^S < 2^62 (round to nearest)
+SMERF_HD int64_t fx_from_double(uint64_t bits, int S)
+{
+    const int e = (int)((bits >> 52) & 0x7ff), k = e - 1075 + S;
+    const uint64_t m = (bits & 0xfffffffffffffull) | 0x10000000000000ull;
+    uint64_t v = 0;
+    if (e > 0 && k > -54) v = k >= 0 ? m << k : (m + (1ull << (-k - 1))) >> -k;
+    return (int64_t)(bits >> 63 ? 0 - v : v);
+}
+// x 2^-S rounded to a double (below the normal range: 0)
+SMERF_HD uint64_t fx_to_double(int64_t x, int S)
+{
+    const uint64_t sign = (uint64_t)x & 0x8000000000000000ull, a = x < 0 ? 0 - (uint64_t)x : (uint64_t)x;
+    const int n = fx_clz(a | 1), e = 1022 + 63 - n - S;
+    const uint64_t m = a << n, bits = ((uint64_t)(uint32_t)e << 52) + (m >> 11) + ((m >> 10) & 1);
+    return a == 0 || e <= 0 ? sign : bits | sign;
+}
+// a factor of magnitude at most 1 in units of 2^-62 as two signed words, hi 2^32 + lo
+SMERF_HD void fx_split(int64_t w, int32_t& hi, int32_t& lo)
+{
+    lo = (int32_t)(uint32_t)w;
+    hi = (int32_t)((w - lo) >> 32);
+}
+// a.x w.x - a.y w.y (SUB) or a.x w.x + a.y w.y, from the parts (w in units of 2^-62, |a| < 2^62, |w|
+// <= 1 as complex numbers, so that the middle sum stays below 2^63): the high words' products to
+// all bits, the mixed ones rounded, the low words' products (below one unit) left out
+template <bool SUB>
+SMERF_HD int64_t fx_dot(int32_t axh, int32_t axl, int32_t wxh, int32_t wxl, int32_t ayh, int32_t ayl, int32_t wyh, int32_t wyl)
+{
+    const int64_t h0 = (int64_t)axh * wxh, h1 = (int64_t)ayh * wyh;
+    const int64_t m0 = (int64_t)axh * wxl + (int64_t)axl * wxh, m1 = (int64_t)ayh * wyl + (int64_t)ayl * wyh;
+    const int64_t hh = SUB ? h0 - h1 : h0 + h1, mid = SUB ? m0 - m1 : m0 + m1;
+    return (int64_t)((uint64_t)hh << 2) + ((mid + (1ll << 29)) >> 30);
 }
 
 }  // namespace smerf

@@ -68,6 +68,9 @@ struct smerf_plan {
     // per-pass twiddles of the high-radix plans (hr_* below, MB = 4 and 3), recursion precision
     void* tw2;
     void* tw3;
+    // FP64 recursion: tw and pre in fixed point (int4 each)
+    void* twx;
+    void* prex;
     size_t table_bytes;
     size_t step_table_bytes;  // the two step tables' part of table_bytes
     double setup_ms;
@@ -104,6 +107,8 @@ struct SampleParams {
     const void* pre;  // complex e^{2 pi i s / n_phi}, s < Nc
     const void* tw2;  // per-pass complex twiddles of the high-radix plan, MB = 4 (hr_off)
     const void* tw3;  // the same for MB = 3
+    const void* twx;  // FP64 recursion: tw and pre in fixed point (int4: Re hi, lo, Im hi, lo)
+    const void* prex;
     void* anc;        // anchor states [c][r][j][2M][n_slots]
     void* out;
     uint64_t seed;

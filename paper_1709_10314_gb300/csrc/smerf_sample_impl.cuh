@@ -1096,6 +1096,162 @@ __device__ __forceinline__ void grp_c2r_rt(C* buf0, C* buf1, int R, int lgNc, co
     }
 }
 
+// ---- the FP64 mode's ring FFT in 64-bit fixed point.  On the FP64 pipe (2 lanes per SM) a ring's
+// C2R FFT took two thirds of what is left of the FP64 instructions once the noise is off it; in
+// integers a radix-4 pass costs some 34 instructions per point on 64 to 128 lanes.  A ring's
+// coefficients are scaled by one power of two 2^S that keeps 4 sum |g_m|, a bound of every
+// intermediate value, below 2^62; the sum is formed in integers (largest exponent first, then 17-bit
+// magnitudes rounded up), so that the scale, and with it the field's bits, depend on no thread
+// count.  Values then keep 2^-60 of that sum, so that a field's error against 64-bit references is
+// not above the FP64 FFT's (3.3e-15 -> 3.1e-15 at 64 x 128, 3.9e-15 -> 3.5e-15 at 32 x 64, 1.3e-13 ->
+// 1.0e-13 and 8.6e-13 -> 5.1e-13 on larger grids, the tables' own error).  1024 x 2048, p = 2, 16
+// realisations: 2161 -> 1393 us; 20001 of 32 x 64: 3057 -> 2523 us.  Factors e^{2 pi i k / n} are exact to 2^-62, stored as two words
+// per component (int4: Re hi, lo, Im hi, lo).
+using fxc = longlong2;
+
+__device__ __forceinline__ fxc fxc_mul(fxc a, int4 w)
+{
+    int32_t axh, axl, ayh, ayl;
+    fx_split(a.x, axh, axl);
+    fx_split(a.y, ayh, ayl);
+    fxc r;
+    r.x = fx_dot<true>(axh, axl, w.x, w.y, ayh, ayl, w.z, w.w);
+    r.y = fx_dot<false>(axh, axl, w.z, w.w, ayh, ayl, w.x, w.y);
+    return r;
+}
+
+constexpr int kFxRings = 16;  // rings of one call (the band kernel's chunk)
+
+// scale of ring r from its largest exponent and its sum of magnitudes (units of 2^(e - 16))
+__device__ __forceinline__ int fx_scale(const int* red, int r)
+{
+    return 60 - (red[r] - 1039 + 32 - __clz(red[kFxRings + r]));
+}
+
+// The rings' largest exponents into red[r], their sums into red[kFxRings + r]
+__device__ __forceinline__ void grp_fx_scales(const double2* buf, int R, int lgNc, int* red, int ftid, int nf, int bar)
+{
+    const int total = R << lgNc;
+    const bool whole = lgNc >= 5;  // a warp's 32 neighbouring elements lie in one ring
+    if (ftid < R) red[ftid] = red[kFxRings + ftid] = 0;
+    bar_sync(bar, nf);
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        unsigned acc = 0;
+        for (int b = ftid; b < total; b += nf) {
+            const double2 v = buf[b];
+            const int r = b >> lgNc;
+            const unsigned hx = (unsigned)__double2hiint(v.x) & 0x7fffffffu, hy = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
+            unsigned t;
+            if (pass == 0) {
+                t = (hx > hy ? hx : hy) >> 20;
+            } else {
+                // 2^16 times the magnitude over 2^(largest exponent), rounded up
+                const int top = red[r];
+                const int sx = top - (int)(hx >> 20), sy = top - (int)(hy >> 20);
+                t = (sx > 20 ? 0u : ((hx & 0xfffffu) | 0x100000u) >> 4 >> sx) + (sy > 20 ? 0u : ((hy & 0xfffffu) | 0x100000u) >> 4 >> sy) + 2u;
+            }
+            if (!whole) {
+                if (pass == 0) atomicMax(reinterpret_cast<unsigned*>(red) + r, t);
+                else atomicAdd(reinterpret_cast<unsigned*>(red) + kFxRings + r, t);
+                continue;
+            }
+            acc = pass == 0 ? (acc > t ? acc : t) : acc + t;
+            if (b + nf >= total || (b + nf) >> lgNc != r) {  // the warp's last elements of this ring
+                acc = pass == 0 ? __reduce_max_sync(0xffffffffu, acc) : __reduce_add_sync(0xffffffffu, acc);
+                if ((ftid & 31) == 0) {
+                    if (pass == 0) atomicMax(reinterpret_cast<unsigned*>(red) + r, acc);
+                    else atomicAdd(reinterpret_cast<unsigned*>(red) + kFxRings + r, acc);
+                }
+                acc = 0;
+            }
+        }
+        bar_sync(bar, nf);
+    }
+}
+
+// C2R FFTs of R rings (coefficients in buf0 as double2, buf1 the second buffer), radix-4 passes
+// (radix 2 last when log2 Nc is odd); prex, twx: the plan's factors as int4; red: 2 kFxRings words
+__device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, int lgNc, const int4* __restrict__ twx,
+                                           const int4* __restrict__ prex, RingOut<double2> gout, int* red, int ftid,
+                                           int nf, int bar)
+{
+    const int Nc = 1 << lgNc;
+    grp_fx_scales(buf0, R, lgNc, red, ftid, nf, bar);
+    fxc* src = reinterpret_cast<fxc*>(buf0);
+    fxc* dst = reinterpret_cast<fxc*>(buf1);
+    // to fixed point and packed (c2r_pack) in place, the pair s, Nc - s together
+    const int half = Nc / 2 + 1;
+    for (int b = ftid; b < R * half; b += nf) {
+        const int r = b / half, s = b - r * half, S = fx_scale(red, r);
+        auto get = [&](int i) {
+            const double2 v = buf0[(r << lgNc) + i];
+            fxc f;
+            f.x = fx_from_double((uint64_t)__double_as_longlong(v.x), S);
+            f.y = fx_from_double((uint64_t)__double_as_longlong(v.y), S);
+            return f;
+        };
+        fxc* X = src + (r << lgNc);
+        const fxc a = get(s);
+        if (s == 0) {
+            X[0] = cmk<fxc>(a.x + a.y, a.x - a.y);
+            continue;
+        }
+        const fxc bb = cconj(get(Nc - s));
+        const fxc e = cadd(a, bb), o = cmuli(fxc_mul(csub(a, bb), __ldg(prex + s)));
+        X[s] = cadd(e, o);
+        if (2 * s < Nc) X[Nc - s] = cconj(csub(e, o));
+    }
+    bar_sync(bar, nf);
+    int Ns = 1, off = 0;
+    while (Ns < Nc) {
+        const int RP = pass_radix(lgNc, Ns), LR = RP == 4 ? 2 : 1;
+        const bool first = Ns == 1, last = Ns * RP == Nc;
+        const int lgnb = lgNc - LR, nb = 1 << lgnb, total = R << lgnb;
+        for (int b = ftid; b < total; b += nf) {
+            const int r = b >> lgnb, j = b & (nb - 1), kk = j & (Ns - 1);
+            const fxc* X = src + (r << lgNc);
+            fxc v[4];
+            v[0] = X[j];
+            v[1] = X[j + nb];
+            if (RP == 4) {
+                v[2] = X[j + 2 * nb];
+                v[3] = X[j + 3 * nb];
+            }
+            if (!first) {
+                v[1] = fxc_mul(v[1], __ldg(twx + off + kk));
+                if (RP == 4) {
+                    v[2] = fxc_mul(v[2], __ldg(twx + off + Ns + kk));
+                    v[3] = fxc_mul(v[3], __ldg(twx + off + 2 * Ns + kk));
+                }
+            }
+            if (RP == 4) dft4(v);
+            else dft2(v[0], v[1]);
+            const int idx = ((j - kk) << LR) + kk;
+            if (last) {
+                const int S = fx_scale(red, r);
+                double2* D = gout[r] + idx;
+#pragma unroll
+                for (int a = 0; a < 4; ++a)
+                    if (a < RP)
+                        __stcs(D + a * Ns, make_double2(__longlong_as_double((long long)fx_to_double(v[a].x, S)),
+                                                        __longlong_as_double((long long)fx_to_double(v[a].y, S))));
+            } else {
+                fxc* D = dst + (r << lgNc) + idx;
+#pragma unroll
+                for (int a = 0; a < 4; ++a)
+                    if (a < RP) D[a * Ns] = v[a];
+            }
+        }
+        if (!first) off += (RP - 1) * Ns;
+        Ns *= RP;
+        if (!last) bar_sync(bar, nf);
+        fxc* t = src;
+        src = dst;
+        dst = t;
+    }
+}
+
 // ---- high-radix plan (hr_passes / hr_bits): passes of radix up to 16 held in registers.
 // Between passes the rings sit in shared memory in an XOR-swizzled order, element e at
 // e ^ ((e >> 4) & 15), so that the strided stores of the early passes and the unit-stride
@@ -1268,6 +1424,8 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
     constexpr int NU = unit_vals(M), NC = unit_calls(M);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint4 rk[RMAX][kKeyWords];
+    __shared__ int fxred[sizeof(Real) == 8 ? 2 * kFxRings : 1];
+    (void)fxred;
 
     const Segment sg = P.segs[seg_index];
     const int r0 = group * RMAX;
@@ -1426,10 +1584,10 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
             if (!(c == 1 && pos == 0)) {  // the start ring is written by the northern chain
                 RingOut<C> gout{(C*)((Real*)P.out + ((size_t)r0 * P.n_theta + ring) * (size_t)P.n_phi),
                                 (size_t)P.n_theta * (size_t)(P.n_phi / 2)};
-                if (sizeof(Real) == 4 && !P.fft_r4) {
-                    if constexpr (sizeof(Real) == 4)
-                        hr_c2r<C, ws_lg_lo(UPT, M), ws_lg_hi(UPT, M), PAIR>(P.lgNc, B, W, R, twp, (const C*)P.tw2, pre, gout,
-                                                                       ftid, NF);
+                if constexpr (sizeof(Real) == 8) {
+                    grp_fx_c2r(B, W, R, P.lgNc, (const int4*)P.twx, (const int4*)P.prex, gout, fxred, ftid, NF, kBarFft);
+                } else if (!P.fft_r4) {
+                    hr_c2r<C, ws_lg_lo(UPT, M), ws_lg_hi(UPT, M), PAIR>(P.lgNc, B, W, R, twp, (const C*)P.tw2, pre, gout, ftid, NF);
                 } else {
                     grp_c2r_rt<C>(B, W, R, P.lgNc, twp, pre, gout, ftid, NF);
                 }
@@ -2061,6 +2219,8 @@ int fill_params(const smerf_plan* pl, uint64_t seed, int n, void* out, void* scr
     P.pre = pl->pre;
     P.tw2 = pl->tw2;
     P.tw3 = pl->tw3;
+    P.twx = pl->twx;
+    P.prex = pl->prex;
     P.anc = scratch;
     P.out = out;
     P.seed = seed;

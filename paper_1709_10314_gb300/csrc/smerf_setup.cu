@@ -693,8 +693,18 @@ __host__ __device__ inline int r4_table(int lgNc)  // entries of tw
     for (int l = 2; l < lgNc; l += 2) n += (lgNc - l >= 2 ? 3 : 1) << l;
     return n;
 }
+__device__ inline int4 fx_root(int k, int lgn)  // e^{2 pi i k / 2^lgn} in fixed point
+{
+    int64_t c, s;
+    fx_cis62((uint64_t)(unsigned)k << (64 - lgn), c, s);
+    int4 w;
+    fx_split(c, w.x, w.y);
+    fx_split(s, w.z, w.w);
+    return w;
+}
 template <class R>
-__global__ void __launch_bounds__(256) fft_tables_kernel(int lgNc, cplx<R>* pre, cplx<R>* tw, cplx<R>* tw2, cplx<R>* tw3)
+__global__ void __launch_bounds__(256) fft_tables_kernel(int lgNc, cplx<R>* pre, cplx<R>* tw, cplx<R>* tw2, cplx<R>* tw3,
+                                                         int4* prex, int4* twx)
 {
     const int Nc = 1 << lgNc, t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
     auto root = [](int k, int n) {  // e^{2 pi i k / n}, n a power of two
@@ -702,13 +712,19 @@ __global__ void __launch_bounds__(256) fft_tables_kernel(int lgNc, cplx<R>* pre,
         sincospi(2.0 * (double)k / (double)n, &s, &c);
         return cmk<cplx<R>>((R)c, (R)s);
     };
-    for (int s = t0; s < Nc; s += nt) pre[s] = root(s, 2 * Nc);
+    for (int s = t0; s < Nc; s += nt) {
+        pre[s] = root(s, 2 * Nc);
+        if (sizeof(R) == 8) prex[s] = fx_root(s, lgNc + 1);
+    }
     // entry i of a pass of radix 2^b and stride Ns = 2^l: i = (a - 1) Ns + kk
     auto entry = [&](int i, int l, int b) { return root(((i >> l) + 1) * (i & ((1 << l) - 1)), 1 << (l + b)); };
     int off = 0;
     for (int l = 2; l < lgNc; l += 2) {
         const int b = lgNc - l >= 2 ? 2 : 1, n = ((1 << b) - 1) << l;
-        for (int i = t0; i < n; i += nt) tw[off + i] = entry(i, l, b);
+        for (int i = t0; i < n; i += nt) {
+            tw[off + i] = entry(i, l, b);
+            if (sizeof(R) == 8) twx[off + i] = fx_root(((i >> l) + 1) * (i & ((1 << l) - 1)), l + b);
+        }
         off += n;
     }
     for (int q = 0; q < 2; ++q) {
@@ -1036,7 +1052,8 @@ int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
         const size_t o_beq = part(beq_b), o_c0 = part(coarse_b[0]), o_c1 = part(coarse_b[1]), tables_end = end;
         const size_t o_pre = part(cs << lg), o_tw = part(cs * r4_table(lg)),
                      o_tw2 = part(cs * smerf::hr_off(lg, smerf::hr_passes(lg, 4), 4)),
-                     o_tw3 = part(cs * smerf::hr_off(lg, smerf::hr_passes(lg, SMERF_INPLACE_MB), SMERF_INPLACE_MB));
+                     o_tw3 = part(cs * smerf::hr_off(lg, smerf::hr_passes(lg, SMERF_INPLACE_MB), SMERF_INPLACE_MB)),
+                     o_prex = part(pl->recur64 ? sizeof(int4) << lg : 0), o_twx = part(pl->recur64 ? sizeof(int4) * r4_table(lg) : 0);
         CK(smerf::dev_malloc((void**)&pl->shared, end));
         CK(cudaMemsetAsync(pl->shared, 0, tables_end, st));
         unsigned char* at = (unsigned char*)pl->shared;
@@ -1047,10 +1064,13 @@ int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
         pl->tw = at + o_tw;
         pl->tw2 = at + o_tw2;
         pl->tw3 = at + o_tw3;
+        pl->prex = at + o_prex;
+        pl->twx = at + o_twx;
         pl->table_bytes += beq_b + coarse_b[0] + coarse_b[1];
         const int blocks = ((4 << lg) + 255) / 256 < 152 ? ((4 << lg) + 255) / 256 : 152;
-        if (pl->recur64) fft_tables_kernel<double><<<blocks, 256, 0, st>>>(lg, (double2*)pl->pre, (double2*)pl->tw, (double2*)pl->tw2, (double2*)pl->tw3);
-        else fft_tables_kernel<float><<<blocks, 256, 0, st>>>(lg, (float2*)pl->pre, (float2*)pl->tw, (float2*)pl->tw2, (float2*)pl->tw3);
+        if (pl->recur64) fft_tables_kernel<double><<<blocks, 256, 0, st>>>(lg, (double2*)pl->pre, (double2*)pl->tw, (double2*)pl->tw2, (double2*)pl->tw3,
+                                                                           (int4*)pl->prex, (int4*)pl->twx);
+        else fft_tables_kernel<float><<<blocks, 256, 0, st>>>(lg, (float2*)pl->pre, (float2*)pl->tw, (float2*)pl->tw2, (float2*)pl->tw3, nullptr, nullptr);
         CK(cudaGetLastError());
     }
     for (int c = 0; c < 2; ++c) {
