@@ -19,8 +19,8 @@
 // (4, 2, then the odd primes), one output point per thread from r terms with the roots of unity
 // from a table of the ring's own, a group of threads per ring.  HEALPix's polar rings (4i points)
 // took O(n^2) terms in the FFT warps of one CTA per segment before: Nside 128, 16 realisations,
-// 4266 -> 137 us a call.  One FP64 realisation of 64 x 128 in Alg. 2's order: 166 -> 33 us; one of
-// 181 x 512, p = 2: 31.1 -> 23.6 us (the anchor tiles among them).
+// 4266 -> 119 us a call.  One FP64 realisation of 64 x 128 in Alg. 2's order: 166 -> 26 us; one of
+// 181 x 512, p = 2: 31.1 -> 22.4 us (the anchor tiles among them).
 #pragma once
 
 namespace smerf {
@@ -165,45 +165,44 @@ __device__ __forceinline__ void band_step(const Real (&t)[kG<M>][step_row(M)], c
         }
 }
 
-// What a (ring, unit) of a chunk keeps in shared memory between parts 1 and 2: its normals and,
-// staged, its table rows; an odd number of 16-byte words, so that neighbouring units' vector
-// accesses fall on different banks
-template <class Real, int M, bool STAGE>
-__host__ __device__ constexpr int band_unit_reals()
+// Reals of a unit's staged table rows: an odd number of 16-byte words, so that neighbouring units'
+// vector accesses fall on different banks
+template <class Real, int M>
+__host__ __device__ constexpr int band_row_reals()
 {
-    const int v = unit_vals(M) + (STAGE ? unit_slots(M) * step_row(M) : 0), w = 16 / (int)sizeof(Real);
-    return STAGE && (v / w) % 2 == 0 ? v + w : v;
+    const int v = unit_slots(M) * step_row(M), w = 16 / (int)sizeof(Real);
+    return (v / w) % 2 == 0 ? v + w : v;
 }
 
-// Shared memory (cplx = 2 Real): X [chunk][Nc] cplx; the units' words [chunk][units][UV] Real, the
-// same memory then the FFTs' second buffer [chunk][Nc] cplx; the states [units][NU] Real; the
-// Nyquist chain's rows [chunk][ROW] Real; the root tables [groups][Nc] cplx (ring-dependent
-// longitudes only)
+// Shared memory (cplx = 2 Real), rb realisations: X [rb][chunk][Nc] cplx; the normals [rb][chunk][units][NU]
+// Real, the same memory then the FFTs' second buffer [rb][chunk][Nc] cplx; the staged rows
+// [chunk][units][RV] Real; the states [rb][units][NU] Real; the Nyquist chain's rows [chunk][ROW] Real;
+// the root tables [groups][Nc] cplx (ring-dependent longitudes only)
 template <class Real, int M, bool STAGE>
-__host__ __device__ inline size_t band_smem(int Nc, int chunk, bool rings)
+__host__ __device__ inline size_t band_smem(int Nc, int chunk, int rb, bool rings)
 {
     const int units = Nc / unit_slots(M);
-    const size_t x = (size_t)Nc * 2 * sizeof(Real), uv = (size_t)units * band_unit_reals<Real, M, STAGE>() * sizeof(Real);
-    return chunk * (x + uv + step_row(M) * sizeof(Real)) + (size_t)units * unit_vals(M) * sizeof(Real) +
-           (rings ? (kBandThreads / band_group(Nc)) * x : 0);
+    const size_t x = (size_t)Nc * 2 * sizeof(Real), nz = (size_t)units * unit_vals(M) * sizeof(Real);
+    const size_t rows = (STAGE ? (size_t)units * band_row_reals<Real, M>() : 0) * sizeof(Real) + step_row(M) * sizeof(Real);
+    return chunk * (rb * (x + nz) + rows) + rb * nz + (rings ? (kBandThreads / band_group(Nc)) * x : 0);
 }
 
-// grid (splits, realisations, segments)
+// grid (splits, realisations / rb, segments)
 // STAGE: the chunk's table rows go through shared memory, loaded in part 1 beside the noise by
 // every thread, so that the recursion waits for no global load
 template <class Real, class TabT, int M, bool STAGE>
-__global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SampleParams P, int chunk)
+__global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SampleParams P, int chunk, int rb)
 {
     using C = cplx<Real>;
     constexpr int G = kG<M>, ROW = step_row(M), NU = unit_vals(M), NC = unit_calls(M);
-    constexpr int UV = band_unit_reals<Real, M, STAGE>();
+    constexpr int RV = band_row_reals<Real, M>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint4 rk[kKeyWords];
+    __shared__ uint4 rk[2][kKeyWords];  // rb <= 2
     __shared__ int fxred[sizeof(Real) == 8 ? 2 * kFxRings : 1];
     (void)fxred;
 
     const Segment sg = P.segs[blockIdx.z];
-    const int r = blockIdx.y, c = sg.chain;
+    const int r = blockIdx.y * rb, c = sg.chain, nr = min(rb, P.n_samples - r);  // realisations r .. r + nr - 1
     const int tid = threadIdx.x, nt = kBandThreads;
     const int Nc = P.Nc, n_units = P.n_units;
     const size_t mp = P.n_modes_pad;
@@ -214,22 +213,20 @@ __global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SamplePar
     const int own1 = first + (int)((long long)len * (blockIdx.x + 1) / gridDim.x);
     if (own0 >= own1) return;
 
+    const int cn = chunk * n_units;  // units of a realisation's chunk
     C* X = reinterpret_cast<C*>(smem_raw);
-    Real* NZ = reinterpret_cast<Real*>(X + (size_t)chunk * Nc);
+    Real* NZ = reinterpret_cast<Real*>(X + (size_t)rb * chunk * Nc);
     C* W = reinterpret_cast<C*>(NZ);
-    Real* S = NZ + (size_t)chunk * n_units * UV;
-    Real* NY = S + (size_t)n_units * NU;
+    Real* RW = NZ + (size_t)rb * cn * NU;
+    Real* S = RW + (STAGE ? (size_t)cn * RV : 0);
+    Real* NY = S + (size_t)rb * n_units * NU;
     C* RT = reinterpret_cast<C*>(NY + (size_t)chunk * ROW);
     const Real* anc = (const Real*)P.anc;
+    const size_t anc_r = aoff<M>(P, 0, 1, 0, 0, 0);  // from one realisation's anchor states to the next's
     const Real* xrg = anc + aoff<M>(P, c, r, has_right ? sg.right : 0, 0, 0);
     const Real* xlg = anc + aoff<M>(P, c, r, sg.left, 0, 0);
     const TabT* steps = (const TabT*)(c == 0 ? P.steps[0] : P.steps[1]);
-    if (tid < kKeyWords) rk[tid] = round_key_word(P.seed + (uint64_t)r, tid);
-    for (int u = tid; u < n_units; u += nt) {
-        Real v[NU];
-        VecN<Real, NU>::ldg(xlg + (size_t)NU * u, v);
-        VecN<Real, NU>::st(S + (size_t)NU * u, v);
-    }
+    if (tid < rb * kKeyWords) rk[tid / kKeyWords][tid % kKeyWords] = round_key_word(P.seed + (uint64_t)(r + tid / kKeyWords), tid % kKeyWords);
     __syncthreads();
 
     for (int c0 = sg.p0; c0 < own1; c0 += chunk) {
@@ -238,42 +235,55 @@ __global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SamplePar
         for (int idx = tid; idx < nk * n_units; idx += nt) {
             const int k = idx / n_units, u = idx - k * n_units;
             if (c0 + k == sg.p0) continue;  // the segment's left end: its state is the anchor's
-            Real* w = NZ + (size_t)idx * UV;
             const TabT* tb = steps + (size_t)(c0 + k) * mp * ROW;
             if constexpr (STAGE) {
                 Real t[G][ROW];
                 band_rows<Real, TabT, M>(tb, u, t);
 #pragma unroll
-                for (int g = 0; g < G; ++g) VecN<Real, ROW>::st(w + NU + g * ROW, t[g]);
+                for (int g = 0; g < G; ++g) VecN<Real, ROW>::st(RW + (size_t)idx * RV + g * ROW, t[g]);
             }
             if (u == 0) {
                 Real tn[ROW];
                 load_row<Real, TabT, ROW>(tb + (size_t)Nc * ROW, tn);
                 VecN<Real, ROW>::st(NY + (size_t)k * ROW, tn);
             }
-            Real nr[NU];
-            unit_normals_rk<Real, NC>(rk, (uint32_t)u, (uint32_t)(ring0 + dir * k), nr);
-            VecN<Real, NU>::st(w, nr);
+#pragma unroll 1
+            for (int z = 0; z < nr; ++z) {
+                Real xi[NU];
+                unit_normals_rk<Real, NC>(rk[z], (uint32_t)u, (uint32_t)(ring0 + dir * k), xi);
+                VecN<Real, NU>::st(NZ + ((size_t)z * cn + idx) * NU, xi);
+            }
+        }
+        if (c0 == sg.p0) {
+            // the anchors' states, the first values of the launch before this one
+            wait_launch();
+            for (int idx = tid; idx < nr * n_units; idx += nt) {
+                const int z = idx / n_units, u = idx - z * n_units;
+                Real v[NU];
+                VecN<Real, NU>::ldcg(xlg + z * anc_r + (size_t)NU * u, v);
+                VecN<Real, NU>::st(S + (size_t)NU * idx, v);
+            }
         }
         __syncthreads();
         if constexpr (STAGE) {
             // one thread per real chain f (slot f / 2, Re or Im): a small grid has few units, and in
             // FP64 a warp's multiply-add holds the SM's two lanes for 16 cycles
-            for (int f = tid; f < 2 * Nc; f += nt) {
+            for (int zf = tid; zf < nr * 2 * Nc; zf += nt) {
+                const int z = zf / (2 * Nc), f = zf - z * 2 * Nc;
                 const int u = f / (2 * G), in_unit = f - u * 2 * G;
                 Real x[M], xr[M];
 #pragma unroll
                 for (int q = 0; q < M; ++q) {
-                    x[q] = S[(size_t)f * M + q];
-                    xr[q] = has_right ? __ldg(xrg + (size_t)f * M + q) : (Real)0;
+                    x[q] = S[(size_t)zf * M + q];
+                    xr[q] = has_right ? __ldcg(xrg + z * anc_r + (size_t)f * M + q) : (Real)0;
                 }
 #pragma unroll 2
                 for (int k = 0; k < nk; ++k) {
                     const int pos = c0 + k;
                     if (pos > sg.p0) {
-                        const Real* w = NZ + ((size_t)k * n_units + u) * UV;
+                        const Real* w = NZ + ((size_t)z * cn + (size_t)k * n_units + u) * NU;
                         // chain 1 is the Nyquist mode's (its own table row)
-                        const Real* row = f == 1 ? NY + (size_t)k * ROW : w + NU + (in_unit >> 1) * ROW;
+                        const Real* row = f == 1 ? NY + (size_t)k * ROW : RW + ((size_t)k * n_units + u) * RV + (in_unit >> 1) * ROW;
                         Real t[ROW], xi[M];
                         VecN<Real, ROW>::ld(row, t);
 #pragma unroll
@@ -281,24 +291,24 @@ __global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SamplePar
                         if (has_right) step_state<Real, M, true>(t, x, xi, xr);
                         else step_state<Real, M, false>(t, x, xi, nullptr);
                     }
-                    if (pos >= own0) reinterpret_cast<Real*>(X)[(size_t)k * 2 * Nc + f] = x[0];
+                    if (pos >= own0) reinterpret_cast<Real*>(X)[((size_t)z * chunk + k) * 2 * Nc + f] = x[0];
                 }
 #pragma unroll
-                for (int q = 0; q < M; ++q) S[(size_t)f * M + q] = x[q];
+                for (int q = 0; q < M; ++q) S[(size_t)zf * M + q] = x[q];
             }
         } else {
             for (int u = tid; u < n_units; u += nt) {
                 Real x[NU], xr[NU];
                 VecN<Real, NU>::ld(S + (size_t)NU * u, x);
-                if (has_right) VecN<Real, NU>::ldg(xrg + (size_t)NU * u, xr);
+                if (has_right) VecN<Real, NU>::ldcg(xrg + (size_t)NU * u, xr);
 #pragma unroll 2
                 for (int k = 0; k < nk; ++k) {
                     const int pos = c0 + k;
                     if (pos > sg.p0) {
-                        Real nr[NU], t[G][ROW];
-                        VecN<Real, NU>::ld(NZ + ((size_t)k * n_units + u) * UV, nr);
+                        Real xi[NU], t[G][ROW];
+                        VecN<Real, NU>::ld(NZ + ((size_t)k * n_units + u) * NU, xi);
                         band_rows<Real, TabT, M>(steps + (size_t)pos * mp * ROW, u, t);
-                        band_step<Real, M>(t, NY + (size_t)k * ROW, u == 0, has_right, nr, xr, x);
+                        band_step<Real, M>(t, NY + (size_t)k * ROW, u == 0, has_right, xi, xr, x);
                     }
                     if (pos >= own0) put_unit<C, Real, M>(X + (size_t)k * Nc, u, x);
                 }
@@ -331,6 +341,29 @@ __global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SamplePar
                                        (C*)((Real*)P.out + (size_t)r * P.ring_total + P.ring_off[ring]), tid - g * gs, gs, g);
             }
             __syncthreads();
+        }
+        if constexpr (sizeof(Real) == 8) {
+            if (rb > 1) {
+                // every realisation's rings of this chunk together (none are ring-dependent); chunks that
+                // begin before this CTA's share hold rings to skip, so each realisation's rings move up
+                C* base = (C*)((Real*)P.out + ((size_t)r * P.n_theta + ring0 + dir * k0) * (size_t)P.n_phi);
+                const int per = nk - k0;
+                if (per < chunk) {
+                    for (int z = 0; z < nr; ++z) {
+                        for (int i = tid; i < per * Nc; i += nt) {
+                            const C v = X[((size_t)z * chunk + k0) * Nc + i];
+                            W[(size_t)z * per * Nc + i] = v;
+                        }
+                    }
+                    __syncthreads();
+                    for (int i = tid; i < nr * per * Nc; i += nt) X[i] = W[i];
+                    __syncthreads();
+                }
+                grp_fx_c2r(X, W, nr * per, P.lgNc, (const int4*)P.twx, (const int4*)P.prex,
+                           RingOut2<C>{base, (size_t)((long long)dir * Nc), (size_t)P.n_theta * Nc, per}, fxred, tid, nt, kBarFft);
+                __syncthreads();
+                continue;
+            }
         }
         for (int k = k0; k < nk;) {
             // a run of whole rings: their FFTs together

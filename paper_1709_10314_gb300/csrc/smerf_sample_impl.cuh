@@ -402,10 +402,19 @@ __device__ __forceinline__ void anchor_body(const SampleParams& P, int u, int r,
     (void)T;
 }
 
+// Programmatic dependent launch: a kernel launched with the attribute (launch_band) may start once
+// every CTA of the launch before it has called early_launch; it reads what that launch writes only
+// after wait_launch.  Without the attribute neither has an effect.  64 x 128, p = 1, one FP64
+// realisation: 30.7 -> 26.2 us in Alg. 2's order, 24.6 -> 17.8 us anchored (the launch's latency and
+// the first chunk's noise behind the anchors).
+__device__ __forceinline__ void early_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // one thread per (chain c, realisation r, unit u)
 template <class Real, class TabT, int M>
 __global__ void __launch_bounds__(128, anchor_minb(sizeof(Real), M)) anchor_kernel(SampleParams P)
 {
+    early_launch();
     NoStage h;
     anchor_body<Real, TabT, M>(P, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y, blockIdx.z, h);
 }
@@ -443,6 +452,7 @@ __global__ void __launch_bounds__(tile_threads(M)) anchor_tile_kernel(SamplePara
 {
     constexpr int G = kG<M>, Ec = coarse_elems(M), NU = unit_vals(M), NC = unit_calls(M);
     constexpr int CH = tile_anchors(M), AD = tile_ahead(M);
+    early_launch();
     __shared__ Real nz[2][CH][NU][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int u = blockIdx.x * 32 + lane, r = blockIdx.y, c = blockIdx.z;
@@ -548,6 +558,14 @@ template <class C> struct RingOut {
     size_t stride;
     bool wide = true;
     __device__ __forceinline__ C* operator[](int r) const { return base + (size_t)r * stride; }
+};
+
+// The same for `per` rings each of several realisations
+template <class C> struct RingOut2 {
+    C* base;
+    size_t stride, stride2;
+    int per;
+    __device__ __forceinline__ C* operator[](int r) const { return base + (size_t)(r % per) * stride + (size_t)(r / per) * stride2; }
 };
 
 template <class C>
@@ -1120,7 +1138,7 @@ __device__ __forceinline__ fxc fxc_mul(fxc a, int4 w)
     return r;
 }
 
-constexpr int kFxRings = 16;  // rings of one call (the band kernel's chunk)
+constexpr int kFxRings = 32;  // rings of one call (the band kernel: two realisations' chunks of up to 16)
 
 // scale of ring r from its largest exponent and its sum of magnitudes (units of 2^(e - 16))
 __device__ __forceinline__ int fx_scale(const int* red, int r)
@@ -1133,7 +1151,7 @@ __device__ __forceinline__ void grp_fx_scales(const double2* buf, int R, int lgN
 {
     const int total = R << lgNc;
     const bool whole = lgNc >= 5;  // a warp's 32 neighbouring elements lie in one ring
-    if (ftid < R) red[ftid] = red[kFxRings + ftid] = 0;
+    for (int r = ftid; r < R; r += nf) red[r] = red[kFxRings + r] = 0;
     bar_sync(bar, nf);
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
@@ -1172,9 +1190,9 @@ __device__ __forceinline__ void grp_fx_scales(const double2* buf, int R, int lgN
 
 // C2R FFTs of R rings (coefficients in buf0 as double2, buf1 the second buffer), radix-4 passes
 // (radix 2 last when log2 Nc is odd); prex, twx: the plan's factors as int4; red: 2 kFxRings words
+template <class Out>
 __device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, int lgNc, const int4* __restrict__ twx,
-                                           const int4* __restrict__ prex, RingOut<double2> gout, int* red, int ftid,
-                                           int nf, int bar)
+                                           const int4* __restrict__ prex, Out gout, int* red, int ftid, int nf, int bar)
 {
     const int Nc = 1 << lgNc;
     grp_fx_scales(buf0, R, lgNc, red, ftid, nf, bar);
@@ -1862,6 +1880,7 @@ struct SegConfig {
     size_t smem;
     int ring, radix;
     int band_splits, band_chunk;  // > 0: the band kernel, so many CTAs per segment, rings per chunk
+    int band_rb;                  // realisations per CTA
     bool band_stage;
     size_t band_smem;
 };
@@ -1979,8 +1998,10 @@ inline bool seg_choice(const smerf_plan* pl, int n, int& upt, int& rmax, int& nf
     rmax = 1;
     minb = 1;
     if (sizeof(Real) == 8) {
-        // the FP64 pipe is the limit: half the producers leave it to more FFT threads
-        if (M == 1 && units >= 128 && units <= 512) { upt = 2; nf = units / 2 < 128 ? units / 2 : 128; return true; }
+        // a call of one wave wants the general rule's many threads
+        if (waves(ctas, 1) < 2) return false;
+        if (M == 1 && units == 64) { upt = 1; nf = 64; return true; }
+        if (M == 1 && units >= 256 && units <= 512) { upt = 2; nf = 128; return true; }
         if (M == 2 && units >= 256 && units <= 512) { upt = 2; nf = units / 4; return true; }
         if (M == 2 && units == 1024) { upt = 4; nf = 128; return true; }
         if (M == 3 && units == 256) { upt = 2; nf = 64; return true; }
@@ -2114,19 +2135,26 @@ inline void band_config(const smerf_plan* pl, int n, SegConfig& cfg)
     const int seg_len = pl->H > 0 ? pl->H : (pl->chain[0].len > pl->chain[1].len ? pl->chain[0].len : pl->chain[1].len) + 1;
     long long splits = ctas > 0 && ctas < 152 ? 152 / ctas : 1;  // one CTA per SM
     if (splits > seg_len) splits = seg_len;
+    // FP64, rings of up to 64 points, many CTAs: two realisations per CTA, so that the recursion
+    // has twice the chains for its threads and the staged table rows serve both (20001 realisations of
+    // 32 x 64, p = 2: 2588 -> 2010 us with two, 2028 with four)
+    const int rb = sizeof(Real) == 8 && !rings && ctas >= 1024 && 4 * Nc <= kBandThreads ? 2 : 1;
     auto smem = [&](int chunk, bool stage) {
-        return M == 1 ? (stage ? band_smem<Real, 1, true>(Nc, chunk, rings) : band_smem<Real, 1, false>(Nc, chunk, rings))
-             : M == 2 ? (stage ? band_smem<Real, 2, true>(Nc, chunk, rings) : band_smem<Real, 2, false>(Nc, chunk, rings))
-                      : (stage ? band_smem<Real, 3, true>(Nc, chunk, rings) : band_smem<Real, 3, false>(Nc, chunk, rings));
+        return M == 1 ? (stage ? band_smem<Real, 1, true>(Nc, chunk, rb, rings) : band_smem<Real, 1, false>(Nc, chunk, rb, rings))
+             : M == 2 ? (stage ? band_smem<Real, 2, true>(Nc, chunk, rb, rings) : band_smem<Real, 2, false>(Nc, chunk, rb, rings))
+                      : (stage ? band_smem<Real, 3, true>(Nc, chunk, rb, rings) : band_smem<Real, 3, false>(Nc, chunk, rb, rings));
     };
     size_t budget = ctas * splits <= 152 ? kMaxSmem : kMaxSmem / 2;
-    bool stage = Nc / unit_slots(M) <= 128 && smem(4, true) <= budget;
+    // the rows of a chunk through shared memory while the recursion's latency is what counts: for few
+    // units, or few CTAs (Nside 128, 16 realisations: 137 us with, 115 us without)
+    bool stage = Nc / unit_slots(M) <= (ctas < 152 && !rings ? 128 : 64) && smem(4, true) <= budget;
     if (smem(1, stage) > budget) budget = kMaxSmem;
     if (smem(1, stage) > budget) return;
     int chunk = 1;
     while (chunk < 16 && chunk < seg_len && smem(chunk + 1, stage) <= budget) ++chunk;
     cfg.band_splits = (int)splits;
     cfg.band_chunk = chunk;
+    cfg.band_rb = stage ? rb : 1;
     cfg.band_stage = stage;
     cfg.band_smem = smem(chunk, stage);
 }
@@ -2136,9 +2164,19 @@ int launch_band(const SampleParams& P, int n_segments, const SegConfig& cfg, cud
 {
     auto kern = cfg.band_stage ? segment_band_kernel<Real, TabT, M, true> : segment_band_kernel<Real, TabT, M, false>;
     if (set_smem_attr(kern, cfg.band_smem) != cudaSuccess) return SMERF_ECUDA;
-    dim3 grid(cfg.band_splits, P.n_samples, n_segments);
-    kern<<<grid, kBandThreads, cfg.band_smem, st>>>(P, cfg.band_chunk);
-    return cudaGetLastError() == cudaSuccess ? SMERF_OK : SMERF_ECUDA;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(cfg.band_splits, (P.n_samples + cfg.band_rb - 1) / cfg.band_rb, n_segments);
+    lc.blockDim = dim3(kBandThreads);
+    lc.dynamicSmemBytes = cfg.band_smem;
+    lc.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    // early start only while every CTA of both launches fits the GPU: beyond that the waiting CTAs
+    // would hold slots that the anchors' want (Nside 128, 16 realisations: 119 us without, 123 with)
+    lc.attrs = &at;
+    lc.numAttrs = (long long)lc.gridDim.x * lc.gridDim.y * lc.gridDim.z <= 304 ? 1 : 0;
+    return cudaLaunchKernelEx(&lc, kern, P, cfg.band_chunk, cfg.band_rb) == cudaSuccess ? SMERF_OK : SMERF_ECUDA;
 }
 
 template <class Real, class TabT, int M>

@@ -26,6 +26,9 @@ KAPPA = {1: (9.0,), 2: (6.0, 15.0), 3: (6.0, 11.0, 25.0)}
     (3, 40, 64, 4, 3),
     (3, 27, 256, 5, 1),
     (1, 34, 2048, 16, 40),    # FP32: the longest ring the band kernel takes
+    (2, 33, 64, 5, 401),      # FP64: two realisations per CTA, an odd count of them, chunks that end mid-segment
+    (1, 20, 32, 0, 1025),
+    (3, 24, 64, 6, 257),
 ])
 def test_same_field_as_the_batch_kernels(fp64, p, n_theta, n_phi, H, n):
     import torch
