@@ -19,8 +19,8 @@
 // (4, 2, then the odd primes), one output point per thread from r terms with the roots of unity
 // from a table of the ring's own, a group of threads per ring.  HEALPix's polar rings (4i points)
 // took O(n^2) terms in the FFT warps of one CTA per segment before: Nside 128, 16 realisations,
-// 4266 -> 119 us a call.  One FP64 realisation of 64 x 128 in Alg. 2's order: 166 -> 26 us; one of
-// 181 x 512, p = 2: 31.1 -> 22.4 us (the anchor tiles among them).
+// 4266 -> 119 us a call.  One FP64 realisation of 64 x 128 in Alg. 2's order: 166 -> 26.6 us (the
+// fixed-point FFT among them); one of 181 x 512, p = 2: 31.1 -> 22.7 us (the anchor tiles among them).
 #pragma once
 
 namespace smerf {

@@ -207,7 +207,8 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, PhiloxKey key)
 // denormals around the instruction (about 6 instructions per pair).  With the round keys read two
 // rounds at a time (round_key_word): 1024 x 2048, 64 realisations, p = 2 834 -> 756 us a call,
 // p = 3 2086 -> 1759 us; 4096 x 8192, 16 realisations, p = 1 1990 -> 1877 us; 16384 x 32768, 4
-// realisations 6603 -> 6417 us; the same fields bit for bit.
+// realisations 6603 -> 6417 us; the same fields bit for bit (the first two are 645 and 1441 us with
+// seg_choice's launches).
 __device__ __forceinline__ float lg2_ftz(float x) { float y; asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float rsqrt_ftz(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 

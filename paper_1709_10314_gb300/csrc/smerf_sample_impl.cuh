@@ -864,10 +864,19 @@ __device__ __forceinline__ uint4 philox_rk(uint4 c, const uint4* rk)
     return c;
 }
 
+// Box-Muller out of line (see ws_body)
+template <class Real>
+__device__ __noinline__ cplx<Real> box_muller_call(uint32_t a, uint32_t b)
+{
+    cplx<Real> r;
+    box_muller(a, b, r.x, r.y);
+    return r;
+}
+
 // The normals of one Philox call for NB realisations at once (round keys rk[0..NB)): the NB
 // generator chains are independent and run interleaved; the first round's products, which
 // depend on the counter only, are shared.
-template <class Real, int NB, int NC = 1>
+template <class Real, int NB, int NC, bool CALL>
 __device__ __forceinline__ void unit_normals_multi(const uint4 (*rk)[kKeyWords], uint32_t u, uint32_t ring, Real (&n)[NB][4 * NC])
 {
 #pragma unroll
@@ -885,8 +894,16 @@ __device__ __forceinline__ void unit_normals_multi(const uint4 (*rk)[kKeyWords],
         }
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
-            box_muller(c[b].x, c[b].y, n[b][4 * j], n[b][4 * j + 1]);
-            box_muller(c[b].z, c[b].w, n[b][4 * j + 2], n[b][4 * j + 3]);
+            if constexpr (CALL) {
+                const cplx<Real> v = box_muller_call<Real>(c[b].x, c[b].y), w = box_muller_call<Real>(c[b].z, c[b].w);
+                n[b][4 * j] = v.x;
+                n[b][4 * j + 1] = v.y;
+                n[b][4 * j + 2] = w.x;
+                n[b][4 * j + 3] = w.y;
+            } else {
+                box_muller(c[b].x, c[b].y, n[b][4 * j], n[b][4 * j + 1]);
+                box_muller(c[b].z, c[b].w, n[b][4 * j + 2], n[b][4 * j + 3]);
+            }
         }
     }
 }
@@ -1123,8 +1140,9 @@ __device__ __forceinline__ void grp_c2r_rt(C* buf0, C* buf1, int R, int lgNc, co
 // count.  Values then keep 2^-60 of that sum, so that a field's error against 64-bit references is
 // not above the FP64 FFT's (3.3e-15 -> 3.1e-15 at 64 x 128, 3.9e-15 -> 3.5e-15 at 32 x 64, 1.3e-13 ->
 // 1.0e-13 and 8.6e-13 -> 5.1e-13 on larger grids, the tables' own error).  1024 x 2048, p = 2, 16
-// realisations: 2161 -> 1393 us; 20001 of 32 x 64: 3057 -> 2523 us.  Factors e^{2 pi i k / n} are exact to 2^-62, stored as two words
-// per component (int4: Re hi, lo, Im hi, lo).
+// realisations: 2161 -> 1393 us (1323 with box_muller_call); 20001 of 32 x 64: 3057 -> 2523 us (2010 with two realisations per
+// CTA, band_config).  Factors e^{2 pi i k / n} are exact to 2^-62, stored as two words per component
+// (int4: Re hi, lo, Im hi, lo).
 using fxc = longlong2;
 
 __device__ __forceinline__ fxc fxc_mul(fxc a, int4 w)
@@ -1439,6 +1457,10 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
     constexpr int G = kG<M>;
     constexpr int ROW = step_row(M);
     constexpr int RB = RMAX < SMERF_RB ? RMAX : SMERF_RB;  // realisations whose noise is drawn together
+    // FP64 Box-Muller as a call where a thread's units repeat it most (instruction fetch stalls 1.08 of
+    // 10 cycles per issue): 1024 x 2048, p = 2, 16 realisations 1394 -> 1323 us; inline elsewhere (p = 2
+    // with 2 units per thread 398 and 405 us with the call, p = 3 with 4 units 2800 and 2973)
+    constexpr bool CALL = sizeof(Real) == 8 && M == 2 && UPT == 4;
     constexpr int NU = unit_vals(M), NC = unit_calls(M);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint4 rk[RMAX][kKeyWords];
@@ -1512,7 +1534,7 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
                         // 24-value table row at a time, so that two rows are never live together
                         static_assert(RMAX == 1, "p = 3 builds hold one realisation per CTA");
                         Real nr[NU];
-                        unit_normals_multi<Real, 1, NC>(rk, (uint32_t)u, (uint32_t)ring, *reinterpret_cast<Real(*)[1][NU]>(nr));
+                        unit_normals_multi<Real, 1, NC, CALL>(rk, (uint32_t)u, (uint32_t)ring, *reinterpret_cast<Real(*)[1][NU]>(nr));
 #pragma unroll
                         for (int g = 0; g < G; ++g) {
                             Real tg[ROW];
@@ -1549,7 +1571,7 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
                         if (rb >= R) continue;
                         // normals of realisations rb .. rb + RB - 1 (those past R are not used)
                         Real nrb[RB][NU];
-                        unit_normals_multi<Real, RB, NC>(rk + rb, (uint32_t)u, (uint32_t)ring, nrb);
+                        unit_normals_multi<Real, RB, NC, CALL>(rk + rb, (uint32_t)u, (uint32_t)ring, nrb);
 #pragma unroll
                     for (int r = rb; r < rb + RB; ++r) {
                         if (r >= R) continue;
