@@ -40,12 +40,20 @@ def alg_ops_per_item(p, Nc, fp64=False):
     rsqrt, product, sin, cos, 2 products), the recursion x = A x + B xi on the Re and Im
     chains (Eq. (state_space)), and this item's share of the ring's C2R FFT (10 for the
     packing, 3.5 log2 Nc for a radix-4 complex FFT).  With fp64 only the floating-point part
-    (Box-Muller, recursion, FFT), which runs on the FP64 pipe."""
+    (Box-Muller, recursion, FFT)."""
     philox = 40.0 * (2 * p) / 4.0
     box_muller = 12.0 * p
     recursion = 2.0 * (p * p + p * (p + 1) / 2.0)
     fft = 10.0 + 3.5 * math.log2(Nc)
     return (box_muller + recursion + fft) if fp64 else (philox + box_muller + recursion + fft)
+
+
+def fp64_pipe_ops_per_item(p, Nc):
+    """The operations of an item that the FP64 recursion mode leaves on the FP64 pipe: the
+    recursion; the noise is formed in 64-bit fixed point on the integer lanes, and so is the FFT
+    of rings up to 2048 complex points (the in-place kernel's longer rings keep FP64 FFTs)."""
+    recursion = 2.0 * (p * p + p * (p + 1) / 2.0)
+    return recursion + (10.0 + 3.5 * math.log2(Nc) if Nc > 2048 else 0.0)
 
 
 def sfu_ops_per_item(p):
@@ -352,7 +360,8 @@ def run_gb300(args, rank, world, local_rank):
         points = n * cfg["n_theta"] * cfg["n_phi"]
         out_bytes = points * (8 if recur == "fp64" else 4)
         fp64_alu = recur == "fp64"
-        alg_ops = n * cfg["n_theta"] * (cfg["n_phi"] // 2) * alg_ops_per_item(len(cfg["kappa"]), cfg["n_phi"] // 2, fp64_alu)
+        item_ops = fp64_pipe_ops_per_item if fp64_alu else alg_ops_per_item
+        alg_ops = n * cfg["n_theta"] * (cfg["n_phi"] // 2) * item_ops(len(cfg["kappa"]), cfg["n_phi"] // 2)
         table_bytes = info["table_bytes"]
         # what the segment kernel reads: the step tables and the anchor states
         seg_read_bytes = info["step_table_bytes"], n * info["scratch_bytes_per_sample"]
@@ -403,7 +412,7 @@ def run_gb300(args, rank, world, local_rank):
         seg_ms = sum(a.elapsed_time(b) for a, b in zip(s0, s1)) / args.steps
         ring = (not ws_kernel) and len(FIXED[wl]["kappa"]) == 1 and (args.recur or FIXED[wl]["recur"]) == "fp32" \
             and FIXED[wl]["n_phi"] in (16384, 32768)
-        kernel = "segment_ws_kernel" if ws_kernel else ("ring_kernel" if ring else "segment_kernel")
+        kernel = "segment_ws_kernel (small requests: segment_band_kernel)" if ws_kernel else ("ring_kernel" if ring else "segment_kernel")
     else:
         seg_ms = step_ms  # the graph replay: all groups' anchor + segment launches
         kernel = "batched graph replay (anchor + segment launches of every group)"

@@ -184,15 +184,17 @@ int smerf_last_device_status(void* stream);
  * take their temporary device memory (anchor states, FP32 copies of FP64 tables, the field on
  * the host path) stream-ordered from that pool, which keeps it between calls so that a call
  * after a synchronisation maps no new memory; the pool holds at most the largest amount that
- * calls in flight used together.  SMERF_OK, or SMERF_ECUDA.
+ * calls in flight used together.  Plan creation takes temporaries of up to 128 MB from the same
+ * pool.  SMERF_OK, or SMERF_ECUDA.
  */
 int smerf_scratch_trim(void);
 
 /*
  * smerf_sample_launches -- how many kernels one smerf_sample(plan, ., n_samples, ...) call
  * launches on its stream: the anchor kernel and the segment kernel, and, when the plan keeps
- * FP64 tables, recurses in FP32 and n_samples >= 4, one short conversion of the coarse and
- * start tables to FP32 ahead of them (the anchor kernel's threads convert the step tables).
+ * FP64 tables, recurses in FP32 and n_samples >= 4, one conversion to FP32 ahead of them (of the
+ * coarse and start tables when the anchor kernel's threads convert the step tables; of all
+ * tables in small requests, whose anchors run in tiles).
  * 0 for n_samples == 0; SMERF_EINVAL (negative) for a NULL plan or a negative count.
  */
 int smerf_sample_launches(const smerf_plan* plan, int n_samples);
@@ -345,15 +347,15 @@ int smerf_plan_info(const smerf_plan* plan, smerf_plan_info_t* info);
  * remark that the method holds on any iso-latitude grid; HEALPix rings with the colatitudes of
  * smerf_plan_create_theta).  Ring k keeps its colatitude theta_k and holds n_phi_ring[k] points
  * phi = phi0_ring[k] + 2 pi j / n_phi_ring[k], j < n_phi_ring[k]; each n_phi_ring[k] even with
- * 4 <= n_phi_ring[k] <= n_phi of the plan (a power of two takes a radix-4 FFT, other counts a
- * direct synthesis, O(n_phi_ring[k]^2) per ring); phi0_ring may be NULL (no offsets).  Host
+ * 4 <= n_phi_ring[k] <= n_phi of the plan (each takes a mixed-radix FFT over the prime factors of
+ * n_phi_ring[k] / 2, O(r) per point and factor r); phi0_ring may be NULL (no offsets).  Host
  * arrays of n_theta values.  The modes
  * m = 0..n_phi/2, their recursion and noise stay those of the plan; each ring's values are the
  * m-truncated field evaluated at its points: T(phi) = g_0 + 2 sum_{0<m<n_phi/2} Re(g_m e^{i m phi})
  * + Re(g_{n_phi/2}) cos(n_phi phi / 2), so modes above the ring's own Nyquist alias onto it.
  * Output of a sample call: realisation r's rings back to back, ring k at
  * r * P + sum_{k'<k} n_phi_ring[k'] (P = smerf_plan_info's points_per_sample).  Only plans run by
- * the warp-specialised kernels (n_phi <= 8192 with FP32 recursion, <= 4096 with FP64) take rings
+ * the band and warp-specialised kernels (n_phi <= 8192 with FP32 recursion, <= 4096 with FP64) take rings
  * (else SMERF_EUNSUPPORTED); in a batch such a plan's request is launched individually.
  * n_phi_ring = NULL restores the full grid.  Host only, synchronous; must not run while other
  * calls use the plan, nor while a batch made with the plan exists (a batch takes each plan's
@@ -403,7 +405,9 @@ int smerf_plan_launch_candidates(const smerf_plan* plan, int* cand, int max_n);
 /*
  * smerf_plan_set_launch -- fix the segment-kernel launch configuration (SMERF_LAUNCH_INTS
  * integers) to one of the candidates (e.g. a choice smerf_plan_autotune made in an earlier
- * process), or with config == NULL return to the built-in choice (radix plan 16 in FP32).
+ * process), or with config == NULL return to the built-in choice, which depends on n_samples
+ * (radix plan 16 in FP32).  Small requests and plans with ring-dependent longitudes run on the
+ * band kernel, which takes only the radix plan from it.
  * SMERF_EINVAL if config is not a candidate.  Host only.
  */
 int smerf_plan_set_launch(smerf_plan* plan, const int* config);
