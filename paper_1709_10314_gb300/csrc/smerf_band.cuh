@@ -19,13 +19,14 @@
 // (4, 2, then the odd primes), one output point per thread from r terms with the roots of unity
 // from a table of the ring's own, a group of threads per ring.  HEALPix's polar rings (4i points)
 // took O(n^2) terms in the FFT warps of one CTA per segment before: Nside 128, 16 realisations,
-// 4266 -> 119 us a call.  One FP64 realisation of 64 x 128 in Alg. 2's order: 166 -> 26.6 us (the
+// 4266 -> 119 us a call.  One FP64 realisation of 64 x 128 in Alg. 2's order: 166 -> 24.6 us (the
 // fixed-point FFT among them); one of 181 x 512, p = 2: 31.1 -> 22.7 us (the anchor tiles among them).
 #pragma once
 
 namespace smerf {
 
-constexpr int kBandThreads = 256;
+constexpr int kBandThreads = 256;      // two CTAs per SM
+constexpr int kBandThreadsFew = 512;   // requests of at most one CTA per SM (band_config)
 
 // e^{2 pi i p}, p = ph 2^-64 turns
 template <class Real> __device__ __forceinline__ cplx<Real> cis_turns(uint64_t ph)
@@ -190,8 +191,8 @@ __host__ __device__ inline size_t band_smem(int Nc, int chunk, int rb, bool ring
 // grid (splits, realisations / rb, segments)
 // STAGE: the chunk's table rows go through shared memory, loaded in part 1 beside the noise by
 // every thread, so that the recursion waits for no global load
-template <class Real, class TabT, int M, bool STAGE>
-__global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SampleParams P, int chunk, int rb)
+template <class Real, class TabT, int M, bool STAGE, int NT>
+__global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_kernel(SampleParams P, int chunk, int rb)
 {
     using C = cplx<Real>;
     constexpr int G = kG<M>, ROW = step_row(M), NU = unit_vals(M), NC = unit_calls(M);
@@ -203,7 +204,9 @@ __global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SamplePar
 
     const Segment sg = P.segs[blockIdx.z];
     const int r = blockIdx.y * rb, c = sg.chain, nr = min(rb, P.n_samples - r);  // realisations r .. r + nr - 1
-    const int tid = threadIdx.x, nt = kBandThreads;
+    constexpr int nt = NT;
+    const bool rings = NT == kBandThreads && P.ring_n;  // the ragged rings' groups are of kBandThreads
+    const int tid = threadIdx.x;
     const int Nc = P.Nc, n_units = P.n_units;
     const size_t mp = P.n_modes_pad;
     const bool has_right = sg.right >= 0;
@@ -318,7 +321,7 @@ __global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SamplePar
         __syncthreads();
         const int k0 = max(0, own0 - c0);
         if (k0 >= nk) continue;  // nothing of this chunk is this CTA's (NZ is rewritten: no reader is left)
-        if (P.ring_n) {
+        if (rings) {
             // whole rings with an offset become whole rings without one; rings of their own
             // point count are synthesised by the thread groups
             const int gs = band_group(Nc), g = tid / gs, groups = nt / gs;
@@ -370,7 +373,7 @@ __global__ void __launch_bounds__(kBandThreads, 2) segment_band_kernel(SamplePar
             int e = nk;
             const int ring = ring0 + dir * k;
             C* base = (C*)((Real*)P.out + ((size_t)r * P.n_theta + ring) * (size_t)P.n_phi);
-            if (P.ring_n) {
+            if (rings) {
                 if (P.ring_n[ring] != P.n_phi) {
                     ++k;
                     continue;

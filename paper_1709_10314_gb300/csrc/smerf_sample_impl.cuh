@@ -405,7 +405,7 @@ __device__ __forceinline__ void anchor_body(const SampleParams& P, int u, int r,
 // Programmatic dependent launch: a kernel launched with the attribute (launch_band) may start once
 // every CTA of the launch before it has called early_launch; it reads what that launch writes only
 // after wait_launch.  Without the attribute neither has an effect.  64 x 128, p = 1, one FP64
-// realisation: 30.7 -> 26.2 us in Alg. 2's order, 24.6 -> 17.8 us anchored (the launch's latency and
+// realisation, 256-thread CTAs: 30.7 -> 26.2 us in Alg. 2's order, 24.6 -> 17.8 us anchored (the launch's latency and
 // the first chunk's noise behind the anchors).
 __device__ __forceinline__ void early_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -1903,6 +1903,7 @@ struct SegConfig {
     int ring, radix;
     int band_splits, band_chunk;  // > 0: the band kernel, so many CTAs per segment, rings per chunk
     int band_rb;                  // realisations per CTA
+    int band_threads;             // threads per CTA
     bool band_stage;
     size_t band_smem;
 };
@@ -2139,9 +2140,12 @@ inline SegConfig seg_config(const smerf_plan* pl, int n)
 // timed over n_phi 128 to 8192, p = 1 .. 3, FP32 and FP64, 1 to 256 realisations, Alg. 2's and the
 // anchored order.  In FP32 the band kernel wins while its CTAs fit the GPU two per SM (1.1 to 2.5
 // times; up to 3.7 in Alg. 2's order), longer for rings so short that its CTAs are brief (64
-// points up to 1280 CTAs); from 2048 complex points on it loses at every count.  In FP64 a split
-// segment repeats its recursion on the narrow FP64 pipe, so the line lies lower, and for p = 3
-// (24-value table rows) it stops at 128 points.
+// points up to 1280 CTAs); at 2048 complex points one 2048 x 4096 realisation takes 63 us against 56
+// (p = 1) and 122 against 95 (p = 2).  In FP64 a split segment repeats its recursion on the narrow FP64
+// pipe, so the line lies lower: p = 1 at 512 points 132 CTAs 99 against 107 us, at 1024 points 65 CTAs
+// 147 against 155 us and 130 CTAs 185 against 156; p = 2 at 512 points 132 CTAs 149 against 126, at
+// 1024 points 2 CTAs 5.2 against 5.8 ms and 65 CTAs 250 against 228 us.  For p = 3 (24-value table
+// rows) it stops at 128 points.
 template <class Real>
 inline void band_config(const smerf_plan* pl, int n, SegConfig& cfg)
 {
@@ -2151,8 +2155,8 @@ inline void band_config(const smerf_plan* pl, int n, SegConfig& cfg)
     long long most;
     if (sizeof(Real) == 8 && Nc <= (M == 3 ? 32 : 64)) most = 1ll << 40;
     else if (M == 3) most = Nc <= 128 ? 20480 / Nc : 0;
-    else if (sizeof(Real) == 8) most = Nc <= 512 ? 38912 / Nc : 0;
-    else most = Nc <= 128 ? 73728 / Nc : Nc <= 512 ? 304 : Nc <= 1024 && ctas >= 100 ? 304 : 0;
+    else if (sizeof(Real) == 8) most = Nc > 1024 ? 0 : M == 1 && Nc > 256 ? 77824 / Nc : M == 2 && Nc > 512 ? 19456 / Nc : 38912 / Nc;
+    else most = Nc <= 128 ? 73728 / Nc : Nc <= 1024 ? 304 : 0;
     if (!rings && ctas > most) return;
     const int seg_len = pl->H > 0 ? pl->H : (pl->chain[0].len > pl->chain[1].len ? pl->chain[0].len : pl->chain[1].len) + 1;
     long long splits = ctas > 0 && ctas < 152 ? 152 / ctas : 1;  // one CTA per SM
@@ -2177,6 +2181,10 @@ inline void band_config(const smerf_plan* pl, int n, SegConfig& cfg)
     cfg.band_splits = (int)splits;
     cfg.band_chunk = chunk;
     cfg.band_rb = stage ? rb : 1;
+    // at most one CTA per SM: all of the SM's registers for it (181 x 512 and smaller, anchored: p = 1 14.5
+    // -> 11.5 us, p = 2 20.6 -> 16.6; 512 x 1024, p = 2: 32.9 -> 24.4, in Alg. 2's order 408 -> 259; FP64 64 x
+    // 128 in that order 26.2 -> 24.6); with p = 3's registers 128-point rings lose 8 %
+    cfg.band_threads = !rings && ctas * splits <= 152 && (M < 3 || Nc <= 64) ? kBandThreadsFew : kBandThreads;
     cfg.band_stage = stage;
     cfg.band_smem = smem(chunk, stage);
 }
@@ -2184,11 +2192,13 @@ inline void band_config(const smerf_plan* pl, int n, SegConfig& cfg)
 template <class Real, class TabT, int M>
 int launch_band(const SampleParams& P, int n_segments, const SegConfig& cfg, cudaStream_t st)
 {
-    auto kern = cfg.band_stage ? segment_band_kernel<Real, TabT, M, true> : segment_band_kernel<Real, TabT, M, false>;
+    const bool few = cfg.band_threads == kBandThreadsFew;
+    auto kern = cfg.band_stage ? (few ? segment_band_kernel<Real, TabT, M, true, kBandThreadsFew> : segment_band_kernel<Real, TabT, M, true, kBandThreads>)
+                               : (few ? segment_band_kernel<Real, TabT, M, false, kBandThreadsFew> : segment_band_kernel<Real, TabT, M, false, kBandThreads>);
     if (set_smem_attr(kern, cfg.band_smem) != cudaSuccess) return SMERF_ECUDA;
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(cfg.band_splits, (P.n_samples + cfg.band_rb - 1) / cfg.band_rb, n_segments);
-    lc.blockDim = dim3(kBandThreads);
+    lc.blockDim = dim3(cfg.band_threads);
     lc.dynamicSmemBytes = cfg.band_smem;
     lc.stream = st;
     cudaLaunchAttribute at{};

@@ -29,6 +29,9 @@ KAPPA = {1: (9.0,), 2: (6.0, 15.0), 3: (6.0, 11.0, 25.0)}
     (2, 33, 64, 5, 401),      # FP64: two realisations per CTA, an odd count of them, chunks that end mid-segment
     (1, 20, 32, 0, 1025),
     (3, 24, 64, 6, 257),
+    (1, 36, 1024, 16, 30),    # FP64, p = 1: many CTAs of 512 threads
+    (1, 20, 2048, 0, 3),      # the longest rings, few CTAs: one ring per chunk and a segment in many parts
+    (2, 33, 2048, 16, 2),
 ])
 def test_same_field_as_the_batch_kernels(fp64, p, n_theta, n_phi, H, n):
     import torch
