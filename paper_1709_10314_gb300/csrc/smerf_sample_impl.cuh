@@ -403,8 +403,10 @@ __device__ __forceinline__ void anchor_body(const SampleParams& P, int u, int r,
 }
 
 // Programmatic dependent launch: a kernel launched with the attribute (launch_band) may start once
-// every CTA of the launch before it has called early_launch; it reads what that launch writes only
-// after wait_launch.  Without the attribute neither has an effect.  64 x 128, p = 1, one FP64
+// every CTA of the launch before it has called early_launch or ended; it reads what that launch
+// writes only after wait_launch, and before it only what earlier launches wrote.  Without the
+// attribute neither has an effect.  The band kernel reads its step tables before wait_launch, so
+// the attribute is not set behind anchor_stage_kernel, which writes them.  64 x 128, p = 1, one FP64
 // realisation, 256-thread CTAs: 30.7 -> 26.2 us in Alg. 2's order, 24.6 -> 17.8 us anchored (the launch's latency and
 // the first chunk's noise behind the anchors).
 __device__ __forceinline__ void early_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -2190,7 +2192,7 @@ inline void band_config(const smerf_plan* pl, int n, SegConfig& cfg)
 }
 
 template <class Real, class TabT, int M>
-int launch_band(const SampleParams& P, int n_segments, const SegConfig& cfg, cudaStream_t st)
+int launch_band(const SampleParams& P, int n_segments, const SegConfig& cfg, cudaStream_t st, bool early)
 {
     const bool few = cfg.band_threads == kBandThreadsFew;
     auto kern = cfg.band_stage ? (few ? segment_band_kernel<Real, TabT, M, true, kBandThreadsFew> : segment_band_kernel<Real, TabT, M, true, kBandThreads>)
@@ -2204,17 +2206,19 @@ int launch_band(const SampleParams& P, int n_segments, const SegConfig& cfg, cud
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
-    // early start only while every CTA of both launches fits the GPU: beyond that the waiting CTAs
-    // would hold slots that the anchors' want (Nside 128, 16 realisations: 119 us without, 123 with)
+    // early start only behind a launch that writes nothing but the anchors' states, and while every CTA
+    // of both launches fits the GPU: beyond that the waiting CTAs would hold slots that the anchors'
+    // want (Nside 128, 16 realisations: 119 us without, 123 with)
     lc.attrs = &at;
-    lc.numAttrs = (long long)lc.gridDim.x * lc.gridDim.y * lc.gridDim.z <= 304 ? 1 : 0;
+    lc.numAttrs = early && (long long)lc.gridDim.x * lc.gridDim.y * lc.gridDim.z <= 304 ? 1 : 0;
     return cudaLaunchKernelEx(&lc, kern, P, cfg.band_chunk, cfg.band_rb) == cudaSuccess ? SMERF_OK : SMERF_ECUDA;
 }
 
+// early: the launch before this one writes the anchors' states only (see early_launch)
 template <class Real, class TabT, int M>
-int dispatch_segments(const SampleParams& P, int n_segments, const SegConfig& cfg, cudaStream_t st)
+int dispatch_segments(const SampleParams& P, int n_segments, const SegConfig& cfg, cudaStream_t st, bool early)
 {
-    if (cfg.band_splits > 0) return launch_band<Real, TabT, M>(P, n_segments, cfg, st);
+    if (cfg.band_splits > 0) return launch_band<Real, TabT, M>(P, n_segments, cfg, st, early);
     if (cfg.ws) {
         if constexpr (sizeof(Real) == 8 || M == 3) {
             if (cfg.rmax != 1 || cfg.minb != 1) return SMERF_EUNSUPPORTED;
@@ -2361,7 +2365,7 @@ int launch_sample_m(const smerf_plan* pl, uint64_t seed, int n, void* out, void*
     rc = launch_anchors<Real, TabT, M>(P, st);
     if (rc != SMERF_OK) return rc;
     if (ev0 && cudaEventRecord(ev0, st) != cudaSuccess) return SMERF_ECUDA;
-    rc = dispatch_segments<Real, TabT, M>(P, pl->n_segments, cfg, st);
+    rc = dispatch_segments<Real, TabT, M>(P, pl->n_segments, cfg, st, true);
     if (rc == SMERF_OK && ev1 && cudaEventRecord(ev1, st) != cudaSuccess) return SMERF_ECUDA;
     return rc;
 }
@@ -2431,7 +2435,7 @@ int launch_sample_staged_m(const smerf_plan* sh, const StageSmall& S, StageJob J
         rc = launch_anchors<float, float, M>(P, st);
         if (rc != SMERF_OK) return rc;
         if (ev0 && cudaEventRecord(ev0, st) != cudaSuccess) return SMERF_ECUDA;
-        rc = dispatch_segments<float, float, M>(P, sh->n_segments, cfg, st);
+        rc = dispatch_segments<float, float, M>(P, sh->n_segments, cfg, st, true);
         if (rc == SMERF_OK && ev1 && cudaEventRecord(ev1, st) != cudaSuccess) return SMERF_ECUDA;
         return rc;
     }
@@ -2458,7 +2462,7 @@ int launch_sample_staged_m(const smerf_plan* sh, const StageSmall& S, StageJob J
         if (cudaGetLastError() != cudaSuccess) return SMERF_ECUDA;
     }
     if (ev0 && cudaEventRecord(ev0, st) != cudaSuccess) return SMERF_ECUDA;
-    rc = dispatch_segments<float, float, M>(P, sh->n_segments, cfg, st);
+    rc = dispatch_segments<float, float, M>(P, sh->n_segments, cfg, st, false);  // anchor_stage_kernel wrote the step tables
     if (rc == SMERF_OK && ev1 && cudaEventRecord(ev1, st) != cudaSuccess) return SMERF_ECUDA;
     return rc;
 }
