@@ -291,6 +291,16 @@ const char* smerf_status_string(int status)
     }
 }
 
+static int tune_candidates(const smerf_plan* plan, int* cand, int max_n);
+constexpr int kMaxCand = 128;  // launch candidates a plan can have (the tuner's buffers)
+
+// whether the warp-specialised kernels hold the plan's rings
+static bool runs_on_ws(const smerf_plan* plan)
+{
+    int cand[smerf::kLaunchInts];
+    return tune_candidates(plan, cand, 1) > 0;
+}
+
 static int check_grid(int p, double A, int n_theta, int n_phi, unsigned flags, int anchor_spacing)
 {
     if (p < 1 || p > 3) return SMERF_EINVAL;
@@ -473,10 +483,14 @@ static int create_plan(const double* kappa, const double* kh_re, const double* k
     pl->flags = flags;
     pl->recur64 = (flags & SMERF_RECUR_FP64) != 0;
     pl->tab64 = (flags & SMERF_TABLES_FP64) ? true : ((flags & SMERF_TABLES_FP32) ? false : pl->recur64);
-    pl->packed = p == 1 && !pl->recur64 && !pl->tab64 && (n_phi == 16384 || n_phi == 32768);
     int H = anchor_spacing == 0 ? kDefaultAnchor : anchor_spacing;
     if ((flags & SMERF_ORDER_PAPER) || H >= n_theta) H = 0;
     pl->H = H;
+    // the ring kernel's table layout, for the plans that run on it: p = 1 in FP32 with FP32 tables at 8192
+    // or 16384 complex points.  Without anchors the warp-specialised kernel holds 8192 points too, takes
+    // such plans, and reads whole rows
+    pl->packed = p == 1 && !pl->recur64 && !pl->tab64 && (n_phi == 16384 || n_phi == 32768) &&
+                 !runs_on_ws(pl);
     pl->chain[0].len = pl->k0;
     pl->chain[1].len = n_theta - 1 - pl->k0;
     for (int c = 0; c < 2; ++c) pl->chain[c].n_anchors = H > 0 ? pl->chain[c].len / H : 0;
@@ -674,8 +688,6 @@ int smerf_plan_info(const smerf_plan* plan, smerf_plan_info_t* info)
     return SMERF_OK;
 }
 
-static int tune_candidates(const smerf_plan* plan, int* cand, int max_n);
-constexpr int kMaxCand = 128;  // launch candidates a plan can have (the tuner's buffers)
 
 int smerf_plan_set_rings(smerf_plan* plan, const int* n_phi_ring, const double* phi0_ring)
 {
@@ -701,8 +713,7 @@ int smerf_plan_set_rings(smerf_plan* plan, const int* n_phi_ring, const double* 
         off[k] = total;
         total += nk;
     }
-    int cand[smerf::kLaunchInts * kMaxCand];
-    if (tune_candidates(plan, cand, kMaxCand) == 0) return SMERF_EUNSUPPORTED;  // not a warp-specialised plan
+    if (!runs_on_ws(plan)) return SMERF_EUNSUPPORTED;
     int dev = -1;
     cudaGetDevice(&dev);
     if (dev != plan->dev) return SMERF_EINVAL;
