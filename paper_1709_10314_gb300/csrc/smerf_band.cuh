@@ -107,9 +107,15 @@ __device__ __noinline__ void band_ragged_ring(cplx<Real>* X, cplx<Real>* W, cplx
         for (int e = l; e < N; e += gs) {
             const int blk = e / Wn, w = e - blk * Wn, st = w * unit;  // w = kk + a Ns
             const C* in = src + blk * Ns + w % Ns;
-            C acc = in[0];
+            // large primes in parts of 16 terms, so that an FP32 sum rounds 16 + r / 16 times (2 x 4079
+            // points: 1.3e-6 -> 3.5e-7 of the deviation, 8e-6 -> 1.7e-6 at most)
+            C acc = in[0], sum = cmk<C>(0, 0);
             int t = st;
             for (int i = 1; i < r; ++i) {
+                if ((i & 15) == 0) {
+                    sum = cadd(sum, acc);
+                    acc = cmk<C>(0, 0);
+                }
                 const int u = 2 * t;  // root of order N: e^{2 pi i t / N} = e^{2 pi i u / n}, half a turn from t = N / 2 on
                 const C x = in[i * m], y = u < N ? RT[u] : RT[u - N];
                 const C z = cmul(x, y);
@@ -117,6 +123,7 @@ __device__ __noinline__ void band_ragged_ring(cplx<Real>* X, cplx<Real>* W, cplx
                 t += st;
                 if (t >= N) t -= N;
             }
+            acc = cadd(sum, acc);
             if (rem == 1) __stcs(gout + e, acc);
             else dst[e] = acc;
         }
