@@ -355,8 +355,9 @@ int smerf_plan_info(const smerf_plan* plan, smerf_plan_info_t* info);
  * + Re(g_{n_phi/2}) cos(n_phi phi / 2), so modes above the ring's own Nyquist alias onto it.
  * Output of a sample call: realisation r's rings back to back, ring k at
  * r * P + sum_{k'<k} n_phi_ring[k'] (P = smerf_plan_info's points_per_sample).  Only plans run by
- * the band and warp-specialised kernels (n_phi <= 8192 with FP32 recursion, <= 4096 with FP64) take rings
- * (else SMERF_EUNSUPPORTED); in a batch such a plan's request is launched individually.
+ * the band and warp-specialised kernels (n_phi <= 8192 with FP32 recursion, <= 4096 with FP64; in Alg.
+ * 2's order also 16384 with p = 1 in FP32 and 8192 with p <= 2 in FP64) take rings (else
+ * SMERF_EUNSUPPORTED); in a batch such a plan's request is launched individually.
  * n_phi_ring = NULL restores the full grid.  Host only, synchronous; must not run while other
  * calls use the plan, nor while a batch made with the plan exists (a batch takes each plan's
  * ring layout when it is created).

@@ -185,21 +185,33 @@ __host__ __device__ constexpr int band_row_reals()
 // Shared memory (cplx = 2 Real), rb realisations: X [rb][chunk][Nc] cplx; the normals [rb][chunk][units][NU]
 // Real, the same memory then the FFTs' second buffer [rb][chunk][Nc] cplx; the staged rows
 // [chunk][units][RV] Real; the states [rb][units][NU] Real; the Nyquist chain's rows [chunk][ROW] Real;
-// the root tables [groups][Nc] cplx (ring-dependent longitudes only)
+// the root tables [groups][Nc] cplx (ring-dependent longitudes only).  Where that does not fit (the
+// longest ring-dependent plans, one ring per chunk), lean = 1: the root tables lie behind the FFTs'
+// second buffer in the normals' memory (p = 2 and 3: the normals are two and three times that
+// buffer; p = 3 with 4096 complex points in FP32: 229472 bytes of 262240); lean = 2, Alg. 2's order:
+// the states stay in the anchors' scratch, whose start-ring entry of a chain and realisation
+// belongs to this CTA alone (no other segment, no splits)
+template <class Real, int M>
+__host__ __device__ inline size_t band_noise_reals(int Nc, int chunk, int rb, int lean)
+{
+    const size_t nz = (size_t)Nc / unit_slots(M) * unit_vals(M), fft = (size_t)2 * Nc * (1 + kBandThreads / band_group(Nc));
+    return lean ? (nz > fft ? nz : fft) : rb * chunk * nz;
+}
 template <class Real, int M, bool STAGE>
-__host__ __device__ inline size_t band_smem(int Nc, int chunk, int rb, bool rings)
+__host__ __device__ inline size_t band_smem(int Nc, int chunk, int rb, bool rings, int lean)
 {
     const int units = Nc / unit_slots(M);
     const size_t x = (size_t)Nc * 2 * sizeof(Real), nz = (size_t)units * unit_vals(M) * sizeof(Real);
     const size_t rows = (STAGE ? (size_t)units * band_row_reals<Real, M>() : 0) * sizeof(Real) + step_row(M) * sizeof(Real);
-    return chunk * (rb * (x + nz) + rows) + rb * nz + (rings ? (kBandThreads / band_group(Nc)) * x : 0);
+    return chunk * (rb * x + rows) + band_noise_reals<Real, M>(Nc, chunk, rb, lean) * sizeof(Real) + (lean == 2 ? 0 : rb * nz) +
+           (rings && !lean ? (kBandThreads / band_group(Nc)) * x : 0);
 }
 
 // grid (splits, realisations / rb, segments)
 // STAGE: the chunk's table rows go through shared memory, loaded in part 1 beside the noise by
 // every thread, so that the recursion waits for no global load
 template <class Real, class TabT, int M, bool STAGE, int NT>
-__global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_kernel(SampleParams P, int chunk, int rb)
+__global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_kernel(SampleParams P, int chunk, int rb, int lean)
 {
     using C = cplx<Real>;
     constexpr int G = kG<M>, ROW = step_row(M), NU = unit_vals(M), NC = unit_calls(M);
@@ -227,14 +239,15 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
     C* X = reinterpret_cast<C*>(smem_raw);
     Real* NZ = reinterpret_cast<Real*>(X + (size_t)rb * chunk * Nc);
     C* W = reinterpret_cast<C*>(NZ);
-    Real* RW = NZ + (size_t)rb * cn * NU;
+    constexpr bool LEAN = !STAGE && NT == kBandThreads;  // builds that lean layouts run on
+    Real* RW = NZ + (LEAN ? band_noise_reals<Real, M>(Nc, chunk, rb, lean) : (size_t)rb * cn * NU);
     Real* S = RW + (STAGE ? (size_t)cn * RV : 0);
-    Real* NY = S + (size_t)rb * n_units * NU;
-    C* RT = reinterpret_cast<C*>(NY + (size_t)chunk * ROW);
-    const Real* anc = (const Real*)P.anc;
+    Real* NY = S + (LEAN && lean == 2 ? 0 : (size_t)rb * n_units * NU);
+    C* RT = LEAN && lean ? W + Nc : reinterpret_cast<C*>(NY + (size_t)chunk * ROW);
+    Real* anc = (Real*)P.anc;
     const size_t anc_r = aoff<M>(P, 0, 1, 0, 0, 0);  // from one realisation's anchor states to the next's
     const Real* xrg = anc + aoff<M>(P, c, r, has_right ? sg.right : 0, 0, 0);
-    const Real* xlg = anc + aoff<M>(P, c, r, sg.left, 0, 0);
+    Real* xlg = anc + aoff<M>(P, c, r, sg.left, 0, 0);
     const TabT* steps = (const TabT*)(c == 0 ? P.steps[0] : P.steps[1]);
     if (tid < rb * kKeyWords) rk[tid / kKeyWords][tid % kKeyWords] = round_key_word(P.seed + (uint64_t)(r + tid / kKeyWords), tid % kKeyWords);
     __syncthreads();
@@ -267,7 +280,7 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
         if (c0 == sg.p0) {
             // the anchors' states, the first values of the launch before this one
             wait_launch();
-            for (int idx = tid; idx < nr * n_units; idx += nt) {
+            for (int idx = tid; idx < (LEAN && lean == 2 ? 0 : nr * n_units); idx += nt) {
                 const int z = idx / n_units, u = idx - z * n_units;
                 Real v[NU];
                 VecN<Real, NU>::ldcg(xlg + z * anc_r + (size_t)NU * u, v);
@@ -309,7 +322,8 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
         } else {
             for (int u = tid; u < n_units; u += nt) {
                 Real x[NU], xr[NU];
-                VecN<Real, NU>::ld(S + (size_t)NU * u, x);
+                if (LEAN && lean == 2) VecN<Real, NU>::ldcg(xlg + (size_t)NU * u, x);
+                else VecN<Real, NU>::ld(S + (size_t)NU * u, x);
                 if (has_right) VecN<Real, NU>::ldcg(xrg + (size_t)NU * u, xr);
 #pragma unroll 2
                 for (int k = 0; k < nk; ++k) {
@@ -322,7 +336,8 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
                     }
                     if (pos >= own0) put_unit<C, Real, M>(X + (size_t)k * Nc, u, x);
                 }
-                VecN<Real, NU>::st(S + (size_t)NU * u, x);
+                if (LEAN && lean == 2) VecN<Real, NU>::st(xlg + (size_t)NU * u, x);  // this thread's own in the next chunk
+                else VecN<Real, NU>::st(S + (size_t)NU * u, x);
             }
         }
         __syncthreads();

@@ -1907,6 +1907,7 @@ struct SegConfig {
     int band_rb;                  // realisations per CTA
     int band_threads;             // threads per CTA
     bool band_stage;
+    int band_lean;                // layout of the longest ring-dependent plans (smerf_band.cuh)
     size_t band_smem;
 };
 
@@ -2167,20 +2168,23 @@ inline void band_config(const smerf_plan* pl, int n, SegConfig& cfg)
     // has twice the chains for its threads and the staged table rows serve both (20001 realisations of
     // 32 x 64, p = 2: 2588 -> 2010 us with two, 2028 with four)
     const int rb = sizeof(Real) == 8 && !rings && ctas >= 1024 && 4 * Nc <= kBandThreads ? 2 : 1;
+    int lean = 0;
     auto smem = [&](int chunk, bool stage) {
-        return M == 1 ? (stage ? band_smem<Real, 1, true>(Nc, chunk, rb, rings) : band_smem<Real, 1, false>(Nc, chunk, rb, rings))
-             : M == 2 ? (stage ? band_smem<Real, 2, true>(Nc, chunk, rb, rings) : band_smem<Real, 2, false>(Nc, chunk, rb, rings))
-                      : (stage ? band_smem<Real, 3, true>(Nc, chunk, rb, rings) : band_smem<Real, 3, false>(Nc, chunk, rb, rings));
+        return M == 1 ? (stage ? band_smem<Real, 1, true>(Nc, chunk, rb, rings, lean) : band_smem<Real, 1, false>(Nc, chunk, rb, rings, lean))
+             : M == 2 ? (stage ? band_smem<Real, 2, true>(Nc, chunk, rb, rings, lean) : band_smem<Real, 2, false>(Nc, chunk, rb, rings, lean))
+                      : (stage ? band_smem<Real, 3, true>(Nc, chunk, rb, rings, lean) : band_smem<Real, 3, false>(Nc, chunk, rb, rings, lean));
     };
     size_t budget = ctas * splits <= 152 ? kMaxSmem : kMaxSmem / 2;
     // the rows of a chunk through shared memory while the recursion's latency is what counts: for few
     // units, or few CTAs (Nside 128, 16 realisations: 137 us with, 115 us without)
     bool stage = Nc / unit_slots(M) <= (ctas < 152 && !rings ? 128 : 64) && smem(4, true) <= budget;
     if (smem(1, stage) > budget) budget = kMaxSmem;
+    while (rings && smem(1, stage) > budget && lean < (pl->H > 0 ? 1 : 2)) ++lean;  // only the longest rings: stage is off
     if (smem(1, stage) > budget) return;
     int chunk = 1;
-    while (chunk < 16 && chunk < seg_len && smem(chunk + 1, stage) <= budget) ++chunk;
-    cfg.band_splits = (int)splits;
+    while (!lean && chunk < 16 && chunk < seg_len && smem(chunk + 1, stage) <= budget) ++chunk;
+    cfg.band_lean = lean;
+    cfg.band_splits = lean == 2 ? 1 : (int)splits;
     cfg.band_chunk = chunk;
     cfg.band_rb = stage ? rb : 1;
     // at most one CTA per SM: all of the SM's registers for it (181 x 512 and smaller, anchored: p = 1 14.5
@@ -2211,7 +2215,7 @@ int launch_band(const SampleParams& P, int n_segments, const SegConfig& cfg, cud
     // want (Nside 128, 16 realisations: 119 us without, 123 with)
     lc.attrs = &at;
     lc.numAttrs = early && (long long)lc.gridDim.x * lc.gridDim.y * lc.gridDim.z <= 304 ? 1 : 0;
-    return cudaLaunchKernelEx(&lc, kern, P, cfg.band_chunk, cfg.band_rb) == cudaSuccess ? SMERF_OK : SMERF_ECUDA;
+    return cudaLaunchKernelEx(&lc, kern, P, cfg.band_chunk, cfg.band_rb, cfg.band_lean) == cudaSuccess ? SMERF_OK : SMERF_ECUDA;
 }
 
 // early: the launch before this one writes the anchors' states only (see early_launch)

@@ -36,3 +36,23 @@ def test_large_primes_in_fp32():
     from paper_1709_10314_gb300 import Plan
     plan = Plan([30.0], 1.0, 4, 8192, anchor_spacing=2)
     assert _worst(plan, [8158, 4078, 8158, 4078], [0.0, 0.1, 0.2, 0.0]) < 4e-6
+
+
+@pytest.mark.parametrize("fp64,kappa,n_phi,H", [
+    (False, (6.0, 11.0, 25.0), 8192, 2),   # three factors: the largest states
+    (False, (6.0, 11.0, 25.0), 8192, 0),
+    (True, (6.0, 11.0, 25.0), 4096, 2),
+    (True, (6.0, 11.0, 25.0), 4096, 0),
+    (True, (9.0,), 8192, 0),               # Alg. 2's order, whose single segment per chain has no right anchor
+    (True, (6.0, 15.0), 8192, 0),
+    (False, (9.0,), 16384, 0),
+    (False, (6.0, 15.0), 8192, 2),
+])
+def test_longest_rings_of_every_kind_of_plan(fp64, kappa, n_phi, H):
+    """Bounds: FP32 sums as above (more for the modes' phases); FP64 phases m phi0 of up to 8192 x 0.3 rad
+    round to 2.7e-13."""
+    from paper_1709_10314_gb300 import SMERF_ORDER_PAPER, SMERF_RECUR_FP64, Plan
+    flags = (SMERF_RECUR_FP64 if fp64 else 0) | (0 if H else SMERF_ORDER_PAPER)
+    plan = Plan(list(kappa), 1.0, 8, n_phi, flags=flags, anchor_spacing=H)
+    n = [12, n_phi // 2, n_phi - 2, n_phi, n_phi - 34, n_phi, 502, n_phi // 4]
+    assert _worst(plan, n, [0.1, -0.2, 0.3, 0.0, 0.0, 0.25, 0.3, 0.0]) < (1e-11 if fp64 else 1e-5)
