@@ -407,8 +407,10 @@ int smerf_plan_launch_candidates(const smerf_plan* plan, int* cand, int max_n);
  * smerf_plan_set_launch -- fix the segment-kernel launch configuration (SMERF_LAUNCH_INTS
  * integers) to one of the candidates (e.g. a choice smerf_plan_autotune made in an earlier
  * process), or with config == NULL return to the built-in choice, which depends on n_samples
- * (radix plan 16 in FP32).  Small requests and plans with ring-dependent longitudes run on the
- * band kernel, which takes only the radix plan from it.
+ * (radix plan 16 in FP32).  Small requests and most plans with ring-dependent longitudes run on the
+ * band kernel, which takes only the radix plan from it; the FP32 ring plans that run on the
+ * warp-specialised kernel take the whole configuration where a ring build of it exists, else only
+ * the radix plan.
  * SMERF_EINVAL if config is not a candidate.  Host only.
  */
 int smerf_plan_set_launch(smerf_plan* plan, const int* config);

@@ -50,6 +50,9 @@ void free_rings(smerf_plan* pl)
     pl->rings_ph_dev = nullptr;
     pl->rings_off_dev = nullptr;
     pl->rings_total = 0;
+    pl->rings_ws = false;
+    pl->rings_short = 0;
+    pl->rings_shifted = false;
 }
 
 // output values of one realisation
@@ -700,8 +703,13 @@ int smerf_plan_set_rings(smerf_plan* plan, const int* n_phi_ring, const double* 
     std::vector<unsigned long long> ph(plan->n_theta);
     std::vector<long long> off(plan->n_theta);
     long long total = 0;
+    bool on_ws = true;
+    bool shifted = false;
+    int n_short = 0;
     for (int k = 0; k < plan->n_theta; ++k) {
         const int nk = n_phi_ring[k];
+        n_short += nk != plan->n_phi;
+        on_ws = on_ws && (nk == plan->n_phi || nk <= plan->n_phi / 2);
         const double p0 = phi0_ring ? phi0_ring[k] : 0.0;
         if ((nk & 1) || nk < 4 || nk > plan->n_phi || !isfinite(p0)) return SMERF_EINVAL;
         n[k] = nk;
@@ -710,6 +718,7 @@ int smerf_plan_set_rings(smerf_plan* plan, const int* n_phi_ring, const double* 
         turns -= rint(turns);
         if (turns >= 0.5) turns -= 1.0;
         ph[k] = (unsigned long long)llrint(ldexp(turns, 64));
+        shifted = shifted || ph[k] != 0;
         off[k] = total;
         total += nk;
     }
@@ -733,6 +742,9 @@ int smerf_plan_set_rings(smerf_plan* plan, const int* n_phi_ring, const double* 
         return rc;
     }
     plan->rings_total = total;
+    plan->rings_ws = on_ws;
+    plan->rings_short = n_short;
+    plan->rings_shifted = shifted;
     return SMERF_OK;
 }
 
@@ -936,6 +948,9 @@ int smerf_plan_autotune_anchor(smerf_plan* plan, int n_samples, const int* candi
         std::swap(plan->rings_ph_dev, best->rings_ph_dev);
         std::swap(plan->rings_off_dev, best->rings_off_dev);
         std::swap(plan->rings_total, best->rings_total);
+        std::swap(plan->rings_ws, best->rings_ws);
+        std::swap(plan->rings_short, best->rings_short);
+        std::swap(plan->rings_shifted, best->rings_shifted);
         if (chosen) *chosen = plan->H;
     }
     if (best) smerf_plan_destroy(best);

@@ -13,128 +13,15 @@
 //   3. the C2R FFTs of the chunk's rings side by side, written straight to the output.
 // A segment can be split further over `splits` CTAs: each repeats parts 1 and 2 from the
 // segment's start (they are cheap) and synthesises only its own share of the rings.
-//
-// Rings with their own point count n: Y_q = sum over m = q (mod n) of c_m e^{i m phi0} is formed
-// and packed for an n/2-point complex FFT, which runs in Stockham passes over the factors of n/2
-// (4, 2, then the odd primes), one output point per thread from r terms with the roots of unity
-// from a table of the ring's own, a group of threads per ring.  HEALPix's polar rings (4i points)
-// took O(n^2) terms in the FFT warps of one CTA per segment before: Nside 128, 16 realisations,
-// 4266 -> 119 us a call.  One FP64 realisation of 64 x 128 in Alg. 2's order: 166 -> 24.6 us (the
-// fixed-point FFT among them); one of 181 x 512, p = 2: 31.1 -> 22.7 us (the anchor tiles among them).
+// Rings with their own point count: smerf_ragged.cuh, a group of threads per ring.  One FP64
+// realisation of 64 x 128 in Alg. 2's order: 166 -> 24.6 us (the fixed-point FFT among them); one of
+// 181 x 512, p = 2: 31.1 -> 22.7 us (the anchor tiles among them).
 #pragma once
 
 namespace smerf {
 
 constexpr int kBandThreads = 256;      // two CTAs per SM
 constexpr int kBandThreadsFew = 512;   // requests of at most one CTA per SM (band_config)
-
-// e^{2 pi i p}, p = ph 2^-64 turns
-template <class Real> __device__ __forceinline__ cplx<Real> cis_turns(uint64_t ph)
-{
-    Real sn, cs;
-    if constexpr (sizeof(Real) == 4) sincospif((float)(int32_t)(ph >> 32) * 0x1p-31f, &sn, &cs);
-    else fx_cis(ph, cs, sn);
-    return cmk<cplx<Real>>(cs, sn);
-}
-
-// threads that share a ring of its own point count, and such groups per CTA: a warp for rings up
-// to 512 points, the whole CTA from 4096 on
-__host__ __device__ inline int band_group(int Nc) { return Nc <= 256 ? 32 : Nc >= 2048 ? 256 : Nc / 8; }
-
-__device__ __forceinline__ void band_group_sync(int gs, int g)
-{
-    if (gs == 32) __syncwarp();
-    else bar_sync(6 + g, gs);
-}
-
-// Y_q of the ring's coefficients X (slot 0 = (g_0, Re g_M), slot m = g_m, M = Nc): the real field
-// T(phi) = sum_{|m| <= M} c_m e^{i m phi}, c_0 = g_0, c_{+-m} = g_m, conj g_m, c_{+-M} = Re g_M / 2, has
-// Y_q = sum over m = q (mod n) of c_m e^{i m phi0} (modes above the ring's own Nyquist alias onto it)
-template <class Real>
-__device__ __forceinline__ cplx<Real> band_fold(const cplx<Real>* X, int Nc, int n, uint64_t ph, int q)
-{
-    using C = cplx<Real>;
-    C acc = cmk<C>(0, 0);
-    auto term = [&](int m) {
-        const C g = m == 0 ? cmk<C>(X[0].x, 0) : (m == Nc ? cmk<C>((Real)0.5 * X[0].y, 0) : X[m]);
-        return ph == 0 ? g : cmul(g, cis_turns<Real>((uint64_t)m * ph));
-    };
-    for (int m = q; m <= Nc; m += n) acc = cadd(acc, term(m));
-    for (int m = q == 0 ? n : n - q; m <= Nc; m += n) acc = cadd(acc, cconj(term(m)));  // -m < 0
-    return acc;
-}
-
-// One ring of n = 2 N points from its coefficients in X (destroyed) with W as second buffer and
-// RT for the N roots e^{2 pi i t / n}, by the gs threads of a group (lane l of group g)
-template <class Real>
-__device__ __noinline__ void band_ragged_ring(cplx<Real>* X, cplx<Real>* W, cplx<Real>* RT, int Nc, int n, uint64_t ph,
-                                              cplx<Real>* gout, int l, int gs, int g)
-{
-    using C = cplx<Real>;
-    const int N = n / 2;
-    {
-        // t / n as a 64-bit fraction: t (2^64 / n) with the division's remainder r < n <= 2^13 (t r < 2^26)
-        const uint64_t q = ~0ull / (unsigned)n;
-        const unsigned r = (unsigned)(~0ull - q * (unsigned)n) + 1u;
-        for (int t = l; t < N; t += gs) RT[t] = cis_turns<Real>((uint64_t)t * q + ((unsigned)t * r) / (unsigned)n);
-    }
-    band_group_sync(gs, g);
-    // fold and C2R packing (c2r_pack's Z), the pair q, N - q together
-    for (int q = l; 2 * q <= N; q += gs) {
-        const C a = band_fold<Real>(X, Nc, n, ph, q), b = cconj(band_fold<Real>(X, Nc, n, ph, N - q));
-        if (q == 0) {
-            W[0] = cmk<C>(a.x + b.x, a.x - b.x);
-        } else {
-            const C e = cadd(a, b), o = cmuli(cmul(RT[q], csub(a, b)));
-            W[q] = cadd(e, o);
-            if (2 * q < N) W[N - q] = cconj(csub(e, o));
-        }
-    }
-    band_group_sync(gs, g);
-    C* src = W;
-    C* dst = X;
-    int Ns = 1, rem = N, p = 3;
-    while (rem > 1) {
-        int r;
-        if ((rem & 3) == 0) r = 4;
-        else if ((rem & 1) == 0) r = 2;
-        else {
-            while (p * p <= rem && rem % p) p += 2;
-            r = rem % p ? rem : p;
-        }
-        rem /= r;
-        const int Wn = Ns * r, m = N / r, unit = N / Wn;
-        for (int e = l; e < N; e += gs) {
-            const int blk = e / Wn, w = e - blk * Wn, st = w * unit;  // w = kk + a Ns
-            const C* in = src + blk * Ns + w % Ns;
-            // large primes in parts of 16 terms, so that an FP32 sum rounds 16 + r / 16 times (2 x 4079
-            // points: 1.3e-6 -> 3.5e-7 of the deviation, 8e-6 -> 1.7e-6 at most)
-            C acc = in[0], sum = cmk<C>(0, 0);
-            int t = st;
-            for (int i = 1; i < r; ++i) {
-                if ((i & 15) == 0) {
-                    sum = cadd(sum, acc);
-                    acc = cmk<C>(0, 0);
-                }
-                const int u = 2 * t;  // root of order N: e^{2 pi i t / N} = e^{2 pi i u / n}, half a turn from t = N / 2 on
-                const C x = in[i * m], y = u < N ? RT[u] : RT[u - N];
-                const C z = cmul(x, y);
-                acc = u < N ? cadd(acc, z) : csub(acc, z);
-                t += st;
-                if (t >= N) t -= N;
-            }
-            acc = cadd(sum, acc);
-            if (rem == 1) __stcs(gout + e, acc);
-            else dst[e] = acc;
-        }
-        Ns = Wn;
-        band_group_sync(gs, g);
-        C* s = src;
-        src = dst;
-        dst = s;
-    }
-    if (N == 1 && l == 0) __stcs(gout, W[0]);
-}
 
 // Table rows of unit u at one position, G rows of step_row(M) values, converted to Real; ny: the
 // Nyquist chain's row (unit 0 only)
@@ -191,6 +78,7 @@ __host__ __device__ constexpr int band_row_reals()
 // buffer; p = 3 with 4096 complex points in FP32: 229472 bytes of 262240); lean = 2, Alg. 2's order:
 // the states stay in the anchors' scratch, whose start-ring entry of a chain and realisation
 // belongs to this CTA alone (no other segment, no splits)
+template <class Real> constexpr bool band_global_states(int M) { return M == 1 || (M == 2 && sizeof(Real) == 8); }
 template <class Real, int M>
 __host__ __device__ inline size_t band_noise_reals(int Nc, int chunk, int rb, int lean)
 {
@@ -210,7 +98,8 @@ __host__ __device__ inline size_t band_smem(int Nc, int chunk, int rb, bool ring
 // grid (splits, realisations / rb, segments)
 // STAGE: the chunk's table rows go through shared memory, loaded in part 1 beside the noise by
 // every thread, so that the recursion waits for no global load
-template <class Real, class TabT, int M, bool STAGE, int NT>
+// GS: lean = 2
+template <class Real, class TabT, int M, bool STAGE, int NT, bool GS>
 __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_kernel(SampleParams P, int chunk, int rb, int lean)
 {
     using C = cplx<Real>;
@@ -242,7 +131,7 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
     constexpr bool LEAN = !STAGE && NT == kBandThreads;  // builds that lean layouts run on
     Real* RW = NZ + (LEAN ? band_noise_reals<Real, M>(Nc, chunk, rb, lean) : (size_t)rb * cn * NU);
     Real* S = RW + (STAGE ? (size_t)cn * RV : 0);
-    Real* NY = S + (LEAN && lean == 2 ? 0 : (size_t)rb * n_units * NU);
+    Real* NY = S + (GS ? 0 : (size_t)rb * n_units * NU);
     C* RT = LEAN && lean ? W + Nc : reinterpret_cast<C*>(NY + (size_t)chunk * ROW);
     Real* anc = (Real*)P.anc;
     const size_t anc_r = aoff<M>(P, 0, 1, 0, 0, 0);  // from one realisation's anchor states to the next's
@@ -280,7 +169,7 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
         if (c0 == sg.p0) {
             // the anchors' states, the first values of the launch before this one
             wait_launch();
-            for (int idx = tid; idx < (LEAN && lean == 2 ? 0 : nr * n_units); idx += nt) {
+            for (int idx = tid; idx < (GS ? 0 : nr * n_units); idx += nt) {
                 const int z = idx / n_units, u = idx - z * n_units;
                 Real v[NU];
                 VecN<Real, NU>::ldcg(xlg + z * anc_r + (size_t)NU * u, v);
@@ -322,7 +211,7 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
         } else {
             for (int u = tid; u < n_units; u += nt) {
                 Real x[NU], xr[NU];
-                if (LEAN && lean == 2) VecN<Real, NU>::ldcg(xlg + (size_t)NU * u, x);
+                if constexpr (GS) VecN<Real, NU>::ldcg(xlg + (size_t)NU * u, x);
                 else VecN<Real, NU>::ld(S + (size_t)NU * u, x);
                 if (has_right) VecN<Real, NU>::ldcg(xrg + (size_t)NU * u, xr);
 #pragma unroll 2
@@ -336,7 +225,7 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
                     }
                     if (pos >= own0) put_unit<C, Real, M>(X + (size_t)k * Nc, u, x);
                 }
-                if (LEAN && lean == 2) VecN<Real, NU>::st(xlg + (size_t)NU * u, x);  // this thread's own in the next chunk
+                if constexpr (GS) VecN<Real, NU>::st(xlg + (size_t)NU * u, x);  // this thread's own in the next chunk
                 else VecN<Real, NU>::st(S + (size_t)NU * u, x);
             }
         }
@@ -362,8 +251,8 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
                 const int ring = ring0 + dir * k, n = P.ring_n[ring];
                 if (n == P.n_phi) continue;
                 if (turn++ % groups != g) continue;
-                band_ragged_ring<Real>(X + (size_t)k * Nc, W + (size_t)k * Nc, RT + (size_t)g * Nc, Nc, n, P.ring_ph[ring],
-                                       (C*)((Real*)P.out + (size_t)r * P.ring_total + P.ring_off[ring]), tid - g * gs, gs, g);
+                ragged_ring<Real>(X + (size_t)k * Nc, W + (size_t)k * Nc, RT + (size_t)g * Nc, true, Nc, n, P.ring_ph[ring],
+                                  (C*)((Real*)P.out + (size_t)r * P.ring_total + P.ring_off[ring]), tid - g * gs, gs, 6 + g);
             }
             __syncthreads();
         }

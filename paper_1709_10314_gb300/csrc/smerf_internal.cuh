@@ -80,6 +80,9 @@ struct smerf_plan {
     unsigned long long* rings_ph_dev;  // offsets as 64-bit fractions of a turn
     long long* rings_off_dev;
     long long rings_total;
+    bool rings_ws;    // every ring whole or of at most n_phi / 2 points (the warp-specialised kernel's room)
+    bool rings_shifted;  // some ring has an offset
+    int rings_short;  // rings that are not whole
     // launch parameters chosen by smerf_plan_autotune (valid = 0: built-in heuristic)
     struct { int valid, upt, rmax, np, nf, minb, radix; float ms; } tune;
 };

@@ -1442,6 +1442,12 @@ __host__ __device__ constexpr int ws_lg_hi(int UPT, int M)
                : 12;
 }
 
+}  // namespace smerf
+
+#include "smerf_ragged.cuh"
+
+namespace smerf {
+
 // Warp-specialised segment kernel.  Threads [0, NP) are the producer group: the recursion of
 // ring k (state in registers, units tid, tid + NP, ...) into coefficient buffer B[k & 1].
 // Threads [NP, NP + NF) are the FFT group: the C2R FFT of ring k from B[k & 1] (with W as
@@ -1452,7 +1458,9 @@ __host__ __device__ constexpr int ws_lg_hi(int UPT, int M)
 // Every FULL/EMPTY barrier counts NP + NF threads; the FFT passes use a group barrier.
 // CG: the anchor states were written by the same launch (read through L2, not the read-only path).
 // PAIR: see hr_pass (false in the persistent batch kernels).
-template <class Real, class TabT, int M, int UPT, int RMAX, bool CG = false, bool PAIR = true>
+// RINGS: ring-dependent longitudes (FP32): whole rings, with or without an offset, and rings of up to n_phi
+// / 2 points, whose buffer and roots share W.
+template <class Real, class TabT, int M, int UPT, int RMAX, bool CG = false, bool PAIR = true, bool RINGS = false>
 __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, int group)
 {
     using C = cplx<Real>;
@@ -1626,7 +1634,32 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
             if (!(c == 1 && pos == 0)) {  // the start ring is written by the northern chain
                 RingOut<C> gout{(C*)((Real*)P.out + ((size_t)r0 * P.n_theta + ring) * (size_t)P.n_phi),
                                 (size_t)P.n_theta * (size_t)(P.n_phi / 2)};
-                if constexpr (sizeof(Real) == 8) {
+                bool whole = true;
+                if constexpr (RINGS) {
+                    const int n = P.ring_n[ring];
+                    const uint64_t ph = P.ring_ph[ring];
+                    gout.base = (C*)((Real*)P.out + (size_t)r0 * P.ring_total + P.ring_off[ring]);
+                    gout.stride = (size_t)(P.ring_total / 2);
+                    gout.wide = (reinterpret_cast<uintptr_t>(gout.base) & 15) == 0 && (R == 1 || P.ring_total % 4 == 0);
+                    whole = n == P.n_phi;
+                    if (!whole) {
+                        for (int r = 0; r < R; ++r)
+                            ragged_ring<Real>(B + (size_t)r * Nc, W + (size_t)r * Nc, W + Nc / 2, r == 0, Nc, n, ph, gout[r],
+                                              ftid, NF, kBarFft);
+                    } else if (ph != 0) {
+                        for (int s = ftid; s < Nc; s += NF) {
+                            const C w = cis_turns<Real>((uint64_t)(s == 0 ? Nc : s) * ph);
+                            for (int r = 0; r < R; ++r) {
+                                C* x = B + (size_t)r * Nc + s;
+                                if (s == 0) x->y *= w.x;
+                                else *x = cmul(*x, w);
+                            }
+                        }
+                        bar_sync(kBarFft, NF);
+                    }
+                }
+                if (RINGS && !whole) {
+                } else if constexpr (sizeof(Real) == 8) {
                     grp_fx_c2r(B, W, R, P.lgNc, (const int4*)P.twx, (const int4*)P.prex, gout, fxred, ftid, NF, kBarFft);
                 } else if (!P.fft_r4) {
                     hr_c2r<C, ws_lg_lo(UPT, M), ws_lg_hi(UPT, M), PAIR>(P.lgNc, B, W, R, twp, (const C*)P.tw2, pre, gout, ftid, NF);
@@ -1639,10 +1672,10 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
     }
 }
 
-template <class Real, class TabT, int M, int UPT, int RMAX, int MINB>
+template <class Real, class TabT, int M, int UPT, int RMAX, int MINB, bool RINGS>
 __global__ void __launch_bounds__(ws_max_threads(MINB, M), MINB) segment_ws_kernel(SampleParams P)
 {
-    ws_body<Real, TabT, M, UPT, RMAX>(P, blockIdx.y, blockIdx.x);
+    ws_body<Real, TabT, M, UPT, RMAX, false, true, RINGS>(P, blockIdx.y, blockIdx.x);
 }
 
 // batched: item = (request, segment, realisation group); all requests of a launch share the
@@ -1855,10 +1888,10 @@ inline cudaError_t set_smem_attr(K kern, size_t smem)
 constexpr int kMaxThreads = 1024;
 constexpr size_t kMaxSmem = 226 * 1024;  // leaves room for the static shared arrays
 
-template <class Real, class TabT, int M, int UPT, int RMAX, int MINB = 1>
+template <class Real, class TabT, int M, int UPT, int RMAX, int MINB = 1, bool RINGS = false>
 int launch_ws(const SampleParams& P, int n_segments, int nt, size_t smem, cudaStream_t st)
 {
-    auto kern = segment_ws_kernel<Real, TabT, M, UPT, RMAX, MINB>;
+    auto kern = segment_ws_kernel<Real, TabT, M, UPT, RMAX, MINB, RINGS>;
     if (set_smem_attr(kern, smem) != cudaSuccess) return SMERF_ECUDA;
     dim3 grid((P.n_samples + RMAX - 1) / RMAX, n_segments);
     kern<<<grid, nt, smem, st>>>(P);
@@ -1956,6 +1989,15 @@ template <class Real> inline bool ws_built(int upt, int rmax, int minb, int M)
     if (sizeof(Real) == 8) return rmax == 1 && (upt == 1 || upt == 2 || upt == 4 || upt == 8);
     return (upt == 1 && rmax == 4) || (upt == 2 && (rmax == 4 || rmax == 2)) || (upt == 4 && (rmax == 2 || rmax == 1)) ||
            (upt == 8 && rmax == 1);
+}
+
+// the same with ring-dependent longitudes: the built-in choices (seg_config) in FP32
+template <class Real> inline bool ws_rings_built(int upt, int rmax, int minb, int M)
+{
+    if (sizeof(Real) != 4) return false;
+    if (M == 3) return minb == 1 && rmax == 1;
+    if (minb == 2) return upt == 4 && rmax == 1;
+    return (upt == 1 && rmax == 4) || (upt == 2 && rmax == 2) || (upt == 4 && rmax <= 2) || (upt == 8 && rmax == 1);
 }
 
 // Every warp-specialised configuration that fits the plan, as kLaunchInts integers (units per
@@ -2068,6 +2110,7 @@ inline SegConfig seg_config(const smerf_plan* pl, int n)
     const int n_units = pl->n_slots / unit_slots(M);
     const int Nc = pl->n_phi / 2;
     if (pl->tune.valid && ws_built<Real>(pl->tune.upt, pl->tune.rmax, pl->tune.minb, M) &&
+        (!pl->rings_total || ws_rings_built<Real>(pl->tune.upt, pl->tune.rmax, pl->tune.minb, M)) &&
         ws_smem<Real>(pl, pl->tune.rmax) <= 226 * 1024 &&
         (n_units + pl->tune.upt - 1) / pl->tune.upt <= pl->tune.np &&
         pl->tune.np + pl->tune.nf <= ws_max_threads(pl->tune.minb, M)) {
@@ -2137,13 +2180,46 @@ inline SegConfig seg_config(const smerf_plan* pl, int n)
     return cfg;
 }
 
+// With ring-dependent longitudes that the warp-specialised kernel can take (FP32), the most CTAs
+// (segments x realisations) for which the band kernel is the faster one; whole: the line for plans
+// whose rings are all whole.  Timed both ways over 512 to 16384 longitudes, p = 1 .. 3, 1 to 64 realisations,
+// anchored and in Alg. 2's order: whole rings with and without offsets; eight short rings among
+// whole ones, and offsets in Alg. 2's order (the second set of lines); reduced grids, a third of whose rings are shorter (the last: the FFT group's few
+// threads synthesise them one after another, and the band kernel's 256 side by side).  E.g. band
+// against warp-specialised kernel, us: 2048 x 4096, p = 2, 4 realisations, whole 505 / 279, reduced 724 / 813;
+// 4096 x 8192, 4 realisations, p = 1 whole 1342 / 527, reduced 2095 / 1263; 512 x 1024, p = 1, 4 realisations,
+// whole 43 / 56, reduced 81 / 302.
+inline long long rings_band_ctas(const smerf_plan* pl, int n, long long whole)
+{
+    const int Nc = pl->n_phi / 2, M = pl->p;
+    const bool anchored = pl->H > 0;
+    if (pl->rings_short == 0 && (anchored || !pl->rings_shifted)) {
+        if (Nc <= 128) return whole;
+        if (Nc <= 256) return 304;
+        if (Nc <= 512) return anchored ? (M == 3 ? 152 : 304) : M == 1 ? 304 : 64;
+        return Nc == 1024 && M == 1 ? (anchored ? 200 : 64) : 0;
+    }
+    if (pl->rings_short <= pl->n_theta / 8) {
+        if (Nc <= 128) return whole;
+        if (Nc <= 512) return anchored && M != 2 ? (M == 1 && Nc == 256 ? 2000 : 608) : 304;
+        if (Nc == 1024) return M == 1 ? (anchored ? 304 : 152) : M == 2 ? (anchored ? 152 : 64) : 0;
+        return Nc <= 4096 && M == 1 && !anchored ? 64 : 0;
+    }
+    if (Nc <= 512) return 1ll << 40;
+    if (M == 3 && !anchored) return Nc <= 4096 ? 16 : 0;
+    if (Nc == 1024) return !anchored ? 1ll << 40 : M == 1 ? 2000 : M == 2 ? 1000 : 1500;
+    if (Nc == 2048) return M == 1 ? (anchored ? 304 : 100) : M == 2 && (n > 1 || !anchored) ? (anchored ? 1500 : 304) : 0;
+    return Nc == 4096 && M == 1 && !anchored ? 304 : 0;
+}
+
 // Whether a request runs on the band kernel (smerf_band.cuh) in place of the warp-specialised one,
-// and with how many CTAs per segment and rings per chunk: always with ring-dependent longitudes;
+// and with how many CTAs per segment and rings per chunk: with ring-dependent longitudes always in FP64 and
+// below rings_band_ctas in FP32 (always for layouts that the warp-specialised kernel has no room for);
 // else where the CTAs (segments x realisations) are few for the ring length.  Both kernels were
 // timed over n_phi 128 to 8192, p = 1 .. 3, FP32 and FP64, 1 to 256 realisations, Alg. 2's and the
 // anchored order.  In FP32 the band kernel wins while its CTAs fit the GPU two per SM (1.1 to 2.5
 // times; up to 3.7 in Alg. 2's order), longer for rings so short that its CTAs are brief (64
-// points up to 1280 CTAs); at 2048 complex points one 2048 x 4096 realisation takes 63 us against 56
+// points up to 1152 CTAs); at 2048 complex points one 2048 x 4096 realisation takes 63 us against 56
 // (p = 1) and 122 against 95 (p = 2).  In FP64 a split segment repeats its recursion on the narrow FP64
 // pipe, so the line lies lower: p = 1 at 512 points 132 CTAs 99 against 107 us, at 1024 points 65 CTAs
 // 147 against 155 us and 130 CTAs 185 against 156; p = 2 at 512 points 132 CTAs 149 against 126, at
@@ -2160,7 +2236,10 @@ inline void band_config(const smerf_plan* pl, int n, SegConfig& cfg)
     else if (M == 3) most = Nc <= 128 ? 20480 / Nc : 0;
     else if (sizeof(Real) == 8) most = Nc > 1024 ? 0 : M == 1 && Nc > 256 ? 77824 / Nc : M == 2 && Nc > 512 ? 19456 / Nc : 38912 / Nc;
     else most = Nc <= 128 ? 73728 / Nc : Nc <= 1024 ? 304 : 0;
-    if (!rings && ctas > most) return;
+    if (rings && sizeof(Real) == 4 && pl->rings_ws && ws_rings_built<Real>(cfg.upt, cfg.rmax, cfg.minb, M))
+        most = rings_band_ctas(pl, n, most);
+    else if (rings) most = ctas;
+    if (ctas > most) return;
     const int seg_len = pl->H > 0 ? pl->H : (pl->chain[0].len > pl->chain[1].len ? pl->chain[0].len : pl->chain[1].len) + 1;
     long long splits = ctas > 0 && ctas < 152 ? 152 / ctas : 1;  // one CTA per SM
     if (splits > seg_len) splits = seg_len;
@@ -2179,7 +2258,7 @@ inline void band_config(const smerf_plan* pl, int n, SegConfig& cfg)
     // units, or few CTAs (Nside 128, 16 realisations: 137 us with, 115 us without)
     bool stage = Nc / unit_slots(M) <= (ctas < 152 && !rings ? 128 : 64) && smem(4, true) <= budget;
     if (smem(1, stage) > budget) budget = kMaxSmem;
-    while (rings && smem(1, stage) > budget && lean < (pl->H > 0 ? 1 : 2)) ++lean;  // only the longest rings: stage is off
+    while (rings && smem(1, stage) > budget && lean < (pl->H == 0 && band_global_states<Real>(M) ? 2 : 1)) ++lean;  // only the longest rings: stage is off
     if (smem(1, stage) > budget) return;
     int chunk = 1;
     while (!lean && chunk < 16 && chunk < seg_len && smem(chunk + 1, stage) <= budget) ++chunk;
@@ -2199,8 +2278,11 @@ template <class Real, class TabT, int M>
 int launch_band(const SampleParams& P, int n_segments, const SegConfig& cfg, cudaStream_t st, bool early)
 {
     const bool few = cfg.band_threads == kBandThreadsFew;
-    auto kern = cfg.band_stage ? (few ? segment_band_kernel<Real, TabT, M, true, kBandThreadsFew> : segment_band_kernel<Real, TabT, M, true, kBandThreads>)
-                               : (few ? segment_band_kernel<Real, TabT, M, false, kBandThreadsFew> : segment_band_kernel<Real, TabT, M, false, kBandThreads>);
+    auto kern = cfg.band_stage ? (few ? segment_band_kernel<Real, TabT, M, true, kBandThreadsFew, false> : segment_band_kernel<Real, TabT, M, true, kBandThreads, false>)
+                               : (few ? segment_band_kernel<Real, TabT, M, false, kBandThreadsFew, false> : segment_band_kernel<Real, TabT, M, false, kBandThreads, false>);
+    if constexpr (band_global_states<Real>(M)) {
+        if (cfg.band_lean == 2) kern = segment_band_kernel<Real, TabT, M, false, kBandThreads, true>;
+    }
     if (set_smem_attr(kern, cfg.band_smem) != cudaSuccess) return SMERF_ECUDA;
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(cfg.band_splits, (P.n_samples + cfg.band_rb - 1) / cfg.band_rb, n_segments);
@@ -2218,11 +2300,41 @@ int launch_band(const SampleParams& P, int n_segments, const SegConfig& cfg, cud
     return cudaLaunchKernelEx(&lc, kern, P, cfg.band_chunk, cfg.band_rb, cfg.band_lean) == cudaSuccess ? SMERF_OK : SMERF_ECUDA;
 }
 
+// Ring-dependent longitudes on the warp-specialised kernel (FP32), the builds of ws_rings_built
+template <class TabT, int M>
+int launch_ws_rings(const SampleParams& P, int n_segments, const SegConfig& cfg, cudaStream_t st)
+{
+    const int key = cfg.minb * 100 + cfg.upt * 10 + cfg.rmax;
+    if constexpr (M == 3) {
+        switch (key) {
+            case 111: return launch_ws<float, TabT, M, 1, 1, 1, true>(P, n_segments, cfg.nt, cfg.smem, st);
+            case 121: return launch_ws<float, TabT, M, 2, 1, 1, true>(P, n_segments, cfg.nt, cfg.smem, st);
+            case 141: return launch_ws<float, TabT, M, 4, 1, 1, true>(P, n_segments, cfg.nt, cfg.smem, st);
+            case 181: return launch_ws<float, TabT, M, 8, 1, 1, true>(P, n_segments, cfg.nt, cfg.smem, st);
+            default: return SMERF_EUNSUPPORTED;
+        }
+    } else {
+        switch (key) {
+            case 114: return launch_ws<float, TabT, M, 1, 4, 1, true>(P, n_segments, cfg.nt, cfg.smem, st);
+            case 122: return launch_ws<float, TabT, M, 2, 2, 1, true>(P, n_segments, cfg.nt, cfg.smem, st);
+            case 141: return launch_ws<float, TabT, M, 4, 1, 1, true>(P, n_segments, cfg.nt, cfg.smem, st);
+            case 142: return launch_ws<float, TabT, M, 4, 2, 1, true>(P, n_segments, cfg.nt, cfg.smem, st);
+            case 181: return launch_ws<float, TabT, M, 8, 1, 1, true>(P, n_segments, cfg.nt, cfg.smem, st);
+            case 241: return launch_ws<float, TabT, M, 4, 1, 2, true>(P, n_segments, cfg.nt, cfg.smem, st);
+            default: return SMERF_EUNSUPPORTED;
+        }
+    }
+}
+
 // early: the launch before this one writes the anchors' states only (see early_launch)
 template <class Real, class TabT, int M>
 int dispatch_segments(const SampleParams& P, int n_segments, const SegConfig& cfg, cudaStream_t st, bool early)
 {
     if (cfg.band_splits > 0) return launch_band<Real, TabT, M>(P, n_segments, cfg, st, early);
+    if (P.ring_n) {
+        if constexpr (sizeof(Real) == 4) return launch_ws_rings<TabT, M>(P, n_segments, cfg, st);
+        return SMERF_EUNSUPPORTED;
+    }
     if (cfg.ws) {
         if constexpr (sizeof(Real) == 8 || M == 3) {
             if (cfg.rmax != 1 || cfg.minb != 1) return SMERF_EUNSUPPORTED;
@@ -2317,6 +2429,7 @@ int fill_params(const smerf_plan* pl, uint64_t seed, int n, void* out, void* scr
     if (cfg.smem > kMaxSmem) return SMERF_EUNSUPPORTED;  // one ring per realisation must fit on chip
     if (!cfg.ws && (pl->n_slots / unit_slots(pl->p) + cfg.upt - 1) / cfg.upt > kMaxThreads) return SMERF_EUNSUPPORTED;
     if (pl->n_segments > 65535) return SMERF_EUNSUPPORTED;
+    if (pl->rings_total && pl->tune.valid) cfg.radix = pl->tune.radix;  // of a configuration without a ring build
     P.pingpong = cfg.ws;
     P.np = cfg.np;
     P.fft_r4 = cfg.ws && cfg.radix == 4;
@@ -2331,7 +2444,9 @@ int fill_params(const smerf_plan* pl, uint64_t seed, int n, void* out, void* scr
     // warp-specialised kernels hold (up to 4096 complex points in FP32, 2048 in FP64)
     if ((pl->rings_total || pl->p == 3) && !cfg.ws) return SMERF_EUNSUPPORTED;
     if (cfg.ws && n > 0 && !batch) band_config<Real>(pl, n, cfg);
-    if (pl->rings_total && n > 0 && !batch && cfg.band_splits == 0) return SMERF_EUNSUPPORTED;
+    if (pl->rings_total && n > 0 && !batch && cfg.band_splits == 0 &&
+        !(pl->rings_ws && ws_rings_built<Real>(cfg.upt, cfg.rmax, cfg.minb, pl->p)))
+        return SMERF_EUNSUPPORTED;
     return SMERF_OK;
 }
 
