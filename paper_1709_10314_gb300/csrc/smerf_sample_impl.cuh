@@ -1136,35 +1136,21 @@ __device__ __forceinline__ void grp_c2r_rt(C* buf0, C* buf1, int R, int lgNc, co
 // ---- the FP64 mode's ring FFT in 64-bit fixed point.  On the FP64 pipe (2 lanes per SM) a ring's
 // C2R FFT took two thirds of what is left of the FP64 instructions once the noise is off it; in
 // integers a radix-4 pass costs some 34 instructions per point on 64 to 128 lanes.  A ring's
-// coefficients are scaled by one power of two 2^S that keeps 4 sum |g_m|, a bound of every
-// intermediate value, below 2^62; the sum is formed in integers (largest exponent first, then 17-bit
-// magnitudes rounded up), so that the scale, and with it the field's bits, depend on no thread
-// count.  Values then keep 2^-60 of that sum, so that a field's error against 64-bit references is
-// not above the FP64 FFT's (3.3e-15 -> 3.1e-15 at 64 x 128, 3.9e-15 -> 3.5e-15 at 32 x 64, 1.3e-13 ->
-// 1.0e-13 and 8.6e-13 -> 5.1e-13 on larger grids, the tables' own error).  1024 x 2048, p = 2, 16
-// realisations: 2161 -> 1393 us (1323 with box_muller_call); 20001 of 32 x 64: 3057 -> 2523 us (2010 with two realisations per
-// CTA, band_config).  Factors e^{2 pi i k / n} are exact to 2^-62, stored as two words per component
-// (int4: Re hi, lo, Im hi, lo).
+// values are in units of 2^-S with S falling from pass to pass as their bound grows (fx_unit, from
+// the largest exponent and the sum of magnitudes, formed in integers so that the units, and with
+// them the field's bits, depend on no thread count).  A field's
+// error against 64-bit references is 3.2e-15 at 64 x 128 (3.3e-15 with the FP64 FFT), 3.5e-15 at 32 x 64 (3.9e-15) and
+// 5.2e-13 at 1024 x 2048, p = 2 (8.6e-13; the tables' own error, set-up included).  That grid, 16 realisations: 2161 ->
+// 1332 us (with box_muller_call); 20001 of 32 x 64: 3057 -> 2036 us (with two realisations per CTA,
+// band_config).  One unit for the whole transform took 1322 and 2014 us, and had fewer bits than FP64 from
+// 512 points on.
+// Factors e^{2 pi i k / n} are exact to 2^-62, stored as two words per component (int4: Re hi, lo, Im
+// hi, lo).
 using fxc = longlong2;
 
-__device__ __forceinline__ fxc fxc_mul(fxc a, int4 w)
-{
-    int32_t axh, axl, ayh, ayl;
-    fx_split(a.x, axh, axl);
-    fx_split(a.y, ayh, ayl);
-    fxc r;
-    r.x = fx_dot<true>(axh, axl, w.x, w.y, ayh, ayl, w.z, w.w);
-    r.y = fx_dot<false>(axh, axl, w.z, w.w, ayh, ayl, w.x, w.y);
-    return r;
-}
+__device__ __forceinline__ fxc fxc_mul(fxc a, int4 w, int d) { return fx_cmul(a, w.x, w.y, w.z, w.w, d); }
 
 constexpr int kFxRings = 32;  // rings of one call (the band kernel: two realisations' chunks of up to 16)
-
-// scale of ring r from its largest exponent and its sum of magnitudes (units of 2^(e - 16))
-__device__ __forceinline__ int fx_scale(const int* red, int r)
-{
-    return 60 - (red[r] - 1039 + 32 - __clz(red[kFxRings + r]));
-}
 
 // The rings' largest exponents into red[r], their sums into red[kFxRings + r]
 __device__ __forceinline__ void grp_fx_scales(const double2* buf, int R, int lgNc, int* red, int ftid, int nf, int bar)
@@ -1184,10 +1170,8 @@ __device__ __forceinline__ void grp_fx_scales(const double2* buf, int R, int lgN
             if (pass == 0) {
                 t = (hx > hy ? hx : hy) >> 20;
             } else {
-                // 2^16 times the magnitude over 2^(largest exponent), rounded up
                 const int top = red[r];
-                const int sx = top - (int)(hx >> 20), sy = top - (int)(hy >> 20);
-                t = (sx > 20 ? 0u : ((hx & 0xfffffu) | 0x100000u) >> 4 >> sx) + (sy > 20 ? 0u : ((hy & 0xfffffu) | 0x100000u) >> 4 >> sy) + 2u;
+                t = fx_share(hx, top) + fx_share(hy, top) + 2u;
             }
             if (!whole) {
                 if (pass == 0) atomicMax(reinterpret_cast<unsigned*>(red) + r, t);
@@ -1209,8 +1193,9 @@ __device__ __forceinline__ void grp_fx_scales(const double2* buf, int R, int lgN
 }
 
 // C2R FFTs of R rings (coefficients in buf0 as double2, buf1 the second buffer), radix-4 passes
-// (radix 2 last when log2 Nc is odd); prex, twx: the plan's factors as int4; red: 2 kFxRings words
-template <class Out>
+// (radix 2 last when log2 Nc is odd); prex, twx: the plan's factors as int4; red: 2 kFxRings words; ONE: R is 1
+// (the units and shifts are then the same for every butterfly of a pass)
+template <bool ONE, class Out>
 __device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, int lgNc, const int4* __restrict__ twx,
                                            const int4* __restrict__ prex, Out gout, int* red, int ftid, int nf, int bar)
 {
@@ -1218,10 +1203,12 @@ __device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, 
     grp_fx_scales(buf0, R, lgNc, red, ftid, nf, bar);
     fxc* src = reinterpret_cast<fxc*>(buf0);
     fxc* dst = reinterpret_cast<fxc*>(buf1);
-    // to fixed point and packed (c2r_pack) in place, the pair s, Nc - s together
-    const int half = Nc / 2 + 1;
+    auto unit = [&](int r, int lgL) { return fx_unit(red[r], fx_spread(red[kFxRings + r]), lgL); };
+    // to fixed point, in the unit after the first pass, and packed (c2r_pack) in place, the pair s, Nc - s
+    // together
+    const int half = Nc / 2 + 1, lg1 = lgNc >= 2 ? 2 : 1;
     for (int b = ftid; b < R * half; b += nf) {
-        const int r = b / half, s = b - r * half, S = fx_scale(red, r);
+        const int r = ONE ? 0 : b / half, s = b - r * half, S = unit(r, lg1);
         auto get = [&](int i) {
             const double2 v = buf0[(r << lgNc) + i];
             fxc f;
@@ -1236,18 +1223,18 @@ __device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, 
             continue;
         }
         const fxc bb = cconj(get(Nc - s));
-        const fxc e = cadd(a, bb), o = cmuli(fxc_mul(csub(a, bb), __ldg(prex + s)));
+        const fxc e = cadd(a, bb), o = cmuli(fxc_mul(csub(a, bb), __ldg(prex + s), 0));
         X[s] = cadd(e, o);
         if (2 * s < Nc) X[Nc - s] = cconj(csub(e, o));
     }
     bar_sync(bar, nf);
-    int Ns = 1, off = 0;
+    int Ns = 1, off = 0, lgNs = 0;
     while (Ns < Nc) {
         const int RP = pass_radix(lgNc, Ns), LR = RP == 4 ? 2 : 1;
         const bool first = Ns == 1, last = Ns * RP == Nc;
         const int lgnb = lgNc - LR, nb = 1 << lgnb, total = R << lgnb;
         for (int b = ftid; b < total; b += nf) {
-            const int r = b >> lgnb, j = b & (nb - 1), kk = j & (Ns - 1);
+            const int r = ONE ? 0 : b >> lgnb, j = b & (nb - 1), kk = j & (Ns - 1);
             const fxc* X = src + (r << lgNc);
             fxc v[4];
             v[0] = X[j];
@@ -1257,17 +1244,19 @@ __device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, 
                 v[3] = X[j + 3 * nb];
             }
             if (!first) {
-                v[1] = fxc_mul(v[1], __ldg(twx + off + kk));
+                const int d = fx_shift(fx_spread(red[kFxRings + r]), lgNs, LR);
+                v[0] = fx_cshift(v[0], d);
+                v[1] = fxc_mul(v[1], __ldg(twx + off + kk), d);
                 if (RP == 4) {
-                    v[2] = fxc_mul(v[2], __ldg(twx + off + Ns + kk));
-                    v[3] = fxc_mul(v[3], __ldg(twx + off + 2 * Ns + kk));
+                    v[2] = fxc_mul(v[2], __ldg(twx + off + Ns + kk), d);
+                    v[3] = fxc_mul(v[3], __ldg(twx + off + 2 * Ns + kk), d);
                 }
             }
             if (RP == 4) dft4(v);
             else dft2(v[0], v[1]);
             const int idx = ((j - kk) << LR) + kk;
             if (last) {
-                const int S = fx_scale(red, r);
+                const int S = unit(r, lgNc);
                 double2* D = gout[r] + idx;
 #pragma unroll
                 for (int a = 0; a < 4; ++a)
@@ -1283,6 +1272,7 @@ __device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, 
         }
         if (!first) off += (RP - 1) * Ns;
         Ns *= RP;
+        lgNs += LR;
         if (!last) bar_sync(bar, nf);
         fxc* t = src;
         src = dst;
@@ -1660,7 +1650,7 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
                 }
                 if (RINGS && !whole) {
                 } else if constexpr (sizeof(Real) == 8) {
-                    grp_fx_c2r(B, W, R, P.lgNc, (const int4*)P.twx, (const int4*)P.prex, gout, fxred, ftid, NF, kBarFft);
+                    grp_fx_c2r<RMAX == 1>(B, W, R, P.lgNc, (const int4*)P.twx, (const int4*)P.prex, gout, fxred, ftid, NF, kBarFft);
                 } else if (!P.fft_r4) {
                     hr_c2r<C, ws_lg_lo(UPT, M), ws_lg_hi(UPT, M), PAIR>(P.lgNc, B, W, R, twp, (const C*)P.tw2, pre, gout, ftid, NF);
                 } else {
