@@ -273,8 +273,9 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
                     for (int i = tid; i < nr * per * Nc; i += nt) X[i] = W[i];
                     __syncthreads();
                 }
-                grp_fx_c2r<false>(X, W, nr * per, P.lgNc, (const int4*)P.twx, (const int4*)P.prex,
-                           RingOut2<C>{base, (size_t)((long long)dir * Nc), (size_t)P.n_theta * Nc, per}, fxred, tid, nt, kBarFft);
+                // rb > 1 only on short rings (band_config)
+                grp_fx_c2r<false, true>(X, W, nr * per, P.lgNc, (const int4*)P.twx, (const int4*)P.prex,
+                                        RingOut2<C>{base, (size_t)((long long)dir * Nc), (size_t)P.n_theta * Nc, per}, fxred, tid, nt, kBarFft);
                 __syncthreads();
                 continue;
             }
@@ -300,7 +301,10 @@ __global__ void __launch_bounds__(NT, NT == kBandThreads ? 2 : 1) segment_band_k
                 if (!P.fft_r4) hr_c2r<C, 2, 12, true>(P.lgNc, x, w, e - k, (const C*)P.tw, (const C*)P.tw2, pre, gout, tid, nt);
                 else grp_c2r_rt<C>(x, w, e - k, P.lgNc, (const C*)P.tw, pre, gout, tid, nt);
             } else {
-                grp_fx_c2r<false>(x, w, e - k, P.lgNc, (const int4*)P.twx, (const int4*)P.prex, gout, fxred, tid, nt, kBarFft);
+                if (P.lgNc <= kFxFlat)
+                    grp_fx_c2r<false, true>(x, w, e - k, P.lgNc, (const int4*)P.twx, (const int4*)P.prex, gout, fxred, tid, nt, kBarFft);
+                else
+                    grp_fx_c2r<false, false>(x, w, e - k, P.lgNc, (const int4*)P.twx, (const int4*)P.prex, gout, fxred, tid, nt, kBarFft);
                 __syncthreads();  // fxred serves the next run
             }
             k = e;

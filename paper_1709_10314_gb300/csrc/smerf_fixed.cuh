@@ -13,7 +13,7 @@
 // 1024 x 2048, p = 2, 16 realisations: 6.92 -> 2.27 ms a call; 20001 realisations of 32 x 64:
 // 10.9 -> 5.36 ms; 64 x 128, p = 1, Alg. 2's order: 205 -> 166 us; the error of the fields
 // against 64-bit references is unchanged (8.7e-13, 3.9e-15, 3.5e-15).  With the fixed-point ring FFT
-// (grp_fx_c2r) and the band kernel the same calls take 1.33 ms, 2.04 ms and 24.7 us.
+// (grp_fx_c2r) and the band kernel the same calls take 1.33 ms, 2.03 ms and 24.6 us.
 // Plain integer code: it compiles for the host too, where the tests hold it against long
 // arithmetic at the words' extremes.
 #pragma once
@@ -291,13 +291,15 @@ SMERF_HD int64_t fx_from_double(uint64_t bits, int S)
     if (e > 0 && k > -54) v = k >= 0 ? m << k : (m + (1ull << (-k - 1))) >> -k;
     return (int64_t)(bits >> 63 ? 0 - v : v);
 }
-// x 2^-S rounded to a double (below the normal range: 0)
-SMERF_HD uint64_t fx_to_double(int64_t x, int S)
+// x 2^-S rounded to a double (below the normal range: 0; above: infinity; TOP = false: S >= kFxTop, from
+// which on nothing lies above)
+constexpr int kFxTop = -960;
+template <bool TOP = true> SMERF_HD uint64_t fx_to_double(int64_t x, int S)
 {
     const uint64_t sign = (uint64_t)x & 0x8000000000000000ull, a = x < 0 ? 0 - (uint64_t)x : (uint64_t)x;
     const int n = fx_clz(a | 1), e = 1022 + 63 - n - S;
     const uint64_t m = a << n, bits = ((uint64_t)(uint32_t)e << 52) + (m >> 11) + ((m >> 10) & 1);
-    return a == 0 || e <= 0 ? sign : bits | sign;
+    return a == 0 || e <= 0 ? sign : (TOP && e > 2045 ? 0x7ff0000000000000ull : bits) | sign;
 }
 // a factor of magnitude at most 1 in units of 2^-62 as two signed words, hi 2^32 + lo
 SMERF_HD void fx_split(int64_t w, int32_t& hi, int32_t& lo)
@@ -343,7 +345,7 @@ template <class C> SMERF_HD C fx_cshift(C a, int d)
 // transform of 8 to 4096 points then errs by 0.2 to 0.9 of what the same passes in FP64 do, at
 // flat and falling spectra alike (at 2048 points, of the ring's deviation: flat 6.7e-17 against 2.4e-16,
 // m^-1/2 1.6e-16 against 2.2e-16, m^-2 1.2e-16 against 1.8e-16; one unit for the whole transform, that of the sum,
-// rounded the early passes to 2^-49 of a flat coefficient: 1.5e-15).
+// rounded the early passes to 2^-49 of a flat coefficient: 1.5e-15; up to 256 points one unit is as good).
 SMERF_HD unsigned fx_share(uint32_t h, int top)  // of 2^(top - 1039), rounded up but for a unit; h: high word of |v|
 {
     const int s = top - (int)(h >> 20);

@@ -1141,7 +1141,7 @@ __device__ __forceinline__ void grp_c2r_rt(C* buf0, C* buf1, int R, int lgNc, co
 // them the field's bits, depend on no thread count).  A field's
 // error against 64-bit references is 3.2e-15 at 64 x 128 (3.3e-15 with the FP64 FFT), 3.5e-15 at 32 x 64 (3.9e-15) and
 // 5.2e-13 at 1024 x 2048, p = 2 (8.6e-13; the tables' own error, set-up included).  That grid, 16 realisations: 2161 ->
-// 1332 us (with box_muller_call); 20001 of 32 x 64: 3057 -> 2036 us (with two realisations per CTA,
+// 1332 us (with box_muller_call); 20001 of 32 x 64: 3057 -> 2029 us (with two realisations per CTA,
 // band_config).  One unit for the whole transform took 1322 and 2014 us, and had fewer bits than FP64 from
 // 512 points on.
 // Factors e^{2 pi i k / n} are exact to 2^-62, stored as two words per component (int4: Re hi, lo, Im
@@ -1194,8 +1194,10 @@ __device__ __forceinline__ void grp_fx_scales(const double2* buf, int R, int lgN
 
 // C2R FFTs of R rings (coefficients in buf0 as double2, buf1 the second buffer), radix-4 passes
 // (radix 2 last when log2 Nc is odd); prex, twx: the plan's factors as int4; red: 2 kFxRings words; ONE: R is 1
-// (the units and shifts are then the same for every butterfly of a pass)
-template <bool ONE, class Out>
+// (the units and shifts are then the same for every butterfly of a pass); FLAT: lgNc is at most
+// kFxFlat, up to which one unit serves the whole transform (either build gives the same bits)
+constexpr int kFxFlat = 7;  // log2 Nc; 20001 realisations of 32 x 64: 2029 us with, 2054 without
+template <bool ONE, bool FLAT, class Out>
 __device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, int lgNc, const int4* __restrict__ twx,
                                            const int4* __restrict__ prex, Out gout, int* red, int ftid, int nf, int bar)
 {
@@ -1206,7 +1208,8 @@ __device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, 
     auto unit = [&](int r, int lgL) { return fx_unit(red[r], fx_spread(red[kFxRings + r]), lgL); };
     // to fixed point, in the unit after the first pass, and packed (c2r_pack) in place, the pair s, Nc - s
     // together
-    const int half = Nc / 2 + 1, lg1 = lgNc >= 2 ? 2 : 1;
+    const bool flat = FLAT || lgNc <= kFxFlat;
+    const int half = Nc / 2 + 1, lg1 = flat ? lgNc : 2;
     for (int b = ftid; b < R * half; b += nf) {
         const int r = ONE ? 0 : b / half, s = b - r * half, S = unit(r, lg1);
         auto get = [&](int i) {
@@ -1244,8 +1247,8 @@ __device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, 
                 v[3] = X[j + 3 * nb];
             }
             if (!first) {
-                const int d = fx_shift(fx_spread(red[kFxRings + r]), lgNs, LR);
-                v[0] = fx_cshift(v[0], d);
+                const int d = flat ? 0 : fx_shift(fx_spread(red[kFxRings + r]), lgNs, LR);
+                if (!FLAT) v[0] = fx_cshift(v[0], d);
                 v[1] = fxc_mul(v[1], __ldg(twx + off + kk), d);
                 if (RP == 4) {
                     v[2] = fxc_mul(v[2], __ldg(twx + off + Ns + kk), d);
@@ -1258,11 +1261,18 @@ __device__ __forceinline__ void grp_fx_c2r(double2* buf0, double2* buf1, int R, 
             if (last) {
                 const int S = unit(r, lgNc);
                 double2* D = gout[r] + idx;
+                if (S < kFxTop) {
+                    // values that may reach the top of the range; an infinity or NaN among the coefficients makes the
+                    // whole ring NaN, as in FP64
+                    auto conv = [&](int64_t x) { return __longlong_as_double(red[r] == 0x7ff ? 0x7ff8000000000000ll : (long long)fx_to_double(x, S)); };
+                    for (int a = 0; a < RP; ++a) __stcs(D + a * Ns, make_double2(conv(v[a].x), conv(v[a].y)));
+                    continue;
+                }
 #pragma unroll
                 for (int a = 0; a < 4; ++a)
                     if (a < RP)
-                        __stcs(D + a * Ns, make_double2(__longlong_as_double((long long)fx_to_double(v[a].x, S)),
-                                                        __longlong_as_double((long long)fx_to_double(v[a].y, S))));
+                        __stcs(D + a * Ns, make_double2(__longlong_as_double((long long)fx_to_double<false>(v[a].x, S)),
+                                                        __longlong_as_double((long long)fx_to_double<false>(v[a].y, S))));
             } else {
                 fxc* D = dst + (r << lgNc) + idx;
 #pragma unroll
@@ -1650,7 +1660,7 @@ __device__ __forceinline__ void ws_body(const SampleParams& P, int seg_index, in
                 }
                 if (RINGS && !whole) {
                 } else if constexpr (sizeof(Real) == 8) {
-                    grp_fx_c2r<RMAX == 1>(B, W, R, P.lgNc, (const int4*)P.twx, (const int4*)P.prex, gout, fxred, ftid, NF, kBarFft);
+                    grp_fx_c2r<RMAX == 1, false>(B, W, R, P.lgNc, (const int4*)P.twx, (const int4*)P.prex, gout, fxred, ftid, NF, kBarFft);
                 } else if (!P.fft_r4) {
                     hr_c2r<C, ws_lg_lo(UPT, M), ws_lg_hi(UPT, M), PAIR>(P.lgNc, B, W, R, twp, (const C*)P.tw2, pre, gout, ftid, NF);
                 } else {

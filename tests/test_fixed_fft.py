@@ -34,6 +34,7 @@ static fxc mul(fxc a, int64_t k, int lgn, int d)  // by e^{2 pi i k / 2^lgn}
 typedef std::complex<double> cd;
 static cd root(int64_t k, int lgn) { ld t = 2 * 3.14159265358979323846264338327950288L * k / ((ld)(1ll << lgn)); return cd((double)cosl(t), (double)sinl(t)); }
 
+extern "C" double to_double(int64_t x, int S) { return back(fx_to_double(x, S)); }
 // g: 2^lg coefficients (slot 0 = g_0, Re g_M); fx, fp: the ring's 2^(lg + 1) values; returns the largest
 // |component| of any intermediate value over 2^62
 extern "C" double transform(const double* g, int lg, double* fx, double* fp)
@@ -43,7 +44,8 @@ extern "C" double transform(const double* g, int lg, double* fx, double* fp)
     unsigned sum = 0;
     for (int i = 0; i < 2 * N; ++i) { int e = (int)((bits(g[i]) >> 52) & 0x7ff); if (e > top) top = e; }
     for (int i = 0; i < 2 * N; ++i) sum += fx_share((uint32_t)(bits(g[i]) >> 32) & 0x7fffffffu, top) + 1u;
-    const int spread = fx_spread(sum), S = fx_unit(top, spread, lg >= 2 ? 2 : 1);
+    const bool flat = lg <= 7;  // one unit for the whole transform (kFxFlat)
+    const int spread = fx_spread(sum), S = fx_unit(top, spread, flat ? lg : 2);
     std::vector<fxc> X(N), Y(N);
     std::vector<cd> A(N), B(N);
     double worst = 0;
@@ -63,7 +65,7 @@ extern "C" double transform(const double* g, int lg, double* fx, double* fp)
     }
     for (int s = 0; s < N; ++s) see(X[s]);
     for (int ln = 0; ln < lg;) {
-        const int LR = lg - ln >= 2 ? 2 : 1, R = 1 << LR, Ns = 1 << ln, nb = N >> LR, d = ln ? fx_shift(spread, ln, LR) : 0;
+        const int LR = lg - ln >= 2 ? 2 : 1, R = 1 << LR, Ns = 1 << ln, nb = N >> LR, d = ln && !flat ? fx_shift(spread, ln, LR) : 0;
         for (int j = 0; j < nb; ++j) {
             const int kk = j & (Ns - 1), idx = ((j - kk) << LR) + kk;
             fxc v[4];
@@ -168,3 +170,13 @@ def test_values_stay_below_the_bound(lib, lg):
     for g in cases:
         fx, fp, largest = _transform(lib, g)
         assert largest < 1 and fx < 2 * fp + 2.0 ** -106
+
+
+def test_overflow_is_infinity(lib):
+    """Fixed point to doubles at the top of their range: the largest finite value, then infinities."""
+    lib.to_double.restype = ctypes.c_double
+    one = lambda x, S: lib.to_double(ctypes.c_int64(x), S)  # noqa: E731
+    assert one(2 ** 62, -961) == 2.0 ** 1023 and one(-2 ** 62, -961) == -2.0 ** 1023
+    assert one(2 ** 53 - 1, -971) == np.finfo(np.float64).max
+    for x, S in ((2 ** 62, -962), (2 ** 62 - 1, -962), (2 ** 62, -1500), (2 ** 61, -964)):
+        assert one(x, S) == np.inf and one(-x, S) == -np.inf

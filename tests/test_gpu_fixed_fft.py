@@ -24,3 +24,17 @@ def test_every_second_point_of_a_whole_ring(kappa, n_phi, n):
     half = plan.sample(5, n).view(n, n_theta, n_phi // 2)
     err = float((whole[:, :, ::2] - half).abs().max() / whole.std())
     assert err < 4e-15
+
+
+@pytest.mark.parametrize("n_phi,n,H", [(64, 3, 4), (64, 1500, 4), (1024, 2, 4), (1024, 200, 4), (4096, 2, 0)])
+def test_rings_with_coefficients_that_are_not_finite(n_phi, n, H):
+    """A kappa that 12 rings do not resolve (its step grows as e^785) overflows the tables: the rings whose
+    coefficients are not finite are NaN throughout, as FP32's are, and no others."""
+    import torch
+    from paper_1709_10314_gb300 import SMERF_ORDER_PAPER, SMERF_RECUR_FP64, SMERF_TABLES_FP32, Plan
+    flags = SMERF_TABLES_FP32 | (0 if H else SMERF_ORDER_PAPER)
+    f32, f64 = (Plan([3000.0], 1.0, 12, n_phi, flags=flags | f, anchor_spacing=H).sample(5, n) for f in (0, SMERF_RECUR_FP64))
+    bad = torch.isnan(f64)
+    assert bool(bad.any()) and bool((bad.any(2) == bad.all(2)).all())
+    assert torch.equal(bad.any(2), torch.isnan(f32).any(2))
+    assert bool(torch.isfinite(f64[~bad]).all())
