@@ -374,8 +374,10 @@ int smerf_plan_set_rings(smerf_plan* plan, const int* n_phi_ring, const double* 
  * length); FP64 recursion offers 4 only.  The first five integers change launch parameters
  * only; the radix plan changes the FFT's rounding (FP32: ~1e-7 of the field std), so configurations
  * with the same radix plan give identical output.  Synchronous; allocates a temporary output;
- * must not run while other calls use the plan.  chosen (may be NULL) receives the chosen
- * configuration, all 0 when the plan's shape has no tunable kernel.
+ * must not run while other calls use the plan.  A request that runs on the band kernel (small ones, most
+ * ring-dependent plans) has nothing to tune: the plan keeps the built-in choice, which depends on
+ * each call's n_samples.  chosen (may be NULL) receives the chosen configuration (the built-in one
+ * of n_samples there), all 0 when the plan's shape has no tunable kernel.
  */
 #define SMERF_LAUNCH_INTS 6
 int smerf_plan_autotune(smerf_plan* plan, int n_samples, void* stream, int* chosen);

@@ -789,6 +789,20 @@ static int tune_candidates(const smerf_plan* plan, int* cand, int max_n)
                          : (plan->tab64 ? smerf_tune_candidates_fd(plan, cand, max_n) : smerf_tune_candidates_ff(plan, cand, max_n));
 }
 
+static int request_launch(const smerf_plan* plan, int n, int* c)
+{
+    return plan->recur64 ? (plan->tab64 ? smerf_request_launch_dd(plan, n, c) : smerf_request_launch_df(plan, n, c))
+                         : (plan->tab64 ? smerf_request_launch_fd(plan, n, c) : smerf_request_launch_ff(plan, n, c));
+}
+
+// the same launch but for the radix plan (an FFT length without a high-radix plan takes radix 4 either way)
+static bool same_launch(const int* a, const int* b)
+{
+    for (int k = 0; k < smerf::kLaunchInts - 1; ++k)
+        if (a[k] != b[k]) return false;
+    return true;
+}
+
 int smerf_plan_launch_candidates(const smerf_plan* plan, int* cand, int max_n)
 {
     if (!plan || max_n < 0 || (max_n > 0 && !cand)) return SMERF_EINVAL;
@@ -847,6 +861,20 @@ int smerf_plan_autotune(smerf_plan* plan, int n_samples, void* stream, int* chos
             for (int k = 0; k < smerf::kLaunchInts; ++k) chosen[k] = 0;
         return SMERF_OK;  // no warp-specialised configuration: the built-in choice stays
     }
+    int builtin[smerf::kLaunchInts];
+    const int band = request_launch(plan, n_samples, builtin);
+    if (band < 0) return band;
+    if (band) {
+        // every configuration would time the band kernel's one launch: the built-in choice, which depends
+        // on the count of a call, stays
+        for (int i = 0; chosen && i < nc; ++i) {
+            const int* c = cand + smerf::kLaunchInts * i;
+            if (same_launch(c, builtin))
+                for (int k = 0; k < smerf::kLaunchInts; ++k) chosen[k] = c[k];
+            if (same_launch(c, builtin) && c[smerf::kLaunchInts - 1] == builtin[smerf::kLaunchInts - 1]) break;
+        }
+        return SMERF_OK;
+    }
     cudaStream_t st = (cudaStream_t)stream;
     const size_t ob = (size_t)n_samples * plan_points(plan) * (plan->recur64 ? 8 : 4);
     void* out = nullptr;
@@ -862,6 +890,9 @@ int smerf_plan_autotune(smerf_plan* plan, int n_samples, void* stream, int* chos
     int bi = -1;
     for (int i = 0; rc == SMERF_OK && i < nc; ++i) {
         set_tune(plan, cand + smerf::kLaunchInts * i);
+        int runs[smerf::kLaunchInts];
+        // ring-dependent longitudes: not a configuration with a ring build (or the band kernel takes it)
+        if (request_launch(plan, n_samples, runs) != 0 || !same_launch(runs, cand + smerf::kLaunchInts * i)) continue;
         float tot = 0.0f;
         for (int it = 0; rc == SMERF_OK && it < 4; ++it) {
             rc = smerf_launch_sample_staged(plan, 1 + it, n_samples, out, scratch,

@@ -315,8 +315,11 @@ SMERF_DECLARE_QUEUE(ff)
 SMERF_DECLARE_QUEUE(fd)
 
 // launch-configuration candidates of a plan for the autotuner (per precision pair XX):
-// writes up to max_n (upt, rmax, np, nf, minb) tuples of kLaunchInts, returns how many
-#define SMERF_DECLARE_TUNE(XX) int smerf_tune_candidates_##XX(const smerf_plan* pl, int* cand, int max_n);
+// writes up to max_n (upt, rmax, np, nf, minb) tuples of kLaunchInts, returns how many; the launch of a
+// request of n realisations, 1 if it runs on the band kernel instead
+#define SMERF_DECLARE_TUNE(XX)                                              \
+    int smerf_tune_candidates_##XX(const smerf_plan* pl, int* cand, int max_n); \
+    int smerf_request_launch_##XX(const smerf_plan* pl, int n, int* c);
 SMERF_DECLARE_TUNE(ff)
 SMERF_DECLARE_TUNE(fd)
 SMERF_DECLARE_TUNE(dd)

@@ -2679,6 +2679,20 @@ int queue_ctas(size_t smem)
     return (per1 < per2 ? per1 : per2) * sms;
 }
 
+// The launch of a request's segments: c as kLaunchInts integers (0: not warp-specialised); 1 if it runs on
+// the band kernel instead, 0 if not, or a negative status
+template <class Real, class TabT>
+int request_launch(const smerf_plan* pl, int n, int* c)
+{
+    SampleParams P;
+    SegConfig cfg;
+    const int rc = fill_params<Real, TabT>(pl, 0, n, nullptr, nullptr, P, cfg);
+    if (rc != SMERF_OK) return rc;
+    const int v[kLaunchInts] = {cfg.upt, cfg.rmax, cfg.np, cfg.nt - cfg.np, cfg.minb, cfg.radix};
+    for (int k = 0; k < kLaunchInts; ++k) c[k] = cfg.ws ? v[k] : 0;
+    return cfg.band_splits > 0 ? 1 : 0;
+}
+
 template <class Real, class TabT>
 int fill_params_c(const smerf_plan* pl, uint64_t seed, int n, void* out, void* scratch, SampleParams* P,
                   int* batchable, int* rmax)
@@ -2760,6 +2774,7 @@ int launch_group_m(const smerf_plan* rep, const SampleParams* d, const int4* anc
     {                                                                                                       \
         return smerf::tune_candidates<REAL>(pl, cand, max_n);                                               \
     }                                                                                                            \
+    int smerf_request_launch_##XX(const smerf_plan* pl, int n, int* c) { return smerf::request_launch<REAL, TABT>(pl, n, c); } \
     size_t smerf_ws_smem_##XX(const smerf_plan* pl, int rmax) { return smerf::ws_smem<REAL>(pl, rmax); }
 
 // The persistent batch launch of an FP32-recursion precision pair (its own translation unit,
