@@ -185,7 +185,8 @@ int smerf_last_device_status(void* stream);
  * the host path) stream-ordered from that pool, which keeps it between calls so that a call
  * after a synchronisation maps no new memory; the pool holds at most the largest amount that
  * calls in flight used together.  Plan creation takes temporaries of up to 128 MB from the same
- * pool.  SMERF_OK, or SMERF_ECUDA.
+ * pool, at most 512 MB of it over all creations in flight (beyond that from the device's default pool).
+ * SMERF_OK, or SMERF_ECUDA.
  */
 int smerf_scratch_trim(void);
 

@@ -258,6 +258,22 @@ cudaError_t smerf_scratch_alloc(void** p, size_t bytes, int dev, cudaStream_t st
     return pool ? smerf::dev_malloc_pool(p, bytes, pool, st) : smerf::dev_malloc_async(p, bytes, st);
 }
 
+static std::atomic<size_t> g_setup_pooled(0);
+
+bool smerf_setup_reserve(size_t bytes, size_t* held)
+{
+    if (bytes <= *held) return true;
+    const size_t more = bytes - *held;
+    size_t now = g_setup_pooled.load();
+    do {
+        if (now + more > ((size_t)512 << 20)) return false;
+    } while (!g_setup_pooled.compare_exchange_weak(now, now + more));
+    *held = bytes;
+    return true;
+}
+
+void smerf_setup_release(size_t held) { g_setup_pooled.fetch_sub(held); }
+
 // allocation-failure injection (smerf_debug_fail_alloc): -1 = off, k >= 0 = the allocation
 // after k more succeeds fails
 static std::atomic<long> g_alloc_countdown(-1);
@@ -318,7 +334,7 @@ static int check_grid(int p, double A, int n_theta, int n_phi, unsigned flags, i
 
 static int create_plan(const double* kappa, const double* kh_re, const double* kh_im, int complex_spec, int p,
                        double A, int n_theta, int n_phi, unsigned flags, int anchor_spacing, smerf_plan** out_plan,
-                       cudaStream_t st = 0, bool sync = true, const double* theta = nullptr);
+                       cudaStream_t st = 0, size_t* held = nullptr, const double* theta = nullptr);
 
 // ring colatitudes of an iso-latitude grid: finite, strictly increasing inside (0, pi) (any such
 // set of rings: the Markov property along the colatitude holds on every iso-latitude grid, Sec. 2)
@@ -331,9 +347,10 @@ static int check_colatitudes(const double* theta, int n_theta)
     return SMERF_OK;
 }
 
-// smerf_plan_create_ex with the set-up ordered on `st` (sync: wait for it)
+// smerf_plan_create_ex with the set-up ordered on `st`; held: the stream's share of the scratch pool, kept by
+// a caller that waits for the stream itself (null: wait here)
 static int create_ex_on(const double* kappa, int p, double A, int n_theta, int n_phi, unsigned flags,
-                        int anchor_spacing, smerf_plan** out_plan, cudaStream_t st, bool sync)
+                        int anchor_spacing, smerf_plan** out_plan, cudaStream_t st, size_t* held)
 {
     if (!out_plan) return SMERF_EINVAL;
     *out_plan = nullptr;
@@ -349,13 +366,13 @@ static int create_ex_on(const double* kappa, int p, double A, int n_theta, int n
         }
     double kr[kMaxP + 1] = {0}, ki[kMaxP + 1] = {0};
     for (int i = 0; i < p && i <= kMaxP; ++i) kr[i] = kappa[i] * kappa[i];
-    return create_plan(kappa, kr, ki, 0, p, A, n_theta, n_phi, flags, anchor_spacing, out_plan, st, sync);
+    return create_plan(kappa, kr, ki, 0, p, A, n_theta, n_phi, flags, anchor_spacing, out_plan, st, held);
 }
 
 int smerf_plan_create_ex(const double* kappa, int p, double A, int n_theta, int n_phi,
                          unsigned flags, int anchor_spacing, smerf_plan** out_plan)
 {
-    return create_ex_on(kappa, p, A, n_theta, n_phi, flags, anchor_spacing, out_plan, 0, true);
+    return create_ex_on(kappa, p, A, n_theta, n_phi, flags, anchor_spacing, out_plan, 0, nullptr);
 }
 
 int smerf_plan_create_many(const smerf_plan_spec* specs, int n, smerf_plan** out_plans)
@@ -366,6 +383,7 @@ int smerf_plan_create_many(const smerf_plan_spec* specs, int n, smerf_plan** out
     // the set-ups go round-robin onto a few non-blocking streams and overlap on the GPU
     const int ns = n < 16 ? n : 16;
     std::vector<cudaStream_t> streams((size_t)ns, nullptr);
+    std::vector<size_t> held((size_t)ns, 0);
     int rc = SMERF_OK;
     for (int k = 0; k < ns && rc == SMERF_OK; ++k)
         if (cudaStreamCreateWithFlags(&streams[k], cudaStreamNonBlocking) != cudaSuccess) rc = SMERF_ECUDA;
@@ -373,11 +391,12 @@ int smerf_plan_create_many(const smerf_plan_spec* specs, int n, smerf_plan** out
     for (int i = 0; i < n && rc == SMERF_OK; ++i) {
         const smerf_plan_spec& q = specs[i];
         rc = create_ex_on(q.kappa, q.p, q.A, q.n_theta, q.n_phi, q.flags, q.anchor_spacing, &out_plans[i],
-                          streams[i % ns], false);
+                          streams[i % ns], &held[i % ns]);
     }
     for (int k = 0; k < ns; ++k) {
         if (!streams[k]) continue;
         if (cudaStreamSynchronize(streams[k]) != cudaSuccess && rc == SMERF_OK) rc = SMERF_ECUDA;
+        smerf_setup_release(held[k]);
         cudaStreamDestroy(streams[k]);
     }
     const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -436,7 +455,7 @@ static int create_khat(const double* khat_re, const double* khat_im, int p, doub
             const double s = fmax(hypot(khat_re[i], khat_im[i]), hypot(khat_re[j], khat_im[j]));
             if (d < 1e-6 * s) return SMERF_EILLCOND;
         }
-    return create_plan(nullptr, khat_re, khat_im, 1, p, A, n_theta, n_phi, flags, anchor_spacing, out_plan, 0, true,
+    return create_plan(nullptr, khat_re, khat_im, 1, p, A, n_theta, n_phi, flags, anchor_spacing, out_plan, 0, nullptr,
                        theta);
 }
 
@@ -458,7 +477,7 @@ int smerf_plan_create_khat_theta(const double* khat_re, const double* khat_im, i
 
 static int create_plan(const double* kappa, const double* kh_re, const double* kh_im, int complex_spec, int p,
                        double A, int n_theta, int n_phi, unsigned flags, int anchor_spacing, smerf_plan** out_plan,
-                       cudaStream_t st, bool sync, const double* theta)
+                       cudaStream_t st, size_t* held, const double* theta)
 {
     if (p > kMaxP) return SMERF_EUNSUPPORTED;
     if (!is_pow2(n_phi) || n_phi < 8 || n_phi > 32768) return SMERF_EUNSUPPORTED;
@@ -540,7 +559,11 @@ static int create_plan(const double* kappa, const double* kh_re, const double* k
             if (cudaMemcpy(pl->theta_dev, both.data(), 2 * tb, cudaMemcpyHostToDevice) != cudaSuccess) rc = SMERF_ECUDA;
         }
     }
-    if (rc == SMERF_OK) rc = smerf_setup_tables(pl, st, sync);
+    if (rc == SMERF_OK) {
+        size_t own = 0;
+        rc = smerf_setup_tables(pl, st, !held, held ? held : &own);
+        smerf_setup_release(own);
+    }
     if (rc != SMERF_OK) {
         free_plan_memory(pl);
         delete pl;
@@ -568,7 +591,7 @@ int smerf_plan_create_theta(const double* kappa, int p, double A, int n_theta, c
         }
     double kr[kMaxP + 1] = {0}, ki[kMaxP + 1] = {0};
     for (int i = 0; i < p && i <= kMaxP; ++i) kr[i] = kappa[i] * kappa[i];
-    return create_plan(kappa, kr, ki, 0, p, A, n_theta, n_phi, flags, anchor_spacing, out_plan, 0, true, theta);
+    return create_plan(kappa, kr, ki, 0, p, A, n_theta, n_phi, flags, anchor_spacing, out_plan, 0, nullptr, theta);
 }
 
 int smerf_plan_create(const double* kappa, int p, double A, int n_theta, int n_phi, unsigned flags,
@@ -945,7 +968,7 @@ int smerf_plan_autotune_anchor(smerf_plan* plan, int n_samples, const int* candi
     for (int i = 0; rc == SMERF_OK && i < n_cand; ++i) {
         smerf_plan* cp = nullptr;
         rc = create_plan(plan->p > 0 ? plan->kappa : nullptr, plan->khat_re, plan->khat_im, plan->complex_spec, plan->p,
-                         plan->A, plan->n_theta, plan->n_phi, plan->flags, candidates[i], &cp, 0, true, plan->theta_host);
+                         plan->A, plan->n_theta, plan->n_phi, plan->flags, candidates[i], &cp, 0, nullptr, plan->theta_host);
         if (rc != SMERF_OK) break;
         cp->tune = plan->tune;  // the plan's launch configuration, if it fixed one
         const size_t sb = (smerf_scratch_bytes(cp, n_samples) + 255) / 256 * 256;

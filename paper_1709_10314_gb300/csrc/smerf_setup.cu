@@ -996,15 +996,15 @@ __global__ void repack_rows_kernel(const float* __restrict__ rows, float* __rest
 }
 
 // A set-up's temporaries: from the library's scratch pool (which keeps its memory between calls, so
-// that a program that makes plan after plan maps none), or, when large, from the default pool,
-// which returns them at the set-up's end
-cudaError_t setup_alloc(void** p, size_t bytes, int dev, cudaStream_t st)
+// that a program that makes plan after plan maps none), or, when large or beyond the share of the
+// pool that set-ups have, from the default pool, which returns them at the set-up's end
+cudaError_t setup_alloc(void** p, size_t bytes, bool pooled, int dev, cudaStream_t st)
 {
-    return bytes <= ((size_t)128 << 20) ? smerf_scratch_alloc(p, bytes, dev, st) : smerf::dev_malloc_async(p, bytes, st);
+    return pooled ? smerf_scratch_alloc(p, bytes, dev, st) : smerf::dev_malloc_async(p, bytes, st);
 }
 
 template <int M>
-int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
+int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync, size_t* held)
 {
     int rc = SMERF_OK;
     Spec sp;
@@ -1111,8 +1111,9 @@ int setup_impl(smerf_plan* pl, cudaStream_t st, bool sync)
             }
             if (len > 0) {
                 const size_t nb = (size_t)(len + 1) * pl->n_modes * M * M * sizeof(double);
-                CK(setup_alloc((void**)&phi, nb, pl->dev, st));
-                CK(setup_alloc((void**)&qv, nb, pl->dev, st));
+                const bool pooled = nb <= ((size_t)128 << 20) && smerf_setup_reserve(2 * nb, held);
+                CK(setup_alloc((void**)&phi, nb, pooled, pl->dev, st));
+                CK(setup_alloc((void**)&qv, nb, pooled, pl->dev, st));
                 if (len > 65535) { rc = SMERF_EUNSUPPORTED; goto done; }
                 dim3 grid(gm, len);
                 if (pl->complex_spec) step_kernel_c<M><<<grid, threads, 0, st>>>(sc, len, phi, qv);
@@ -1202,12 +1203,12 @@ int smerf_start_ring(const double* theta, int n_theta)
     return k0;
 }
 
-int smerf_setup_tables(smerf_plan* pl, cudaStream_t st, bool sync)
+int smerf_setup_tables(smerf_plan* pl, cudaStream_t st, bool sync, size_t* held)
 {
     switch (pl->p) {
-        case 1: return setup_impl<1>(pl, st, sync);
-        case 2: return setup_impl<2>(pl, st, sync);
-        case 3: return setup_impl<3>(pl, st, sync);
+        case 1: return setup_impl<1>(pl, st, sync, held);
+        case 2: return setup_impl<2>(pl, st, sync, held);
+        case 3: return setup_impl<3>(pl, st, sync, held);
         default: return SMERF_EUNSUPPORTED;
     }
 }
