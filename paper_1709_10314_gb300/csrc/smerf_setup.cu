@@ -158,16 +158,6 @@ template <> __device__ inline Mat<2> minv<2>(const Mat<2>& x)
 }
 template <> __device__ inline Mat<3> minv<3>(const Mat<3>& x) { return inv3<Mat<3>, double>(x); }
 
-// 1/x by two Newton steps r += r (1 - x r) from the hardware's approximation (20 bits), within an
-// ulp; x normal and well inside the range.  A division costs twice its FP64 instructions.
-__device__ inline double rcp_newton(double x)
-{
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(r, fma(-x, r, 1.0), r);
-    return fma(r, fma(-x, r, 1.0), r);
-}
-
 // lower Cholesky factor of a symmetric positive semi-definite matrix (0 where it degenerates)
 template <int M> __device__ inline Mat<M> mchol(const Mat<M>& x)
 {

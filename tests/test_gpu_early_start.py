@@ -42,3 +42,34 @@ def test_plans_in_turn_on_one_stream(n_theta, n_phi, H, n):
             o.zero_()
             p.sample(20, n, out=o)
         assert torch.equal(outs[0], ref[0]) and torch.equal(outs[1], ref[1])
+
+
+@pytest.mark.parametrize("p,n_theta,n_phi,H,n,fp64,tables64", [
+    (1, 64, 128, 0, 1, True, False),
+    (2, 181, 512, 16, 1, False, False),
+    (2, 40, 128, 4, 4, False, True),     # tables converted ahead of the tiles
+    (2, 100, 512, 0, 4, False, True),    # tables converted beside the anchors: no early start
+    (2, 32, 64, 0, 1200, True, False),   # two realisations per CTA
+])
+def test_small_requests_captured_and_replayed(p, n_theta, n_phi, H, n, fp64, tables64):
+    """A captured small request (an early start is a programmatic edge of the graph) gives the call's field at
+    every replay, alone and between other work on the stream."""
+    import torch
+    from paper_1709_10314_gb300 import SMERF_ORDER_PAPER, SMERF_RECUR_FP64, SMERF_TABLES_FP64, Plan
+    flags = (SMERF_RECUR_FP64 if fp64 else 0) | (SMERF_TABLES_FP64 if tables64 else 0) | (0 if H else SMERF_ORDER_PAPER)
+    plan = Plan([6.0, 15.0][:p], 1.0, n_theta, n_phi, flags=flags, anchor_spacing=H)
+    ref = plan.sample(9, n)
+    out, s, g = torch.empty_like(ref), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s):
+        plan.sample(9, n, out=out)  # the first launch outside the capture
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s, capture_error_mode="relaxed"):
+        plan.sample(9, n, out=out)
+    for other in (False, True, True):
+        out.zero_()
+        torch.cuda.synchronize()
+        if other:
+            plan.sample(10, n, out=torch.empty_like(out))
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
