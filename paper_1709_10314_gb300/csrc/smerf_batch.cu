@@ -71,14 +71,20 @@ int queue_ctas(int kind, size_t smem)
     return kind == kFF ? smerf_queue_ctas_ff(smem) : smerf_queue_ctas_fd(smem);
 }
 
+int group_np(int kind, const smerf_plan* rep, int n)
+{
+    return kind == kFF ? smerf_group_np_ff(rep, n) : kind == kFD ? smerf_group_np_fd(rep, n) : kind == kDD ? smerf_group_np_dd(rep, n)
+                                                                                            : smerf_group_np_df(rep, n);
+}
+
 int launch_group(int kind, const smerf_plan* rep, const SampleParams* d, const int4* a, int na, const int4* s, int ns,
-                 cudaStream_t st)
+                 int n, cudaStream_t st)
 {
     switch (kind) {
-        case kFF: return smerf_launch_group_ff(rep, d, a, na, s, ns, st);
-        case kFD: return smerf_launch_group_fd(rep, d, a, na, s, ns, st);
-        case kDD: return smerf_launch_group_dd(rep, d, a, na, s, ns, st);
-        default: return smerf_launch_group_df(rep, d, a, na, s, ns, st);
+        case kFF: return smerf_launch_group_ff(rep, d, a, na, s, ns, n, st);
+        case kFD: return smerf_launch_group_fd(rep, d, a, na, s, ns, n, st);
+        case kDD: return smerf_launch_group_dd(rep, d, a, na, s, ns, n, st);
+        default: return smerf_launch_group_df(rep, d, a, na, s, ns, n, st);
     }
 }
 
@@ -89,6 +95,7 @@ struct Group {
     int n_anc = 0;
     int4* d_seg = nullptr;
     int n_seg = 0;
+    int n = 1;  // realisations of `rep` with as many segments in all (chooses the launch)
 };
 
 }  // namespace
@@ -208,6 +215,9 @@ int smerf_batch_create(const smerf_plan* const* plans, const int* n_samples, int
         gr.n_anc = (int)anc[g].size();
         gr.n_seg = (int)seg[g].size();
         if (queued(gr.kind, gr.rep->p)) continue;  // its items go to the persistent queue below
+        gr.n = (gr.n_seg + gr.rep->n_segments - 1) / gr.rep->n_segments;
+        const int np = group_np(gr.kind, gr.rep, gr.n);
+        for (const int4& it : seg[g]) b->h_descs[it.x].np = np;
         if (smerf::dev_malloc((void**)&gr.d_anc, sizeof(int4) * gr.n_anc) != cudaSuccess ||
             smerf::dev_malloc((void**)&gr.d_seg, sizeof(int4) * gr.n_seg) != cudaSuccess) {
             rc = SMERF_ENOMEM;
@@ -342,7 +352,7 @@ int smerf_batch_launch(smerf_batch* b, void* stream)
     }
     for (const Group& g : b->groups) {
         if (queued(g.kind, g.rep->p)) continue;
-        const int rc = launch_group(g.kind, g.rep, b->d_descs, g.d_anc, g.n_anc, g.d_seg, g.n_seg, st);
+        const int rc = launch_group(g.kind, g.rep, b->d_descs, g.d_anc, g.n_anc, g.d_seg, g.n_seg, g.n, st);
         if (rc != SMERF_OK) return rc;
     }
     for (int i : b->singles) {

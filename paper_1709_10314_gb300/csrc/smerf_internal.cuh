@@ -295,13 +295,16 @@ int smerf_launch_sample(const smerf_plan* plan, uint64_t seed, int n_samples, vo
 size_t smerf_scratch_bytes(const smerf_plan* plan, int n_samples);
 // batched launches (smerf_batch.cu): per precision pair XX in {ff, fd, dd, df}
 //   smerf_fill_params_XX: the request's SampleParams and whether it can join a batched group
-//   smerf_launch_group_XX: one anchor and one segment launch over a group's work items
+//   smerf_launch_group_XX: one anchor and one segment launch over a group's work items, in the launch
+//     configuration of n realisations of `rep` (one realisation per CTA in all of them)
+//   smerf_group_np_XX: that configuration's producer threads, for the group's descriptors
 #define SMERF_DECLARE_GROUP(XX)                                                                   \
     int smerf_fill_params_##XX(const smerf_plan* pl, uint64_t seed, int n, void* out, void* scratch, \
                                smerf::SampleParams* P, int* batchable, int* rmax);                 \
     int smerf_launch_group_##XX(const smerf_plan* rep, const smerf::SampleParams* d_descs,          \
-                                const int4* anc_items, int n_anc, const int4* seg_items, int n_seg,  \
-                                cudaStream_t st);
+                                const int4* anc_items, int n_anc, const int4* seg_items, int n_seg, int n, \
+                                cudaStream_t st);                                                   \
+    int smerf_group_np_##XX(const smerf_plan* rep, int n);
 SMERF_DECLARE_GROUP(ff)
 SMERF_DECLARE_GROUP(fd)
 SMERF_DECLARE_GROUP(dd)

@@ -2101,7 +2101,7 @@ inline bool seg_choice(const smerf_plan* pl, int n, int& upt, int& rmax, int& nf
     return false;
 }
 
-// n: the realisations of the call (0: a batch's descriptors, whose launch must not depend on it)
+// n: the realisations of the call, or those of its first plan that a batch's group comes to (0: not known yet)
 template <class Real>
 inline SegConfig seg_config(const smerf_plan* pl, int n)
 {
@@ -2707,9 +2707,9 @@ int fill_params_c(const smerf_plan* pl, uint64_t seed, int n, void* out, void* s
 // One anchor and one segment launch over a batched group's work items (state size M = p).
 template <class Real, class TabT, int M>
 int launch_group_m(const smerf_plan* rep, const SampleParams* d, const int4* anc_items, int n_anc,
-                   const int4* seg_items, int n_seg, cudaStream_t st)
+                   const int4* seg_items, int n_seg, int n, cudaStream_t st)
 {
-    const SegConfig cfg = seg_config<Real>(rep, 0);
+    const SegConfig cfg = seg_config<Real>(rep, n);
     if (!cfg.ws) return SMERF_EUNSUPPORTED;
     if (n_anc > 0) {
         anchor_batched_kernel<Real, TabT, M><<<n_anc, 128, 0, st>>>(d, anc_items);
@@ -2730,10 +2730,10 @@ int launch_group_m(const smerf_plan* rep, const SampleParams* d, const int4* anc
         return smerf::launch_sample_m<REAL, TABT, M>(pl, seed, n, out, scratch, st, ev0, ev1);           \
     }                                                                                                     \
     int smerf_launch_group_##XX##_p##M(const smerf_plan* rep, const smerf::SampleParams* d,               \
-                                       const int4* anc_items, int n_anc, const int4* seg_items, int n_seg, \
+                                       const int4* anc_items, int n_anc, const int4* seg_items, int n_seg, int n, \
                                        cudaStream_t st)                                                   \
     {                                                                                                     \
-        return smerf::launch_group_m<REAL, TABT, M>(rep, d, anc_items, n_anc, seg_items, n_seg, st);     \
+        return smerf::launch_group_m<REAL, TABT, M>(rep, d, anc_items, n_anc, seg_items, n_seg, n, st);     \
     }
 
 // The precision pair's entry points (smerf_sample_XX.cu): dispatch on p to the instantiations.
@@ -2745,11 +2745,11 @@ int launch_group_m(const smerf_plan* rep, const SampleParams* d, const int4* anc
     int smerf_launch_sample_##XX##_p3(const smerf_plan*, uint64_t, int, void*, void*, cudaStream_t, cudaEvent_t, \
                                       cudaEvent_t);                                                         \
     int smerf_launch_group_##XX##_p1(const smerf_plan*, const smerf::SampleParams*, const int4*, int,       \
-                                     const int4*, int, cudaStream_t);                                       \
+                                     const int4*, int, int, cudaStream_t);                                       \
     int smerf_launch_group_##XX##_p2(const smerf_plan*, const smerf::SampleParams*, const int4*, int,       \
-                                     const int4*, int, cudaStream_t);                                       \
+                                     const int4*, int, int, cudaStream_t);                                       \
     int smerf_launch_group_##XX##_p3(const smerf_plan*, const smerf::SampleParams*, const int4*, int,       \
-                                     const int4*, int, cudaStream_t);                                       \
+                                     const int4*, int, int, cudaStream_t);                                       \
     int smerf_launch_sample_##XX(const smerf_plan* pl, uint64_t seed, int n, void* out, void* scratch,      \
                                  cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1)                         \
     {                                                                                                       \
@@ -2763,13 +2763,14 @@ int launch_group_m(const smerf_plan* rep, const SampleParams* d, const int4* anc
         return smerf::fill_params_c<REAL, TABT>(pl, seed, n, out, scratch, P, batchable, rmax);             \
     }                                                                                                       \
     int smerf_launch_group_##XX(const smerf_plan* rep, const smerf::SampleParams* d_descs,                  \
-                                const int4* anc_items, int n_anc, const int4* seg_items, int n_seg,         \
+                                const int4* anc_items, int n_anc, const int4* seg_items, int n_seg, int n, \
                                 cudaStream_t st)                                                            \
     {                                                                                                       \
-        return rep->p == 1   ? smerf_launch_group_##XX##_p1(rep, d_descs, anc_items, n_anc, seg_items, n_seg, st) \
-               : rep->p == 2 ? smerf_launch_group_##XX##_p2(rep, d_descs, anc_items, n_anc, seg_items, n_seg, st) \
-                             : smerf_launch_group_##XX##_p3(rep, d_descs, anc_items, n_anc, seg_items, n_seg, st); \
+        return rep->p == 1   ? smerf_launch_group_##XX##_p1(rep, d_descs, anc_items, n_anc, seg_items, n_seg, n, st) \
+               : rep->p == 2 ? smerf_launch_group_##XX##_p2(rep, d_descs, anc_items, n_anc, seg_items, n_seg, n, st) \
+                             : smerf_launch_group_##XX##_p3(rep, d_descs, anc_items, n_anc, seg_items, n_seg, n, st); \
     }                                                                                                       \
+    int smerf_group_np_##XX(const smerf_plan* rep, int n) { return smerf::seg_config<REAL>(rep, n).np; }         \
     int smerf_tune_candidates_##XX(const smerf_plan* pl, int* cand, int max_n)                              \
     {                                                                                                       \
         return smerf::tune_candidates<REAL>(pl, cand, max_n);                                               \

@@ -60,3 +60,26 @@ def test_tuning_a_ring_plan_takes_a_configuration_with_a_ring_build():
     assert "segment_ws_kernel" in captured(lambda: plan.sample(3, 16, out=out))[0][-1]
     if chosen[5] == 16:
         assert torch.equal(plan.sample(3, 16), ref)
+
+
+def test_a_batch_group_takes_the_launch_of_its_size():
+    """p = 3 requests of one shape: few of them the launch of as many segments of a single call (large CTAs, one
+    wave), many the throughput launch; the same fields."""
+    import re
+    import torch
+    from paper_1709_10314_gb300 import Batch
+    plans = [_plan((10.0 + 0.3 * i, 20.0, 40.0), 64, 2048, 4) for i in range(24)]
+
+    def run(plans, counts):
+        b = Batch(plans, counts)
+        outs = [torch.full((n, p.n_theta, p.n_phi), float("nan"), device="cuda") for p, n in zip(plans, counts)]
+        b.sample(list(range(len(plans))), outs)
+        for i, (p, n, o) in enumerate(zip(plans, counts, outs)):
+            assert torch.equal(o, p.sample(i, n))
+        name = captured(b.launch)[0][-1]
+        b.close()
+        return re.search(r"Li3ELi(\d)ELi1ELi1E", name).group(1)
+
+    upt = lambda n: re.search(r"Li3ELi(\d)ELi1ELi1E", _kernel(plans[0], n)).group(1)  # noqa: E731
+    few, many = run(plans[:2], [1, 1]), run(plans, [3] * 24)
+    assert few == upt(2) and many == upt(72) and few != many
