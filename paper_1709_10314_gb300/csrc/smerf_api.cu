@@ -736,7 +736,8 @@ int smerf_plan_set_rings(smerf_plan* plan, const int* n_phi_ring, const double* 
         const double p0 = phi0_ring ? phi0_ring[k] : 0.0;
         if ((nk & 1) || nk < 4 || nk > plan->n_phi || !isfinite(p0)) return SMERF_EINVAL;
         n[k] = nk;
-        // the offset as a signed 64-bit fraction of a turn (2^-65 turns off at most)
+        // the offset as a signed 64-bit fraction of a turn (off by FP64's rounding of phi0 / pi,
+        // 2^-53 turns within a turn)
         double turns = 0.5 * fmod(p0 / SMERF_PI, 2.0);
         turns -= rint(turns);
         if (turns >= 0.5) turns -= 1.0;

@@ -15,7 +15,7 @@
 // segment's start (they are cheap) and synthesises only its own share of the rings.
 // Rings with their own point count: smerf_ragged.cuh, a group of threads per ring.  One FP64
 // realisation of 64 x 128 in Alg. 2's order: 166 -> 24.6 us (the fixed-point FFT among them); one of
-// 181 x 512, p = 2: 31.1 -> 22.7 us (the anchor tiles among them).
+// 181 x 512, p = 2: 31 -> 20 to 24 us between runs (the anchor tiles among them).
 #pragma once
 
 namespace smerf {
@@ -23,8 +23,7 @@ namespace smerf {
 constexpr int kBandThreads = 256;      // two CTAs per SM
 constexpr int kBandThreadsFew = 512;   // requests of at most one CTA per SM (band_config)
 
-// Table rows of unit u at one position, G rows of step_row(M) values, converted to Real; ny: the
-// Nyquist chain's row (unit 0 only)
+// Table rows of unit u at one position, G rows of step_row(M) values, converted to Real
 template <class Real, class TabT, int M>
 __device__ __forceinline__ void band_rows(const TabT* tb, int u, Real (&t)[kG<M>][step_row(M)])
 {

@@ -13,7 +13,7 @@
 // 1024 x 2048, p = 2, 16 realisations: 6.92 -> 2.27 ms a call; 20001 realisations of 32 x 64:
 // 10.9 -> 5.36 ms; 64 x 128, p = 1, Alg. 2's order: 205 -> 166 us; the error of the fields
 // against 64-bit references is unchanged (8.7e-13, 3.9e-15, 3.5e-15).  With the fixed-point ring FFT
-// (grp_fx_c2r) and the band kernel the same calls take 1.33 ms, 2.03 ms and 24.6 us.
+// (grp_fx_c2r) and the band kernel the same calls take 1.34 ms, 2.03 ms and 24.6 us.
 // Plain integer code: it compiles for the host too, where the tests hold it against long
 // arithmetic at the words' extremes.
 #pragma once

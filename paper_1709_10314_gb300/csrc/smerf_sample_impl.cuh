@@ -1141,7 +1141,7 @@ __device__ __forceinline__ void grp_c2r_rt(C* buf0, C* buf1, int R, int lgNc, co
 // them the field's bits, depend on no thread count).  A field's
 // error against 64-bit references is 3.2e-15 at 64 x 128 (3.3e-15 with the FP64 FFT), 3.5e-15 at 32 x 64 (3.9e-15) and
 // 5.2e-13 at 1024 x 2048, p = 2 (8.6e-13; the tables' own error, set-up included).  That grid, 16 realisations: 2161 ->
-// 1332 us (with box_muller_call); 20001 of 32 x 64: 3057 -> 2029 us (with two realisations per CTA,
+// 1335 us (with box_muller_call); 20001 of 32 x 64: 3057 -> 2029 us (with two realisations per CTA,
 // band_config).  One unit for the whole transform took 1322 and 2014 us, and had fewer bits than FP64 from
 // 512 points on.
 // Factors e^{2 pi i k / n} are exact to 2^-62, stored as two words per component (int4: Re hi, lo, Im
@@ -2055,8 +2055,8 @@ inline long long waves(long long ctas, int per_sm) { return (ctas + 152ll * per_
 // The general rule gives each producer as few units as fit, hence one large CTA per SM; a CTA of
 // fewer, busier producers lets two or three run on an SM and fill each other's barriers.  Timed
 // against every candidate over n_phi 256 to 8192, p = 1 .. 3 and 8 to 512 realisations; e.g. 1024 x
-// 2048, 64 realisations: p = 1 430 -> 387 us, p = 2 756 -> 621 us, p = 3 1714 -> 1401 us; 512 x 1024,
-// 512 realisations, p = 3 4048 -> 2601 us.  n = 0: many realisations (batches).
+// 2048, 64 realisations: p = 2 756 -> 645 us, p = 3 1759 -> 1441 us a call (FP64 tables); p = 1 430 -> 387 us; 512 x
+// 1024, 512 realisations, p = 3 4048 -> 2601 us (FP32 tables).  n = 0: many realisations.
 template <class Real>
 inline bool seg_choice(const smerf_plan* pl, int n, int& upt, int& rmax, int& nf, int& minb)
 {

@@ -25,8 +25,9 @@
 // dz), D_m has leading coefficient (-1)^p (1-z^2)^p, so only the last U-component is
 // driven, with intensity A_amp / (2 pi (1 - s^2)).  It needs only the regular solution,
 // i.e. 2F1 at x <= 1/2, and has no cancellation when z1 and z2 are close.
-// The start covariance J(z0, z0) uses Eq. (Jmatrix_efficient) directly (both solutions
-// at |z0| ~ 0, where both series converge fast).
+// The start covariance J(z0, z0) of a real spectrum comes from ratios of neighbouring orders on both sides of z0
+// (start_kernel); a complex one takes Eq. (Jmatrix_efficient) with its Gamma factors (start_kernel_c).
+// Both solutions are needed at |z0| ~ 0 only, where both series converge fast.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
